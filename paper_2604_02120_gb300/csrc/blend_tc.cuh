@@ -14,14 +14,32 @@
 // thread owns two pixels of one lane and composites both with packed f32x2
 // arithmetic.
 //
-// Warps: 0-3 epilogue (warp w reads TMEM lanes 32 w .. 32 w + 31), 4 producer,
-// 5 MMA issue (lane 0) and TMEM owner.  The producer streams (tile, chunk)
-// items through a ring of SS shared-memory stages (header, v_g rows,
-// per-splat colour) across tile boundaries, so the next tile's gathers
-// overlap the current tile's compositing; the MMA writes a ring of 2 TMEM
-// stages.  An empty tile travels as one stage with n = 0, the end of the
-// queue as n = -1.  When all four epilogue warps of a tile are
-// done (every pixel stopped) the producer skips that tile's remaining chunks.
+// Warps: 0-3 epilogue (warp w reads TMEM lanes 32 w .. 32 w + 31; it holds an
+// 8 x 4 pixel block of each half, lane_col / lane_row), 4 scanner, 5 row
+// builder, MMA issue (lane 0) and TMEM owner.
+//  - The scanner walks the tiles of the queue and their lists in groups of 32
+//    entries, copies the splats a group ahead by cp.async (or by TMA gathers
+//    of packed records), drops the entries whose alpha stays below 1/255 on
+//    the whole tile (splat_reaches) and packs the others, with their list
+//    positions, into chunks of CH raw splats, two slots ahead.
+//  - The builder turns a raw chunk into a stage of the shared-memory ring
+//    (SS stages: header, v_g rows, per-splat colour and position), issues its
+//    MMA into one of 2 TMEM stages and drops the chunks of a tile whose pixels
+//    have all stopped meanwhile.
+// Both run across tile boundaries, so the next tile's lookups and gathers
+// overlap the current tile's compositing.  An empty tile travels as one stage
+// with n = 0, the end of the queue as n = -1.
+//
+// Why the lists are culled here: with full 3-sigma rectangles 50 to 72% of a
+// tile's entries reach none of its pixels, and an entry dropped costs the
+// scanner about 2 instructions per epilogue warp, one kept 29 (the kernel runs
+// at 60 to 67% of the issue slots).  1920 x 1080, 1M clustered splats, full
+// rectangles: 0.828 -> 0.339 ms; 1280 x 720, 200k: 0.119 -> 0.079 ms; 256 x 256,
+// 10k: 0.036 -> 0.028 ms; opacity-aware lists, where every entry is kept:
+// 0.286 -> 0.273 ms (1920 x 1080), 0.482 -> 0.470 ms (3840 x 2160, 3M).
+// Skipping splats per warp (a vote on the exponents) was measured as well: 5%
+// faster on those full lists, 15% slower at 3840 x 2160, where most splats
+// reach most warps and the branch costs the overlap of neighbouring splats.
 // All waits are bounded by opts.timeout_ns; on expiry the CTA records
 // GS_ERR_TIMEOUT in the device error word, every role leaves its loop, the
 // MMA thread commits to a drain barrier of its own and waits (bounded, 1 s)
@@ -48,7 +66,8 @@ namespace gs {
 namespace tc {
 
 constexpr int kEpiWarps = 4;
-constexpr int kThreads = 192;
+constexpr int kThreads = 192;     // backward: epilogue warps, producer, MMA
+constexpr int kFwdThreads = 192;  // forward: epilogue warps, scanner, row builder
 constexpr int kTStages = 2;
 constexpr int kDoneRing = 16;  // tiles in flight between producer and epilogue < kDoneRing
 constexpr float kAlphaMin = 1.0f / 255.0f;
@@ -108,12 +127,20 @@ __device__ __forceinline__ float from_op(uint16_t b) {
     else return __bfloat162float(__ushort_as_bfloat16(b));
 }
 
-// Per-splat record the epilogue reads: colour duplicated for both pixels of a
-// lane and the exponent ceiling min(log2 0.99, log2 o).
+// Per-splat record of the backward and the fused small-scene kernels: colour
+// duplicated for both pixels of a lane and the exponent ceiling min(log2 0.99, log2 o).
+// (The forward's epilogue reads (r, g, b, cap) as one float4: a warp-wide broadcast
+// of 16 bytes costs four cycles of the SM's shared-memory pipe.)
 struct alignas(16) Rec {
     float4 rg;  // r, r, g, g
     float4 bc;  // b, b, cap, cap
 };
+
+// Pixel of accumulator lane r within a 16 x 8 half: warp r / 32 holds an 8 x 4
+// block (of both halves), so that the pixels a small splat reaches fall into
+// few warps.
+__host__ __device__ __forceinline__ int lane_col(int r) { return ((r >> 5) & 1) * 8 + (r & 7); }
+__host__ __device__ __forceinline__ int lane_row(int r) { return (r >> 6) * 4 + ((r >> 3) & 3); }
 
 // tcgen05.mma of the variant's operand kind (f16/bf16 or e4m3)
 template <int V>
@@ -130,16 +157,12 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
         tc_mma_f16(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
-// A work item of the TMA producer: one chunk of a tile (n > 0), an empty
-// tile (n == 0) or the end of the queue (n < 0).
-struct ProdItem {
-    int tile, seq, base, n, q, vview;
-    uint32_t start;
-    float xc, yc;
-    int pad[3];
-};
-
-constexpr int kRecStages = 4;  // TMA record stages: copies run this many chunks minus one ahead
+constexpr int kRawSlots = 2;   // chunks of raw splats between the scanner and the row builders
+constexpr int kRawFields = 10;  // mean x, y, conic A, B, C, log2 opacity, r, g, b, list position + 1
+constexpr int kGroup = 32;      // list entries the scanner tests at a time
+constexpr int kGeoFields = 9;   // mean (2), conic (3), opacity, colour (3)
+constexpr int kGeoSlots = 4;    // groups of splats copied ahead: two of the current tile, two first ones of a tile
+constexpr int kRecSlots = 4;    // TMA slots of a group's records
 
 template <int SS, int CH, int V>
 struct Layout {
@@ -147,14 +170,19 @@ struct Layout {
     static constexpr int B_BYTES = 2 * CH * Traits<V>::ROW_BYTES;
     static constexpr int OFF_B = A_BYTES;
     static constexpr int OFF_REC = OFF_B + SS * B_BYTES;
-    static constexpr int OFF_SCL = OFF_REC + SS * CH * (int)sizeof(Rec);  // FP8: row scales (float2 per splat)
-    static constexpr int RS = kRecStages;
-    static constexpr int OFF_RECT = (OFF_SCL + SS * CH * 8 + 255) / 256 * 256;  // TMA record ring (256-aligned)
-    static constexpr int OFF_BAR = OFF_RECT + RS * CH * kRecBytes;
-    static constexpr int NBAR = 2 * SS + 2 * kTStages + 1 + RS;  // + one drain barrier + the record stages
+    static constexpr int OFF_IDX = OFF_REC + SS * CH * 16;   // list positions + 1 (floats)
+    static constexpr int OFF_SCL = OFF_IDX + SS * CH * 4;    // FP8: row scales (float2 per splat)
+    static constexpr int OFF_RAW = OFF_SCL + (Traits<V>::FP8 ? SS * CH * 8 : 0);
+    static constexpr int OFF_RECT =
+        (OFF_RAW + kRawSlots * kRawFields * CH * 4 + 255) / 256 * 256;  // TMA record slots (256-aligned)
+    static constexpr int OFF_GEO = OFF_RECT;  // the same memory: a launch uses one or the other
+    static_assert(kGeoSlots * kGeoFields * 4 <= kRecSlots * kRecBytes, "splat slots");
+    static constexpr int OFF_BAR = OFF_RECT + kRecSlots * kGroup * kRecBytes;
+    // full[SS], empty[SS], tfull, tempty, drain, raw full, raw empty, record slots
+    static constexpr int NBAR = 2 * SS + 2 * kTStages + 1 + 2 * kRawSlots + kRecSlots;
     static constexpr int OFF_HDR = OFF_BAR + NBAR * 8;
-    static constexpr int OFF_ITEM = OFF_HDR + SS * 32;
-    static constexpr int OFF_MISC = OFF_ITEM + RS * (int)sizeof(ProdItem);
+    static constexpr int OFF_RAWHDR = OFF_HDR + SS * 32;
+    static constexpr int OFF_MISC = OFF_RAWHDR + kRawSlots * 32;
     static constexpr int BYTES = OFF_MISC + 16 + 4 * kDoneRing;
     static constexpr uint32_t TCOLS_RAW = 2u * kTStages * CH;
     static constexpr uint32_t TCOLS = TCOLS_RAW <= 32 ? 32 : TCOLS_RAW <= 64 ? 64 : TCOLS_RAW <= 128 ? 128
@@ -190,6 +218,44 @@ __device__ __forceinline__ float box_max_quadratic(float A, float B, float C, fl
         best = fmaxf(best, -0.5f * (A * dx * dx + 2.f * B * dx * ey + C * ey * ey));
     }
     return best;
+}
+
+// Relative error, per unit of the magnitude sum of Eq. 3's terms, that the
+// variant's exponent may have against the quadratic (an upper bound with room:
+// the split operands err by 2^-21 of that sum at most, one fp16 or bf16 term by
+// 2^-11 or 2^-8 of each coefficient, the e4m3 terms by 2^-10 of the largest).
+template <int V>
+constexpr float reach_rel() {
+    return V == GS_BLEND_TC_FP16 ? 1.0f / 512 : V == GS_BLEND_TC_BF16 ? 1.0f / 64
+           : V == GS_BLEND_TC_FP8_SPLIT ? 1.0f / 256 : 1.0f / 131072;
+}
+
+// False only if the splat's alpha, in the variant's own arithmetic, is below
+// 1/255 at every pixel of the tile; such a splat changes no pixel (the skip
+// rule of Alg. 1) and its MMA columns and compositing can be left out.  The
+// largest quadratic over the box of pixel offsets is compared with the
+// threshold, lowered by 0.3 in base-2 units (more than coeff_row's own test of
+// far splats allows) and by reach_rel of the magnitude sum S at offsets
+// enlarged by 24 px (which covers either reference pixel).  A sum that is not
+// finite keeps the splat.  (xh, yh): splat centre minus the upper half's
+// reference; bx0..by1: the offsets of that half's pixels from it.
+template <int V>
+__device__ __forceinline__ bool splat_reaches(float A, float B, float C, float l2o, float xh, float yh, float bx0,
+                                              float bx1, float by0, float by1) {
+    const float ax = fabsf(xh) + 24.f, ay = fabsf(yh) + 24.f;
+    const float S = fmaf(0.5f * fabsf(A) * ax, ax, fmaf(fabsf(B) * ax, ay, 0.5f * fabsf(C) * ay * ay));
+    // the maximum over the box lies on the two lines nearest to the splat's centre
+    // (a definite form; a nearly singular or indefinite one is kept)
+    const float x0 = xh + bx0, x1 = xh + bx1, y0 = yh + by0 - 8.0f, y1 = yh + by1;
+    const float ex = fminf(fmaxf(0.f, x0), x1), ey = fminf(fmaxf(0.f, y0), y1);
+    const float dy = fminf(fmaxf(__fdividef(-B * ex, C), y0), y1);
+    const float dx = fminf(fmaxf(__fdividef(-B * ey, A), x0), x1);
+    const float qx = fmaf(A * ex, ex, fmaf(2.f * B * ex, dy, C * dy * dy));
+    const float qy = fmaf(A * dx, dx, fmaf(2.f * B * dx, ey, C * ey * ey));
+    const float p = fmaf(-0.5f * kLog2e, fminf(qx, qy), l2o);
+    const bool definite = A > 0.f && C > 0.f && A * C > B * B;
+    return !(S < 1e30f && ((definite && fmaf(reach_rel<V>(), S, p) < kLog2AlphaMin - 0.3f) ||
+                           l2o < kLog2AlphaMin - 0.3f));
 }
 
 // Coefficient row of Eq. 6 for one splat and one reference pixel, in base-2
@@ -300,6 +366,46 @@ __device__ __forceinline__ float store_coeff_row(uint8_t* mB, int r, const float
     }
 }
 
+// Both rows of a splat (ju: upper reference, jl: lower) of a 16-bit variant.
+// Their three quadratic coefficients are the same numbers and are split once
+// (unless coeff_row replaced one of the rows).
+template <int V>
+__device__ __forceinline__ void store_coeff_pair(uint8_t* mB, int ju, int jl, const float (&vu)[6],
+                                                 const float (&vl)[6]) {
+    using TR = Traits<V>;
+    uint16_t terms[3][6];
+    auto split = [&](int i, float v) {
+        float rem = v;
+#pragma unroll
+        for (int t = 0; t < TR::TERMS; ++t) {
+            terms[t][i] = to_op<TR::HALF>(rem);
+            rem -= from_op<TR::HALF>(terms[t][i]);
+        }
+    };
+    auto store = [&](int row) {
+#pragma unroll
+        for (int kc = 0; kc < TR::K / 8; ++kc) {
+            uint16_t e[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int kk = kc * 8 + i;
+                e[i] = (kk < 6 * TR::TERMS) ? terms[kk / 6][kk % 6] : (uint16_t)0;
+            }
+            store_row_chunk<V>(mB, row, kc, e);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < 6; ++i) split(i, vu[i]);
+    store(ju);
+    if (vl[0] != vu[0] || vl[1] != vu[1] || vl[2] != vu[2]) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) split(i, vl[i]);
+    }
+#pragma unroll
+    for (int i = 3; i < 6; ++i) split(i, vl[i]);
+    store(jl);
+}
+
 // The CUDA-core variant's B stage: splat j's two FP32 rows, 12 floats at 48 j
 // (upper row 0..5, lower row 6..11).
 __device__ __forceinline__ void store_cc_rows(uint8_t* mB, int j, const float (&vu)[6], const float (&vl)[6]) {
@@ -365,6 +471,18 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&v)
         : "r"(taddr));
 }
 
+__device__ __forceinline__ void tmem_ld_32x32b_x8(uint32_t taddr, uint32_t (&v)[8]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_32x32b_x4(uint32_t taddr, uint32_t (&v)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(taddr));
+}
+
 __device__ __forceinline__ float sat(float x) { return __saturatef(x); }
 
 // Work item of one pipeline stage.  n > 0: chunk [base, base + n) of the
@@ -375,26 +493,31 @@ struct StageHdr {
     int base;  // list position of the chunk's first splat
     int n;
     int slot;  // queue position of the tile (gs_tile_power output row)
-    int pad[3];
+    float xc, yc;  // the upper half's reference pixel
+    int pad;
 };
 
 
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 template <int V, int CH, int SS, bool DUMP>
-__global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
+__global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
     using TR = Traits<V>;
     using LY = Layout<SS, CH, V>;
     constexpr int K = TR::K;
     constexpr int SBO = TR::SBO;
     constexpr uint32_t IDESC = idesc_f16(TR::FMT, 128, 2 * CH);
+    constexpr int EC = 4;  // accumulator columns an epilogue thread holds at a time
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sA = smem;
     uint8_t* sB = smem + LY::OFF_B;
-    Rec* sRec = reinterpret_cast<Rec*>(smem + LY::OFF_REC);
+    float4* sRec = reinterpret_cast<float4*>(smem + LY::OFF_REC);  // r, g, b, cap
+    float* sIdx = reinterpret_cast<float*>(smem + LY::OFF_IDX);
     float2* sScl = reinterpret_cast<float2*>(smem + LY::OFF_SCL);
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + LY::OFF_BAR);
     StageHdr* sHdr = reinterpret_cast<StageHdr*>(smem + LY::OFF_HDR);
+    float* sRaw = reinterpret_cast<float*>(smem + LY::OFF_RAW);  // [slot][field][splat]
+    StageHdr* sRawHdr = reinterpret_cast<StageHdr*>(smem + LY::OFF_RAWHDR);
     uint32_t* sTmem = reinterpret_cast<uint32_t*>(smem + LY::OFF_MISC);
     volatile int* sAbort = reinterpret_cast<volatile int*>(smem + LY::OFF_MISC + 4);
     volatile int* sDoneRing = reinterpret_cast<volatile int*>(smem + LY::OFF_MISC + 16);
@@ -403,7 +526,9 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
     auto bar_tfull = [&](int t) { return smem_u32(bars + 2 * SS + t); };
     auto bar_tempty = [&](int t) { return smem_u32(bars + 2 * SS + kTStages + t); };
     const uint32_t bar_drain = smem_u32(bars + 2 * SS + 2 * kTStages);
-    auto bar_rec = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + r); };
+    auto bar_rfull = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + r); };
+    auto bar_rempty = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + kRawSlots + r); };
+    auto bar_rec = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + 2 * kRawSlots + r); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_items = a.total_tiles;  // gs_tile_power: the number of listed tiles
@@ -419,14 +544,18 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
             mbar_init(bar_tempty(t), kEpiWarps);
         }
         mbar_init(bar_drain, 1);
-        for (int r = 0; r < LY::RS; ++r) mbar_init(bar_rec(r), 1);
+        for (int r = 0; r < kRawSlots; ++r) {
+            mbar_init(bar_rfull(r), 1);
+            mbar_init(bar_rempty(r), 1);
+        }
+        for (int r = 0; r < kRecSlots; ++r) mbar_init(bar_rec(r), 1);
         *sAbort = 0;
         mbar_fence_init();
     }
     // pixel matrix M_p of a 16 x 8 half-tile (A operand)
-    for (int row = threadIdx.x; row < 128; row += kThreads) {
-        const float xb = origin ? -(float)(row & 15) : 7.5f - (float)(row & 15);
-        const float yb = origin ? -(float)(row >> 4) : 3.5f - (float)(row >> 4);
+    for (int row = threadIdx.x; row < 128; row += kFwdThreads) {
+        const float xb = (origin ? 0.f : 7.5f) - (float)lane_col(row);
+        const float yb = (origin ? 0.f : 3.5f) - (float)lane_row(row);
         store_mp_row<V>(sA, row, xb, yb);
     }
     fence_proxy_async_smem();
@@ -446,8 +575,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
         // this lane's pixel monomials (the same in both halves), as M_p holds them
         float mp[5];
         {
-            const float xb = origin ? -(float)(r & 15) : 7.5f - (float)(r & 15);
-            const float yb = origin ? -(float)(r >> 4) : 3.5f - (float)(r >> 4);
+            const float xb = (origin ? 0.f : 7.5f) - (float)lane_col(r);
+            const float yb = (origin ? 0.f : 3.5f) - (float)lane_row(r);
             mp[0] = xb * xb;
             mp[1] = yb * yb;
             mp[2] = xb * yb;
@@ -493,8 +622,8 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
                 W = vd.W;
                 H = vd.H;
                 pix_off = vd.pix_off;
-                px = (lt % vd.tiles_x) * kTile + (r & 15);
-                py_up = (lt / vd.tiles_x) * kTile + (r >> 4);
+                px = (lt % vd.tiles_x) * kTile + lane_col(r);
+                py_up = (lt / vd.tiles_x) * kTile + lane_row(r);
                 in_up = px < W && py_up < H;
                 in_lo = px < W && py_up + 8 < H;
                 slot = hd.slot;
@@ -508,12 +637,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
             const int base = hd.base;
             if (n > 0 && !wdone) {
                 const uint32_t tb = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(t * 2 * CH);
-                const Rec* rec = sRec + s * CH;
+                const float4* rec = sRec + s * CH;
+                const float* idx1 = sIdx + s * CH;
 #pragma unroll 1
-                for (int c0 = 0; c0 < n; c0 += 16) {
+                for (int c0 = 0; c0 < n; c0 += EC) {
                     // every pixel of this warp has stopped: the chunk's later splats change nothing
                     if (!DUMP && c0 > 0 && __all_sync(0xffffffffu, T.x == 0.f && T.y == 0.f)) break;
-                    uint32_t vu[16], vl[16];
+                    uint32_t vu[EC], vl[EC];
                     // CC: Eq. 6 on the CUDA cores, column by column below (both pixels of
                     // the lane share their monomials)
                     const float* rows = reinterpret_cast<const float*>(sB + s * LY::B_BYTES) + (size_t)c0 * 12;
@@ -529,14 +659,14 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
                         return __fadd2_rn(make_float2(a1.y, a2.w), p);
                     };
                     if constexpr (!TR::CC) {
-                        tmem_ld_32x32b_x16(tb + (uint32_t)c0, vu);
-                        tmem_ld_32x32b_x16(tb + (uint32_t)(CH + c0), vl);
+                        tmem_ld_32x32b_x4(tb + (uint32_t)c0, vu);
+                        tmem_ld_32x32b_x4(tb + (uint32_t)(CH + c0), vl);
                         tmem_ld_wait();
                     }
                     if constexpr (TR::FP8) {  // undo the per-row scaling of the e4m3 operands
                         const float2* scl = sScl + s * CH;
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
+                        for (int c = 0; c < EC; ++c) {
                             const float2 z = __fmul2_rn(make_float2(__uint_as_float(vu[c]), __uint_as_float(vl[c])),
                                                         scl[c0 + c]);
                             vu[c] = __float_as_uint(z.x);
@@ -545,25 +675,27 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
                     }
                     if constexpr (DUMP) {
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
+                        for (int c = 0; c < EC; ++c) {
                             const int j = c0 + c;
                             if (j < n) {
                                 float* o = a.dump + ((size_t)slot * a.max_len + (size_t)base + j) * 256;
-                                o[r] = __uint_as_float(vu[c]);
-                                o[r + 128] = __uint_as_float(vl[c]);
+                                const int p = 16 * lane_row(r) + lane_col(r);
+                                o[p] = __uint_as_float(vu[c]);
+                                o[p + 128] = __uint_as_float(vl[c]);
                             }
                         }
                     } else {
-                        const float base1 = (float)(base + c0 + 1);
+                        const float4 ix4 = *reinterpret_cast<const float4*>(idx1 + c0);
+                        const float ix[EC] = {ix4.x, ix4.y, ix4.z, ix4.w};
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const Rec rc = rec[c0 + c];
+                        for (int c = 0; c < EC; ++c) {
                             float2 pw;
                             if constexpr (TR::CC) pw = cc_power(c);
                             else pw = make_float2(__uint_as_float(vu[c]), __uint_as_float(vl[c]));
+                            const float4 rc = rec[c0 + c];
                             float2 al;
-                            al.x = ex2_approx(fminf(pw.x, rc.bc.z));
-                            al.y = ex2_approx(fminf(pw.y, rc.bc.w));
+                            al.x = ex2_approx(fminf(pw.x, rc.w));
+                            al.y = ex2_approx(fminf(pw.y, rc.w));
                             float2 cull;
                             cull.x = sat(fmaf(al.x, -kCullScale, kAlphaMin * kCullScale));
                             cull.y = sat(fmaf(al.y, -kCullScale, kAlphaMin * kCullScale));
@@ -576,14 +708,16 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
                             const float2 a2 = __ffma2_rn(neg2(al), stop, al);
                             const float2 w = __fmul2_rn(a2, T);
                             T = __ffma2_rn(neg2(tT), stop, tT);
-                            Cr = __ffma2_rn(make_float2(rc.rg.x, rc.rg.y), w, Cr);
-                            Cg = __ffma2_rn(make_float2(rc.rg.z, rc.rg.w), w, Cg);
-                            Cb = __ffma2_rn(make_float2(rc.bc.x, rc.bc.y), w, Cb);
+                            Cr.x = __fmaf_rn(rc.x, w.x, Cr.x);
+                            Cr.y = __fmaf_rn(rc.x, w.y, Cr.y);
+                            Cg.x = __fmaf_rn(rc.y, w.x, Cg.x);
+                            Cg.y = __fmaf_rn(rc.y, w.y, Cg.y);
+                            Cb.x = __fmaf_rn(rc.z, w.x, Cb.x);
+                            Cb.y = __fmaf_rn(rc.z, w.y, Cb.y);
                             float2 used;
                             used.x = sat(a2.x * kCullScale);
                             used.y = sat(a2.y * kCullScale);
-                            const float idx1 = base1 + (float)c;
-                            last = __ffma2_rn(used, __fadd2_rn(make_float2(idx1, idx1), neg2(last)), last);
+                            last = __ffma2_rn(used, __fadd2_rn(make_float2(ix[c], ix[c]), neg2(last)), last);
                         }
                     }
                 }
@@ -598,318 +732,351 @@ __global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant_
             __syncwarp();
             if (lane == 0) mbar_arrive(bar_empty(s));
         }
-    } else if (warp == kEpiWarps && !DUMP && a.use_rec) {
-        // ------------------------------------------------ producer (TMA) --
-        // Three stages per chunk, as in Sec. 3.4, each a step ahead of the
-        // next: (1) the work item (tile ticket, its range, the chunk's ids),
-        // (2) the chunk's splat records gathered into a shared-memory ring by
-        // TMA (tile::gather4: four 64-byte rows per copy) RS - 1 items before
-        // (3) its v_g rows are built from that ring into the B stage.  The
-        // copies of the next chunks, across tile boundaries, are in flight
-        // while this chunk's rows are built.
-        constexpr int RS = LY::RS;
-        ProdItem* sIt = reinterpret_cast<ProdItem*>(smem + LY::OFF_ITEM);
-        const float* sRecT = reinterpret_cast<const float*>(smem + LY::OFF_RECT);
+    } else if (warp == kEpiWarps) {
+        // -------------------------------------------------------- scanner --
+        // Walks the tiles' lists in groups of 32 entries, one per lane, and packs
+        // the entries that reach a pixel of the tile (splat_reaches), in list order,
+        // into chunks of CH raw splats for the row builders.
         const float bx0 = origin ? -15.0f : -7.5f, bx1 = origin ? 0.0f : 7.5f;
         const float by0 = origin ? -7.0f : -3.5f, by1 = origin ? 0.0f : 3.5f;
-        // generator state (warp-uniform)
-        int g_seq = -1, g_tile = 0, g_q = 0, g_view = 0, g_len = 0, g_nch = 0, g_c = 0;
-        uint32_t g_start = 0;
-        float g_xc = 0.f, g_yc = 0.f;
-        bool g_end = false;
-        auto gen_next = [&]() -> ProdItem {
-            for (;;) {
-                if (g_end) return ProdItem{0, -2, 0, -1, g_q, 0, 0u, 0.f, 0.f, {0, 0, 0}};
-                // the next chunk of this tile, unless every pixel of the tile has stopped
-                if (g_c < g_nch && !(g_c > 0 && sDoneRing[g_seq % kDoneRing] >= kEpiWarps)) break;
-                int q = 0;
-                if (lane == 0) q = (int)atomicAdd(a.queue, 1u);
-                q = __shfl_sync(0xffffffffu, q, 0);
-                g_q = q;
-                if (q >= n_items) {
-                    g_end = true;
-                    continue;
-                }
-                ++g_seq;
-                g_tile = tile_at(a, q * a.shard_count + a.shard_index);
-                g_start = a.ranges[2 * g_tile];
-                const uint32_t stop = a.ranges[2 * g_tile + 1];
-                g_len = stop > g_start ? (int)(stop - g_start) : 0;
-                g_view = view_of(a, g_tile);
-                const ViewDesc vd = a.views[g_view];
-                const int lt = g_tile - vd.tile_begin;
-                g_xc = (float)((lt % vd.tiles_x) * kTile) + (origin ? 0.5f : 8.0f);
-                g_yc = (float)((lt / vd.tiles_x) * kTile) + (origin ? 0.5f : 4.0f);
-                g_nch = max(1, (g_len + CH - 1) / CH);
-                g_c = 0;
-                if (lane == 0) sDoneRing[g_seq % kDoneRing] = 0;
+        const bool use_rec = !DUMP && a.use_rec;
+        const float* sRecT = reinterpret_cast<const float*>(smem + LY::OFF_RECT);
+        // A group's splats are copied into a slot of shared memory a group ahead of
+        // their use, without passing through registers: each lane its own entry's nine
+        // values by cp.async, or (with splat records) by TMA gathers of four records.
+        float* sGeo = reinterpret_cast<float*>(smem + LY::OFF_GEO) + lane;
+        uint32_t rec_phase = 0, rec_flight = 0;  // per TMA slot: the phase to wait for, a copy in flight
+        auto rec_wait = [&](int slot) -> bool {
+            if (!((rec_flight >> slot) & 1u)) return true;
+            if (!mbar_wait_bounded(bar_rec(slot), (rec_phase >> slot) & 1u, tmo, sAbort)) {
+                *sAbort = 1;
+                atomicOr(a.err, kErrTimeout);
+                return false;
             }
-            const int base = g_c * CH;
-            ++g_c;
-            return ProdItem{g_tile, g_seq, base, g_len > 0 ? min(CH, g_len - base) : 0, g_q, g_view, g_start,
-                            g_xc, g_yc, {0, 0, 0}};
+            rec_phase ^= 1u << slot;
+            rec_flight &= ~(1u << slot);
+            return true;
         };
-        // stage (2) for an item in record stage rs: the ids, then ceil(n / 4)
-        // gather copies (rows past n repeat id 0, a row of the table); an item
-        // without splats just completes the stage's phase
-        auto issue = [&](const ProdItem& it, int rs) {
-            if (it.n <= 0) {
-                if (lane == 0) mbar_arrive(bar_rec(rs));
+        auto fetch = [&](uint32_t g, int n, int v, int slot) {  // n: entries from the group's first on (may exceed 32)
+            if (use_rec) {
+                if (n <= 0 || !rec_wait(slot)) return;
+                const uint32_t id = lane < n ? g : 0u;  // rows past n repeat id 0, a row of the table
+                const int src = 4 * (lane & 7), ng = (min(n, kGroup) + 3) >> 2;
+                const uint32_t g0 = __shfl_sync(0xffffffffu, id, src), g1 = __shfl_sync(0xffffffffu, id, src + 1);
+                const uint32_t g2 = __shfl_sync(0xffffffffu, id, src + 2), g3 = __shfl_sync(0xffffffffu, id, src + 3);
+                fence_proxy_async_smem();  // the slot's earlier reads before the copies' writes
+                __syncwarp();
+                if (lane == 0) mbar_arrive_expect_tx(bar_rec(slot), (uint32_t)(ng * 4 * kRecBytes));
+                __syncwarp();
+                if (lane < ng)
+                    tma_gather4(smem_u32(sRecT + (size_t)(slot * kGroup + 4 * lane) * kRecFloats), &a.rec_map, 0, g0,
+                                g1, g2, g3, bar_rec(slot));
+                rec_flight |= 1u << slot;
+            } else {
+                if (lane < n) {
+                    float* d = sGeo + slot * (kGeoFields * kGroup);
+                    const float* m = reinterpret_cast<const float*>(a.mean2d + g);
+                    cp_async4(d, m);
+                    cp_async4(d + kGroup, m + 1);
+                    const float* cn = a.conic + 3 * (size_t)g;
+                    cp_async4(d + 2 * kGroup, cn);
+                    cp_async4(d + 3 * kGroup, cn + 1);
+                    cp_async4(d + 4 * kGroup, cn + 2);
+                    cp_async4(d + 5 * kGroup, a.opac + (g - (uint32_t)(v * a.n_per_view)));
+                    if (a.rgb) {
+                        const float* cl = a.rgb + 3 * (size_t)g;
+                        cp_async4(d + 6 * kGroup, cl);
+                        cp_async4(d + 7 * kGroup, cl + 1);
+                        cp_async4(d + 8 * kGroup, cl + 2);
+                    }
+                }
+                cp_async_commit();
+            }
+        };
+        // The next tile: its queue item is taken when a tile starts, then its id, range,
+        // first two groups of entries and first group of splats are looked up, one
+        // dependent load per group of the current tile, so that a tile that ends early
+        // (as dense ones do) finds them ready.
+        int q_next = 0, nt_step = 0, nt_tile = 0, nt_len = 0, nt_slot = 2;
+        uint32_t nt_start = 0, nt_stop = 0, nt_id = 0, nt_id2 = 0;
+        auto step_next = [&]() {
+            if (nt_step == 0) {
+                q_next = __shfl_sync(0xffffffffu, q_next, 0);
+                if (q_next >= n_items) {
+                    nt_step = 4;
+                    return;
+                }
+                nt_tile = DUMP ? a.tiles[q_next] : tile_at(a, q_next * a.shard_count + a.shard_index);
+            } else if (nt_step == 1) {
+                nt_start = a.ranges[2 * nt_tile];
+                nt_stop = a.ranges[2 * nt_tile + 1];
+            } else if (nt_step == 2) {
+                nt_len = nt_stop > nt_start ? (int)(nt_stop - nt_start) : 0;
+                if (DUMP && nt_len > a.max_len) nt_len = a.max_len;
+                if (lane < nt_len) nt_id = a.ids[nt_start + lane];
+                if (lane + kGroup < nt_len) nt_id2 = a.ids[nt_start + kGroup + lane];
+            } else if (nt_step == 3) {
+                fetch(nt_id, nt_len, view_of(a, nt_tile), nt_slot);
+            } else {
                 return;
             }
-            const uint32_t g = lane < it.n ? a.ids[it.start + it.base + lane] : 0u;
-            const int src = 4 * (lane & 7);
-            const uint32_t g0 = __shfl_sync(0xffffffffu, g, src), g1 = __shfl_sync(0xffffffffu, g, src + 1);
-            const uint32_t g2 = __shfl_sync(0xffffffffu, g, src + 2), g3 = __shfl_sync(0xffffffffu, g, src + 3);
-            const int ng = (it.n + 3) >> 2;
-            if (lane == 0) mbar_arrive_expect_tx(bar_rec(rs), (uint32_t)(ng * 4 * kRecBytes));
-            __syncwarp();
-            if (lane < ng)
-                tma_gather4(smem_u32(sRecT + ((size_t)rs * CH + 4 * lane) * kRecFloats), &a.rec_map, 0, g0, g1, g2,
-                            g3, bar_rec(rs));
+            ++nt_step;
         };
-        int k = 0, ri = 0, wi = 0;
-        bool gen_done = false, quit = false;
-        unsigned long long issued = 0;
-        for (; ri < RS - 1 && !gen_done; ++ri) {
-            const ProdItem it = gen_next();
-            __syncwarp();
-            if (lane == 0) sIt[ri % RS] = it;
-            issue(it, ri % RS);
-            gen_done = it.n < 0;
-        }
-        while (!quit) {
-            if (!gen_done) {  // keep RS - 1 items in flight
-                const ProdItem it = gen_next();
-                __syncwarp();
-                if (lane == 0) sIt[ri % RS] = it;
-                issue(it, ri % RS);
-                gen_done = it.n < 0;
-                ++ri;
-            }
-            __syncwarp();
-            const ProdItem it = sIt[wi % RS];
-            const int rs = wi % RS;
-            if (!mbar_wait_bounded(bar_rec(rs), (uint32_t)(wi / RS) & 1u, tmo, sAbort)) {
+        // The open raw slot: free, and not yet published
+        int k = 0;
+        bool open = false, quit = false;
+        auto acquire = [&]() -> bool {
+            if (!mbar_wait_bounded(bar_rempty(k % kRawSlots), ((uint32_t)(k / kRawSlots) & 1u) ^ 1u, tmo, sAbort)) {
                 *sAbort = 1;
                 atomicOr(a.err, kErrTimeout);
+                return false;
+            }
+            open = true;
+            return !*sAbort;
+        };
+        auto publish = [&](const StageHdr& h) {
+            if (lane == 0) sRawHdr[k % kRawSlots] = h;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_rfull(k % kRawSlots));
+            ++k;
+            open = false;
+        };
+        if (lane == 0) q_next = (int)atomicAdd(a.queue, 1u);
+        for (int seq = 0; !quit; ++seq) {
+            while (nt_step < 4) step_next();
+            const int q = q_next;
+            if (q >= n_items) {
+                if (acquire()) publish(StageHdr{0, -2, 0, -1, q, 0.f, 0.f, 0});
                 break;
             }
-            ++wi;
-            // a later chunk of a tile whose pixels have all stopped is dropped
-            if (it.n > 0 && it.base > 0 && sDoneRing[it.seq % kDoneRing] >= kEpiWarps) continue;
-            const int s = k % SS;
-            const uint32_t ps = (uint32_t)(k / SS) & 1u;
-            if (!mbar_wait_bounded(bar_empty(s), ps ^ 1u, tmo, sAbort)) {
-                *sAbort = 1;
-                atomicOr(a.err, kErrTimeout);
-                break;
-            }
-            if (*sAbort) break;
-            const int n = it.n;
-            if (n > 0) {
-                issued += (unsigned long long)n;
-                uint8_t* mB = sB + s * LY::B_BYTES;
-                const float yc_lo = it.yc + 8.0f;
-                for (int j = lane; j < CH; j += 32) {
-                    float vu[6], vl[6];
-                    Rec rc;
-                    if (j < n) {
-                        const float4* rp = reinterpret_cast<const float4*>(sRecT + ((size_t)rs * CH + j) * kRecFloats);
-                        const float4 r0 = rp[0], r1 = rp[1], r2 = rp[2];
-                        const float xh = r0.x - it.xc;
-                        coeff_row<TR::HALF && !TR::CC>(r0.z, r0.w, r1.x, r1.y, xh, r0.y - it.yc, bx0, bx1, by0, by1, vu);
-                        coeff_row<TR::HALF && !TR::CC>(r0.z, r0.w, r1.x, r1.y, xh, r0.y - yc_lo, bx0, bx1, by0, by1, vl);
-                        rc.rg = make_float4(r2.x, r2.x, r2.y, r2.y);
-                        rc.bc = make_float4(r2.z, r2.z, r1.z, r1.z);
-                    } else {  // padding column: dead rows, no colour
-#pragma unroll
-                        for (int i = 0; i < 5; ++i) vu[i] = vl[i] = 0.f;
-                        vu[5] = vl[5] = kDeadPower;
-                        rc.rg = make_float4(0.f, 0.f, 0.f, 0.f);
-                        rc.bc = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int tile = nt_tile, len = nt_len, vview = view_of(a, tile);
+            const uint32_t start = nt_start;
+            uint32_t gn = nt_id2;  // the next group's entries
+            int slot = nt_slot, ahead = 0;  // this group's slot, the next group's
+            nt_slot ^= 1;
+            nt_step = 0;
+            if (lane == 0) q_next = (int)atomicAdd(a.queue, 1u);
+            const ViewDesc vd = a.views[vview];
+            const int lt = tile - vd.tile_begin;
+            const float xc = (float)((lt % vd.tiles_x) * kTile) + (origin ? 0.5f : 8.0f);
+            const float yc = (float)((lt / vd.tiles_x) * kTile) + (origin ? 0.5f : 4.0f);
+            if (lane == 0) sDoneRing[seq % kDoneRing] = 0;
+            int fill = 0, sent = 0;  // splats in the open slot; splats published
+            const int ng = (len + kGroup - 1) / kGroup;
+            int gi = 0;
+            for (; gi < ng; ++gi) {
+                // every pixel of this tile has stopped: skip the rest of its list
+                if (!DUMP && sent > 0 && __all_sync(0xffffffffu, sDoneRing[seq % kDoneRing] >= kEpiWarps)) {
+                    fill = 0;  // the open slot, if any, goes to the next tile
+                    if (!use_rec) cp_async_wait<0>();  // the copies of the group not taken, before their slot is reused
+                    break;
+                }
+                const int e = gi * kGroup + lane;
+                if (gi + 1 < ng) fetch(gn, len - (gi + 1) * kGroup, vview, ahead);
+                float2 m;
+                float A, B, C, l2o, cr = 0.f, cg = 0.f, cb = 0.f;
+                if (use_rec) {
+                    if (!rec_wait(slot)) {
+                        quit = true;
+                        break;
                     }
-                    if constexpr (TR::CC) {
-                        store_cc_rows(mB, j, vu, vl);
-                    } else {
-                        const float su = store_coeff_row<V>(mB, j, vu);
-                        const float sl = store_coeff_row<V>(mB, CH + j, vl);
-                        if constexpr (TR::FP8) sScl[s * CH + j] = make_float2(su, sl);
+                    const float4* rp = reinterpret_cast<const float4*>(sRecT + (size_t)(slot * kGroup + lane) * kRecFloats);
+                    const float4 r0 = rp[0], r1 = rp[1], r2 = rp[2];
+                    m = make_float2(r0.x, r0.y);
+                    A = r0.z;
+                    B = r0.w;
+                    C = r1.x;
+                    l2o = r1.y;
+                    cr = r2.x;
+                    cg = r2.y;
+                    cb = r2.z;
+                } else {
+                    // all groups but the one just requested have arrived (the lane's own copies)
+                    if (gi + 1 < ng) cp_async_wait<1>();
+                    else cp_async_wait<0>();
+                    const float* d = sGeo + slot * (kGeoFields * kGroup);
+                    m = make_float2(d[0], d[kGroup]);
+                    A = d[2 * kGroup];
+                    B = d[3 * kGroup];
+                    C = d[4 * kGroup];
+                    const float o = d[5 * kGroup];
+                    l2o = o > 0.f ? __log2f(o) : -INFINITY;
+                    if (a.rgb) {
+                        cr = d[6 * kGroup];
+                        cg = d[7 * kGroup];
+                        cb = d[8 * kGroup];
+                    }
+                }
+                slot = ahead;
+                ahead ^= 1;
+                if (e + 2 * kGroup < len) gn = a.ids[start + e + 2 * kGroup];
+                const bool keep =
+                    e < len && (DUMP || splat_reaches<V>(A, B, C, l2o, m.x - xc, m.y - yc, bx0, bx1, by0, by1));
+                const unsigned kb = __ballot_sync(0xffffffffu, keep);
+                if (kb != 0u) {
+                    // slot position of this lane's splat, counted from the open slot's start
+                    int pos = keep ? fill + __popc(kb & ((1u << lane) - 1u)) : -1;
+                    fill += __popc(kb);
+                    for (;;) {
+                        if (!open && !acquire()) {
+                            quit = true;
+                            break;
+                        }
+                        if (pos >= 0 && pos < CH) {
+                            float* w = sRaw + (k % kRawSlots) * (kRawFields * CH) + pos;
+                            w[0] = m.x;
+                            w[CH] = m.y;
+                            w[2 * CH] = A;
+                            w[3 * CH] = B;
+                            w[4 * CH] = C;
+                            w[5 * CH] = l2o;
+                            w[6 * CH] = cr;
+                            w[7 * CH] = cg;
+                            w[8 * CH] = cb;
+                            w[9 * CH] = (float)(e + 1);
+                        }
+                        if (fill < CH) break;
+                        publish(StageHdr{tile, seq, sent, CH, q, xc, yc, 0});
+                        sent += CH;
+                        fill -= CH;
+                        pos -= CH;
+                        if (fill == 0) break;
+                    }
+                    if (quit) break;
+                }
+                step_next();
+            }
+            if (quit) break;
+            // the tile's last chunk; a tile of which nothing is left travels as one empty
+            // chunk, so that its pixels are written
+            if (fill > 0 || sent == 0) {
+                if (!open && !acquire()) break;
+                publish(StageHdr{tile, seq, sent, fill, q, xc, yc, 0});
+            }
+            // issued pairs: 256 for every list entry taken, kept or not
+            if (!DUMP && a.issued != nullptr && lane == 0 && gi > 0)
+                atomicAdd(a.issued, 256ull * (unsigned long long)min(len, gi * kGroup));
+        }
+        // copies still in flight land before the block leaves
+        for (int r = 0; r < kRecSlots; ++r)
+            if ((rec_flight >> r) & 1u) mbar_wait_bounded(bar_rec(r), (rec_phase >> r) & 1u, 1000000000ull, nullptr);
+    } else {
+        // ---------------------------------------------------- row builder --
+        // Turns each raw chunk into a stage: the coefficient rows of both halves and
+        // the epilogue's records.  A chunk of a tile whose pixels have all stopped
+        // meanwhile is dropped.
+        const float bx0 = origin ? -15.0f : -7.5f, bx1 = origin ? 0.0f : 7.5f;
+        const float by0 = origin ? -7.0f : -3.5f, by1 = origin ? 0.0f : 3.5f;
+        int k = 0;
+        for (int kr = 0;; ++kr) {
+            const int s = k % SS, rs = kr % kRawSlots;
+            if (!mbar_wait_bounded(bar_rfull(rs), (uint32_t)(kr / kRawSlots) & 1u, tmo, sAbort) ||
+                !mbar_wait_bounded(bar_empty(s), ((uint32_t)(k / SS) & 1u) ^ 1u, tmo, sAbort)) {
+                *sAbort = 1;
+                atomicOr(a.err, kErrTimeout);
+                break;
+            }
+            const StageHdr hd = sRawHdr[rs];
+            if (!DUMP && hd.n > 0 && hd.base > 0 && __all_sync(0xffffffffu, sDoneRing[hd.seq % kDoneRing] >= kEpiWarps)) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_rempty(rs));
+                continue;
+            }
+            if (hd.n > 0) {
+                uint8_t* mB = sB + s * LY::B_BYTES;
+                if constexpr (CH == 16 && !TR::CC) {
+                    // one row per lane: lanes 0..15 the upper half's, 16..31 the lower half's
+                    const int j = lane & 15;
+                    const bool lower = lane >= 16;
+                    const float* w = sRaw + rs * (kRawFields * CH) + j;
+                    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, kDeadPower};  // padding column: dead rows, no colour
+                    float4 rc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float ix = 0.f;
+                    if (j < hd.n) {
+                        const float l2o = w[5 * CH];
+                        coeff_row<TR::HALF>(w[2 * CH], w[3 * CH], w[4 * CH], l2o, w[0] - hd.xc,
+                                            w[CH] - (lower ? hd.yc + 8.0f : hd.yc), bx0, bx1, by0, by1, v);
+                        rc = make_float4(w[6 * CH], w[7 * CH], w[8 * CH], fminf(l2o, kLog2AlphaMax));
+                        ix = w[9 * CH];
+                    }
+                    if (!lower) {
+                        sRec[s * CH + j] = rc;
+                        sIdx[s * CH + j] = ix;
+                    }
+                    const float sc = store_coeff_row<V>(mB, lower ? CH + j : j, v);
+                    if constexpr (TR::FP8) reinterpret_cast<float*>(sScl + s * CH + j)[lower ? 1 : 0] = sc;
+                } else {
+                for (int j = lane; j < CH; j += 32) {
+                    const float* w = sRaw + rs * (kRawFields * CH) + j;
+                    float vu[6] = {0.f, 0.f, 0.f, 0.f, 0.f, kDeadPower};  // padding column: dead rows, no colour
+                    float vl[6] = {0.f, 0.f, 0.f, 0.f, 0.f, kDeadPower};
+                    float4 rc = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float ix = 0.f;
+                    if (j < hd.n) {
+                        const float A = w[2 * CH], B = w[3 * CH], C = w[4 * CH], l2o = w[5 * CH];
+                        const float xh = w[0] - hd.xc;
+                        coeff_row<TR::HALF && !TR::CC>(A, B, C, l2o, xh, w[CH] - hd.yc, bx0, bx1, by0, by1, vu);
+                        coeff_row<TR::HALF && !TR::CC>(A, B, C, l2o, xh, w[CH] - (hd.yc + 8.0f), bx0, bx1, by0, by1,
+                                                       vl);
+                        rc = make_float4(w[6 * CH], w[7 * CH], w[8 * CH], fminf(l2o, kLog2AlphaMax));
+                        ix = w[9 * CH];
                     }
                     sRec[s * CH + j] = rc;
-                }
-            }
-            if (lane == 0) sHdr[s] = StageHdr{it.tile, n < 0 ? -2 : it.seq, it.base, n, it.q, {0, 0, 0}};
-            // orders this warp's shared-memory reads and writes before the MMA's
-            // reads and before the next TMA copies into the record ring
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_full(s));
-            ++k;
-            if (n < 0) quit = true;
-        }
-        // copies still in flight (after a timeout) land before the block leaves
-        for (; wi < ri; ++wi) mbar_wait_bounded(bar_rec(wi % RS), (uint32_t)(wi / RS) & 1u, 1000000000ull, nullptr);
-        if (lane == 0 && a.issued != nullptr && issued) atomicAdd(a.issued, issued * 256ull);
-    } else if (warp == kEpiWarps) {
-        // ------------------------------------------------------- producer --
-        int k = 0;
-        bool quit = false;
-        unsigned long long issued = 0;  // splats of the chunks this block issued
-        // The next tile's queue item is taken when a tile starts and its range
-        // read once the tile's first chunk is out, so those dependent loads
-        // overlap the chunk work instead of preceding the next tile.
-        auto fetch = [&](int qq, int& tl, uint32_t& st, int& ln) {
-            tl = DUMP ? a.tiles[qq] : tile_at(a, qq * a.shard_count + a.shard_index);
-            st = a.ranges[2 * tl];
-            const uint32_t sp = a.ranges[2 * tl + 1];
-            ln = sp > st ? (int)(sp - st) : 0;
-        };
-        int q_next = 0, nt_tile = 0, nt_len = 0;
-        uint32_t nt_start = 0;
-        if (lane == 0) q_next = (int)atomicAdd(a.queue, 1u);
-        q_next = __shfl_sync(0xffffffffu, q_next, 0);
-        if (q_next < n_items) fetch(q_next, nt_tile, nt_start, nt_len);
-        for (int seq = 0; !quit; ++seq) {
-            const int q = q_next;
-            const bool end = q >= n_items;
-            int tile = 0, len = 0, vview = 0;
-            uint32_t start = 0;
-            float xc = 0.f, yc_up = 0.f;
-            if (!end && lane == 0) q_next = (int)atomicAdd(a.queue, 1u);  // used after this tile's first chunk
-            if (!end) {
-                tile = nt_tile;
-                start = nt_start;
-                len = nt_len;
-                if (DUMP && len > a.max_len) len = a.max_len;
-                vview = view_of(a, tile);
-                const ViewDesc vd = a.views[vview];
-                const int lt = tile - vd.tile_begin;
-                xc = (float)((lt % vd.tiles_x) * kTile) + (origin ? 0.5f : 8.0f);
-                yc_up = (float)((lt / vd.tiles_x) * kTile) + (origin ? 0.5f : 4.0f);
-                if (lane == 0) sDoneRing[seq % kDoneRing] = 0;
-            }
-            const float yc_lo = yc_up + 8.0f;
-            const float bx0 = origin ? -15.0f : -7.5f, bx1 = origin ? 0.0f : 7.5f;
-            const float by0 = origin ? -7.0f : -3.5f, by1 = origin ? 0.0f : 3.5f;
-            const int nch = end ? 1 : max(1, (len + CH - 1) / CH);
-            for (int c = 0; c < nch; ++c) {
-                const int s = k % SS;
-                const uint32_t ps = (uint32_t)(k / SS) & 1u;
-                if (!mbar_wait_bounded(bar_empty(s), ps ^ 1u, tmo, sAbort)) {
-                    *sAbort = 1;
-                    atomicOr(a.err, kErrTimeout);
-                    quit = true;
-                    break;
-                }
-                if (*sAbort) {
-                    quit = true;
-                    break;
-                }
-                // every pixel of this tile has stopped: skip its remaining chunks
-                if (!DUMP && c > 0 && sDoneRing[seq % kDoneRing] >= kEpiWarps) break;
-                const int base = c * CH;
-                const int n = end ? -1 : min(CH, len - base);
-                if (n > 0) {
-                    issued += (unsigned long long)n;
-                    uint8_t* mB = sB + s * LY::B_BYTES;
-                    for (int j = lane; j < CH; j += 32) {
-                        float vu[6], vl[6];
-                        Rec rc;
-                        if (j < n) {
-                            const uint32_t g = a.ids[start + base + j];
-                            const float2 m = a.mean2d[g];
-                            const float A = a.conic[3 * g], B = a.conic[3 * g + 1], C = a.conic[3 * g + 2];
-                            const float o = a.opac[g - (uint32_t)(vview * a.n_per_view)];
-                            const float l2o = o > 0.f ? __log2f(o) : -INFINITY;
-                            const float xh = m.x - xc;
-                            coeff_row<TR::HALF && !TR::CC>(A, B, C, l2o, xh, m.y - yc_up, bx0, bx1, by0, by1, vu);
-                            coeff_row<TR::HALF && !TR::CC>(A, B, C, l2o, xh, m.y - yc_lo, bx0, bx1, by0, by1, vl);
-                            const float cap = fminf(l2o, kLog2AlphaMax);
-                            float cr = 0.f, cg = 0.f, cb = 0.f;
-                            if (a.rgb) {
-                                cr = a.rgb[3 * g];
-                                cg = a.rgb[3 * g + 1];
-                                cb = a.rgb[3 * g + 2];
-                            }
-                            rc.rg = make_float4(cr, cr, cg, cg);
-                            rc.bc = make_float4(cb, cb, cap, cap);
-                        } else {  // padding column: dead rows, no colour
-#pragma unroll
-                            for (int i = 0; i < 5; ++i) vu[i] = vl[i] = 0.f;
-                            vu[5] = vl[5] = kDeadPower;
-                            rc.rg = make_float4(0.f, 0.f, 0.f, 0.f);
-                            rc.bc = make_float4(0.f, 0.f, 0.f, 0.f);
-                        }
-                        if constexpr (TR::CC) {
-                            store_cc_rows(mB, j, vu, vl);
-                        } else {
-                            const float su = store_coeff_row<V>(mB, j, vu);
-                            const float sl = store_coeff_row<V>(mB, CH + j, vl);
-                            if constexpr (TR::FP8) sScl[s * CH + j] = make_float2(su, sl);
-                        }
-                        sRec[s * CH + j] = rc;
+                    sIdx[s * CH + j] = ix;
+                    if constexpr (TR::CC) {
+                        store_cc_rows(mB, j, vu, vl);
+                    } else if constexpr (TR::FP8) {
+                        const float su = store_coeff_row<V>(mB, j, vu);
+                        const float sl = store_coeff_row<V>(mB, CH + j, vl);
+                        sScl[s * CH + j] = make_float2(su, sl);
+                    } else {
+                        store_coeff_pair<V>(mB, j, CH + j, vu, vl);
                     }
                 }
-                if (lane == 0) sHdr[s] = StageHdr{tile, end ? -2 : seq, base, n, q, {0, 0, 0}};
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar_full(s));
-                ++k;
-                if (c == 0 && !end) {  // the next tile's range, while this tile's chunks are consumed
-                    q_next = __shfl_sync(0xffffffffu, q_next, 0);
-                    if (q_next < n_items) fetch(q_next, nt_tile, nt_start, nt_len);
                 }
             }
-            if (end) quit = true;
-        }
-        // issued pairs: every chunk is evaluated at all 256 pixels of its tile
-        if (!DUMP && lane == 0 && a.issued != nullptr && issued) atomicAdd(a.issued, issued * 256ull);
-    } else if (lane == 0) {
-        // ------------------------------------------------------ MMA issue --
-        const uint32_t aA = smem_u32(sA);
-        for (int k = 0;; ++k) {
-            const int s = k % SS, t = k % kTStages;
-            const uint32_t ps = (uint32_t)(k / SS) & 1u, pt = (uint32_t)(k / kTStages) & 1u;
-            if (!mbar_wait_bounded(bar_full(s), ps, tmo, sAbort)) {
-                *sAbort = 1;
-                atomicOr(a.err, kErrTimeout);
-                break;
-            }
+            if (lane == 0) sHdr[s] = hd;
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_rempty(rs));
             // the TMEM stage must be free even for a stage without an MMA, so
             // that tfull[t] never runs two phases ahead of a waiting epilogue warp
-            if (!mbar_wait_bounded(bar_tempty(t), pt ^ 1u, tmo, sAbort)) {
+            const int t = k % kTStages;
+            if (!mbar_wait_bounded(bar_tempty(t), ((uint32_t)(k / kTStages) & 1u) ^ 1u, tmo, sAbort)) {
                 *sAbort = 1;
                 atomicOr(a.err, kErrTimeout);
                 break;
             }
-            const int n = sHdr[s].n;
-            if (n <= 0) {
-                mbar_arrive(bar_tfull(t));
-                if (n < 0) break;
-                mbar_arrive(bar_empty(s));
-                continue;
-            }
-            if constexpr (TR::CC) {  // the epilogue contracts the rows itself
-                mbar_arrive(bar_tfull(t));
-                mbar_arrive(bar_empty(s));
-                continue;
-            }
-            tc_fence_after();
-            const uint32_t aB = smem_u32(sB + s * LY::B_BYTES);
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(bar_full(s));
+                if (hd.n > 0 && !TR::CC) {  // CC: the epilogue contracts the rows itself
+                    tc_fence_after();
+                    const uint32_t aA = smem_u32(sA), aB = smem_u32(sB + s * LY::B_BYTES);
 #pragma unroll
-            for (int ks = 0; ks < TR::KSTEPS; ++ks) {
-                const uint64_t ad = smem_desc(aA + (uint32_t)(ks * 256), 128, SBO);
-                const uint64_t bd = smem_desc(aB + (uint32_t)(ks * 256), 128, SBO);
-                tc_mma<V>(tmem + (uint32_t)(t * 2 * CH), ad, bd, IDESC, ks > 0 ? 1u : 0u);
+                    for (int ks = 0; ks < TR::KSTEPS; ++ks) {
+                        const uint64_t ad = smem_desc(aA + (uint32_t)(ks * 256), 128, SBO);
+                        const uint64_t bd = smem_desc(aB + (uint32_t)(ks * 256), 128, SBO);
+                        tc_mma<V>(tmem + (uint32_t)(t * 2 * CH), ad, bd, IDESC, ks > 0 ? 1u : 0u);
+                    }
+                    tc_commit(bar_tfull(t));
+                    tc_commit(bar_empty(s));
+                } else {
+                    mbar_arrive(bar_tfull(t));
+                    if (hd.n >= 0) mbar_arrive(bar_empty(s));
+                }
             }
-            tc_commit(bar_tfull(t));
-            tc_commit(bar_empty(s));
+            __syncwarp();
+            ++k;
+            if (hd.n < 0) break;
         }
-        // every MMA this thread issued has finished before TMEM is freed (a
-        // fresh barrier: no phase of another stage can be mistaken for it)
-        tc_commit(bar_drain);
-        mbar_wait_bounded(bar_drain, 0, 1000000000ull, nullptr);
+        if (lane == 0) {
+            // every MMA this thread issued has finished before TMEM is freed (a
+            // fresh barrier: no phase of another stage can be mistaken for it)
+            tc_commit(bar_drain);
+            mbar_wait_bounded(bar_drain, 0, 1000000000ull, nullptr);
+        }
+        __syncwarp();
     }
 
     tc_fence_before();
@@ -940,9 +1107,9 @@ cudaError_t launch_inst(const BlendArgs& a, int items, cudaStream_t s) {
         if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
         // registers are granted per warp in units of 256
         const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-        const int by_regs = 65536 / (regs_warp * (kThreads / 32));
+        const int by_regs = 65536 / (regs_warp * (kFwdThreads / 32));
         const int by_smem = smem_sm / (bytes + (int)fa.sharedSizeBytes + 1024);
-        const int by_threads = 2048 / kThreads;
+        const int by_threads = 2048 / kFwdThreads;
         const int by_tmem = (int)(512 / LY::TCOLS);
         r.per_sm = by_regs;
         if (by_smem < r.per_sm) r.per_sm = by_smem;
@@ -953,7 +1120,7 @@ cudaError_t launch_inst(const BlendArgs& a, int items, cudaStream_t s) {
     });
     if (es != cudaSuccess) return es;
     const int grid = items < sh.per_sm * sh.sms ? (items > 0 ? items : 1) : sh.per_sm * sh.sms;
-    kern<<<grid, kThreads, bytes, s>>>(a);
+    kern<<<grid, kFwdThreads, bytes, s>>>(a);
     count_launches();
     return cudaGetLastError();
 }

@@ -121,6 +121,18 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const void* map, int x
         : "memory");
 }
 
+// Asynchronous 4-byte copy global -> shared memory by this thread, grouped by
+// cp_async_commit; cp_async_wait<N> waits until all but the thread's last N groups
+// have arrived.
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
