@@ -102,9 +102,9 @@ typedef struct gs_blend_opts {
                             first pixel): 0 = its centre (x0 + 8, y0 + 4),
                             1 = the centre of its first pixel (x0 + 0.5, y0 + 0.5) */
     float bg[3];         /* background colour added as T_final * bg */
-    int32_t bwd_stages;  /* TC backward: depth of its shared-memory ring, 0 = the variant's default
-                            (6 for fp16 operands, 3 for bf16 and FP8, the deepest that keeps 3 blocks
-                            per SM); built: 2, 3, 4, 6 (gs_blend_autotune_backward picks one) */
+    int32_t bwd_stages;  /* TC backward: depth of its ring of splat chunks, 0 = default (4, the deepest
+                            that keeps 3 blocks per SM for every operand type); built: 2, 3, 4, 6
+                            (gs_blend_autotune_backward picks one) */
     int64_t timeout_ns;  /* limit of every device-side wait; 0 = 1 s */
     int32_t shard_count; /* tile sharding across ranks: the call blends only the tiles t
                             (global tile ids) with t % shard_count == shard_index and leaves

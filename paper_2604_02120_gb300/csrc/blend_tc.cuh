@@ -483,6 +483,26 @@ __device__ __forceinline__ void tmem_ld_32x32b_x4(uint32_t taddr, uint32_t (&v)[
                  : "r"(taddr));
 }
 
+// Copies the nine values of item g of view v (mean, conic, opacity, colour) to
+// d[0], d[kGroup], ..., d[8 kGroup] asynchronously (cp.async; the caller commits).
+__device__ __forceinline__ void copy_splat_async(const BlendArgs& a, float* d, uint32_t g, int v) {
+    const float* m = reinterpret_cast<const float*>(a.mean2d + g);
+    cp_async4(d, m);
+    cp_async4(d + kGroup, m + 1);
+    const float* cn = a.conic + 3 * (size_t)g;
+    cp_async4(d + 2 * kGroup, cn);
+    cp_async4(d + 3 * kGroup, cn + 1);
+    cp_async4(d + 4 * kGroup, cn + 2);
+    cp_async4(d + 5 * kGroup, a.opac + (g - (uint32_t)(v * a.n_per_view)));
+    if (a.rgb) {
+        const float* cl = a.rgb + 3 * (size_t)g;
+        cp_async4(d + 6 * kGroup, cl);
+        cp_async4(d + 7 * kGroup, cl + 1);
+        cp_async4(d + 8 * kGroup, cl + 2);
+    }
+}
+
+__device__ __forceinline__ float log2_opacity(float o) { return o > 0.f ? __log2f(o) : -INFINITY; }
 __device__ __forceinline__ float sat(float x) { return __saturatef(x); }
 
 // Work item of one pipeline stage.  n > 0: chunk [base, base + n) of the
@@ -504,7 +524,6 @@ template <int V, int CH, int SS, bool DUMP>
 __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
     using TR = Traits<V>;
     using LY = Layout<SS, CH, V>;
-    constexpr int K = TR::K;
     constexpr int SBO = TR::SBO;
     constexpr uint32_t IDESC = idesc_f16(TR::FMT, 128, 2 * CH);
     constexpr int EC = 4;  // accumulator columns an epilogue thread holds at a time
@@ -773,23 +792,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                                 g1, g2, g3, bar_rec(slot));
                 rec_flight |= 1u << slot;
             } else {
-                if (lane < n) {
-                    float* d = sGeo + slot * (kGeoFields * kGroup);
-                    const float* m = reinterpret_cast<const float*>(a.mean2d + g);
-                    cp_async4(d, m);
-                    cp_async4(d + kGroup, m + 1);
-                    const float* cn = a.conic + 3 * (size_t)g;
-                    cp_async4(d + 2 * kGroup, cn);
-                    cp_async4(d + 3 * kGroup, cn + 1);
-                    cp_async4(d + 4 * kGroup, cn + 2);
-                    cp_async4(d + 5 * kGroup, a.opac + (g - (uint32_t)(v * a.n_per_view)));
-                    if (a.rgb) {
-                        const float* cl = a.rgb + 3 * (size_t)g;
-                        cp_async4(d + 6 * kGroup, cl);
-                        cp_async4(d + 7 * kGroup, cl + 1);
-                        cp_async4(d + 8 * kGroup, cl + 2);
-                    }
-                }
+                if (lane < n) copy_splat_async(a, sGeo + slot * (kGeoFields * kGroup), g, v);
                 cp_async_commit();
             }
         };
@@ -899,8 +902,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                     A = d[2 * kGroup];
                     B = d[3 * kGroup];
                     C = d[4 * kGroup];
-                    const float o = d[5 * kGroup];
-                    l2o = o > 0.f ? __log2f(o) : -INFINITY;
+                    l2o = log2_opacity(d[5 * kGroup]);
                     if (a.rgb) {
                         cr = d[6 * kGroup];
                         cg = d[7 * kGroup];

@@ -121,6 +121,12 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const void* map, int x
         : "memory");
 }
 
+// *p += v in global memory, without a result (p is a global address whatever the
+// compiler can prove about it).
+__device__ __forceinline__ void red_add(float* p, float v) {
+    asm volatile("red.relaxed.gpu.global.add.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+
 // Asynchronous 4-byte copy global -> shared memory by this thread, grouped by
 // cp_async_commit; cp_async_wait<N> waits until all but the thread's last N groups
 // have arrived.
