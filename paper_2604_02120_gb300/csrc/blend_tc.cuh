@@ -502,6 +502,17 @@ __device__ __forceinline__ void copy_splat_async(const BlendArgs& a, float* d, u
     }
 }
 
+// Queue items a block claims at once after a short tile, `left` being unclaimed: up
+// to 4 where the tiles come longest first (the next ones are no longer), else up
+// to 2 (more would deal neighbouring dense tiles of an unsorted queue to one
+// block), and no more than half a block's share of what is left, so that the last
+// claims are single.  17190 tiles of 7 splats each, 3053 x 1439: 88 -> 78 us.  (In
+// the backward the same gained 6% there and cost 3% at 3840 x 2160, where the tile
+// headers are hidden anyway: not used.)
+__device__ __forceinline__ int short_claim(int left, bool ordered) {
+    return max(1, min(ordered ? 4 : 2, left / (2 * (int)gridDim.x)));
+}
+
 __device__ __forceinline__ float log2_opacity(float o) { return o > 0.f ? __log2f(o) : -INFINITY; }
 __device__ __forceinline__ float sat(float x) { return __saturatef(x); }
 
@@ -796,28 +807,43 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                 cp_async_commit();
             }
         };
-        // The next tile: its queue item is taken when a tile starts, then its id, range,
+        // The next tile: its queue item is claimed when a tile starts, then its id, range,
         // first two groups of entries and first group of splats are looked up, one
         // dependent load per group of the current tile, so that a tile that ends early
-        // (as dense ones do) finds them ready.
+        // (as dense ones do) finds them ready.  After a short tile, whose next one is not
+        // ready, several items are claimed and looked up together, one per lane (short_claim).
+        int claim = 0, n_claim = 1, b_q = 0, b_n = 0, b_i = 0;  // items b_q + [b_i, b_n) are claimed
+        uint32_t b_tile = 0, b_start = 0, b_stop = 0;           // lane i: item b_q + i
         int q_next = 0, nt_step = 0, nt_tile = 0, nt_len = 0, nt_slot = 2;
-        uint32_t nt_start = 0, nt_stop = 0, nt_id = 0, nt_id2 = 0;
+        uint32_t nt_start = 0, nt_id = 0, nt_id2 = 0;
         auto step_next = [&]() {
-            if (nt_step == 0) {
-                q_next = __shfl_sync(0xffffffffu, q_next, 0);
+            if (nt_step == 0 && b_i == b_n) {
+                b_q = __shfl_sync(0xffffffffu, claim, 0);
+                b_n = n_claim;
+                b_i = 0;
+                const int qi = b_q + lane;
+                if (lane < b_n && qi < n_items)
+                    b_tile = DUMP ? a.tiles[qi] : tile_at(a, qi * a.shard_count + a.shard_index);
+            } else if (nt_step == 1 && b_i == 0) {
+                if (lane < b_n && b_q + lane < n_items) {
+                    b_start = a.ranges[2 * b_tile];
+                    b_stop = a.ranges[2 * b_tile + 1];
+                }
+            } else if (nt_step <= 2) {
+                q_next = b_q + b_i;
                 if (q_next >= n_items) {
                     nt_step = 4;
                     return;
                 }
-                nt_tile = DUMP ? a.tiles[q_next] : tile_at(a, q_next * a.shard_count + a.shard_index);
-            } else if (nt_step == 1) {
-                nt_start = a.ranges[2 * nt_tile];
-                nt_stop = a.ranges[2 * nt_tile + 1];
-            } else if (nt_step == 2) {
-                nt_len = nt_stop > nt_start ? (int)(nt_stop - nt_start) : 0;
+                nt_tile = (int)__shfl_sync(0xffffffffu, b_tile, b_i);
+                nt_start = __shfl_sync(0xffffffffu, b_start, b_i);
+                const uint32_t stop = __shfl_sync(0xffffffffu, b_stop, b_i);
+                ++b_i;
+                nt_len = stop > nt_start ? (int)(stop - nt_start) : 0;
                 if (DUMP && nt_len > a.max_len) nt_len = a.max_len;
                 if (lane < nt_len) nt_id = a.ids[nt_start + lane];
                 if (lane + kGroup < nt_len) nt_id2 = a.ids[nt_start + kGroup + lane];
+                nt_step = 2;
             } else if (nt_step == 3) {
                 fetch(nt_id, nt_len, view_of(a, nt_tile), nt_slot);
             } else {
@@ -844,7 +870,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             ++k;
             open = false;
         };
-        if (lane == 0) q_next = (int)atomicAdd(a.queue, 1u);
+        if (lane == 0) claim = (int)atomicAdd(a.queue, 1u);
         for (int seq = 0; !quit; ++seq) {
             while (nt_step < 4) step_next();
             const int q = q_next;
@@ -858,7 +884,10 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             int slot = nt_slot, ahead = 0;  // this group's slot, the next group's
             nt_slot ^= 1;
             nt_step = 0;
-            if (lane == 0) q_next = (int)atomicAdd(a.queue, 1u);
+            if (b_i == b_n) {
+                n_claim = len > 2 * kGroup ? 1 : short_claim(n_items - b_q, a.order != nullptr);
+                if (lane == 0) claim = (int)atomicAdd(a.queue, (unsigned)n_claim);
+            }
             const ViewDesc vd = a.views[vview];
             const int lt = tile - vd.tile_begin;
             const float xc = (float)((lt % vd.tiles_x) * kTile) + (origin ? 0.5f : 8.0f);
