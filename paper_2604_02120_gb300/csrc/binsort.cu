@@ -925,8 +925,12 @@ __device__ __forceinline__ uint32_t supertile_mask(const SortViews& sv, const fl
 // into lane j's count, adding it to ranges with one atomic per tile when the
 // supertile changes.  32 pairs of several supertiles: one atomic per group
 // of equal supertiles and tile.  With st_count (zeroed by k_dup_coarse), each
-// supertile's total is added there as well.
-constexpr uint32_t kPairSeg = 512;
+// supertile's total is added there as well, and the ends of its pairs go to
+// st_beg / st_end (supertiles without pairs are left alone).  Segments are 128 to 512 pairs
+// (the least that gives every warp at most one), loaded 128 pairs at a time
+// with the next 128 in flight: the kernel waits for memory, not for its
+// arithmetic.
+constexpr uint32_t kPairBatch = 128, kPairSegMax = 512;
 template <bool TIGHT>
 __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__ SortViews sv,
                                                          const float2* __restrict__ mean2d,
@@ -935,7 +939,8 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
                                                          const uint32_t* __restrict__ cval, uint32_t n_host,
                                                          const uint64_t* __restrict__ n_dev, uint32_t n_items,
                                                          bool pack, uint16_t* __restrict__ masks,
-                                                         uint32_t* __restrict__ ranges, uint32_t* st_count) {
+                                                         uint32_t* __restrict__ ranges, uint32_t* st_count,
+                                                         uint32_t* __restrict__ st_beg, uint32_t* __restrict__ st_end) {
     const uint32_t Ic = pass_count(n_host, n_dev);
     const int lane = threadIdx.x & 31;
     // tile j of supertile key (global id) as a global tile index
@@ -949,8 +954,11 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
     };
     const uint64_t warp_id = ((uint64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
     const uint64_t warps = ((uint64_t)gridDim.x * kThreads) >> 5;
-    for (uint64_t s0 = warp_id * kPairSeg; s0 < Ic; s0 += warps * kPairSeg) {
-        const uint64_t s1 = min(s0 + (uint64_t)kPairSeg, (uint64_t)Ic);
+    const uint64_t want = (Ic + warps - 1) / warps;
+    const uint64_t seg = min((uint64_t)kPairSegMax, max((want + kPairBatch - 1) / kPairBatch, (uint64_t)1) * kPairBatch);
+    constexpr int U = kPairBatch / 32;
+    for (uint64_t s0 = warp_id * seg; s0 < Ic; s0 += warps * seg) {
+        const uint64_t s1 = min(s0 + seg, (uint64_t)Ic);
         uint32_t cur = 0xffffffffu;  // the supertile being counted (warp-uniform)
         uint32_t acc = 0;            // lane j < 16: its count of tile j
         auto flush = [&]() {
@@ -961,52 +969,86 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
             }
             acc = 0;
         };
-        for (uint64_t b = s0; b < s1; b += 32) {
-            const uint64_t e = b + (uint64_t)lane;
-            uint32_t key = 0xffffffffu, m = 0;
-            if (e < s1) {
-                key = ckey[e];
-                if (pack) {
-                    m = key >> 16;
-                    key &= 0xFFFFu;
-                } else {
-                    int v = 0;
-                    while (v + 1 < sv.num_views && sv.st_begin[v + 1] <= (int)key) ++v;
-                    const int ls = (int)key - sv.st_begin[v];
-                    const uint32_t it = cval[e];
-                    m = it < n_items ? supertile_mask<TIGHT>(sv, mean2d, radius, it, sv.views[v],
-                                                             (ls % sv.st_x[v]) * kSuper, (ls / sv.st_x[v]) * kSuper)
-                                     : 0u;
-                    masks[e] = (uint16_t)m;
-                }
-            }
-            const uint32_t k0 = __shfl_sync(0xffffffffu, key, 0);  // lane 0 always holds a pair
-            if (!__all_sync(0xffffffffu, key == k0 || e >= s1)) {
-                // pairs of several supertiles: one atomic per group and tile
-                flush();
-                cur = 0xffffffffu;
-                const unsigned peers = __match_any_sync(0xffffffffu, key);
-                const bool leader = lane == __ffs(peers) - 1 && key != 0xffffffffu;
-                uint32_t all = 0;
+        const uint32_t kmask = pack ? 0xFFFFu : 0xFFFFFFFFu;
+        uint32_t last = st_beg != nullptr && s0 > 0 ? ckey[s0 - 1] & kmask : 0xffffffffu;  // the pair before the group's
+        uint32_t kn[U];
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const unsigned bj = __ballot_sync(0xffffffffu, (m >> j) & 1u) & peers;
-                    if (leader && bj) atomicAdd(&ranges[2 * tile_of(key, j) + 1], (uint32_t)__popc(bj));
-                    all += (uint32_t)__popc(bj);
-                }
-                if (st_count != nullptr && leader && all) atomicAdd(&st_count[key], all);
-                continue;
-            }
-            if (k0 != cur) {
-                flush();
-                cur = k0;
-            }
+        for (int u = 0; u < U; ++u) {
+            const uint64_t e = s0 + (uint64_t)(32 * u + lane);
+            kn[u] = e < s1 ? ckey[e] : 0xffffffffu;
+        }
+        for (uint64_t b0 = s0; b0 < s1; b0 += kPairBatch) {
+            uint32_t kb[U];
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                // bits 4w .. 4w + 3 of the mask to bytes 0..3, summed over the warp (<= 32 each)
-                const uint32_t spread = (((m >> (4 * w)) & 0xFu) * 0x00204081u) & 0x01010101u;
-                const uint32_t sum = __reduce_add_sync(0xffffffffu, spread);
-                if ((lane >> 2) == w) acc += (sum >> (8 * (lane & 3))) & 0xFFu;
+            for (int u = 0; u < U; ++u) {
+                kb[u] = kn[u];
+                const uint64_t e = b0 + kPairBatch + (uint64_t)(32 * u + lane);
+                kn[u] = e < s1 ? ckey[e] : 0xffffffffu;
+            }
+#pragma unroll 1
+            for (int u = 0; u < U; ++u) {
+                const uint64_t b = b0 + (uint64_t)(32 * u);
+                if (b >= s1) break;
+                const uint64_t e = b + (uint64_t)lane;
+                uint32_t key = 0xffffffffu, m = 0;
+                if (e < s1) {
+                    key = u == 0 ? kb[0] : u == 1 ? kb[1] : u == 2 ? kb[2] : kb[3];
+                    if (pack) {
+                        m = key >> 16;
+                        key &= 0xFFFFu;
+                    } else {
+                        int v = 0;
+                        while (v + 1 < sv.num_views && sv.st_begin[v + 1] <= (int)key) ++v;
+                        const int ls = (int)key - sv.st_begin[v];
+                        const uint32_t it = cval[e];
+                        m = it < n_items ? supertile_mask<TIGHT>(sv, mean2d, radius, it, sv.views[v],
+                                                                 (ls % sv.st_x[v]) * kSuper, (ls / sv.st_x[v]) * kSuper)
+                                         : 0u;
+                        masks[e] = (uint16_t)m;
+                    }
+                }
+                const uint32_t k0 = __shfl_sync(0xffffffffu, key, 0);  // lane 0 always holds a pair
+                const bool same = __all_sync(0xffffffffu, key == k0 || e >= s1);
+                if (st_beg != nullptr && (!same || k0 != last || b + 32 >= Ic)) {
+                    uint32_t prev = __shfl_up_sync(0xffffffffu, key, 1);
+                    if (lane == 0) prev = last;
+                    if (e < s1) {
+                        if (key != prev) {
+                            st_beg[key] = (uint32_t)e;
+                            if (prev != 0xffffffffu) st_end[prev] = (uint32_t)e;
+                        }
+                        if (e + 1 == Ic) st_end[key] = Ic;
+                    }
+                }
+                last = k0;  // (used only if the segment goes on: the group is full then)
+                if (!same) {
+                    last = __shfl_sync(0xffffffffu, key, 31);
+                    // pairs of several supertiles: one atomic per group and tile
+                    flush();
+                    cur = 0xffffffffu;
+                    const unsigned peers = __match_any_sync(0xffffffffu, key);
+                    const bool leader = lane == __ffs(peers) - 1 && key != 0xffffffffu;
+                    uint32_t all = 0;
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        const unsigned bj = __ballot_sync(0xffffffffu, (m >> j) & 1u) & peers;
+                        if (leader && bj) atomicAdd(&ranges[2 * tile_of(key, j) + 1], (uint32_t)__popc(bj));
+                        all += (uint32_t)__popc(bj);
+                    }
+                    if (st_count != nullptr && leader && all) atomicAdd(&st_count[key], all);
+                    continue;
+                }
+                if (k0 != cur) {
+                    flush();
+                    cur = k0;
+                }
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                    // bits 4w .. 4w + 3 of the mask to bytes 0..3, summed over the warp (<= 32 each)
+                    const uint32_t spread = (((m >> (4 * w)) & 0xFu) * 0x00204081u) & 0x01010101u;
+                    const uint32_t sum = __reduce_add_sync(0xffffffffu, spread);
+                    if ((lane >> 2) == w) acc += (sum >> (8 * (lane & 3))) & 0xFFu;
+                }
             }
         }
         flush();
@@ -1017,13 +1059,21 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
 // given), after k_tile_scan: its items are the sorted pairs [cs, ce) with
 // key s; every instance's id (and key) goes to its tile's next position, in
 // item order, from the pairs' tile masks (in the key's high half when kmask
-// is 0xFFFF, else in masks[]).  Rounds of kFineRound pairs, the next round's
-// loads in flight during the current one: warp w owns tiles w and w + 8 and
-// walks the round's pairs 32 at a time, one ballot per group giving each
-// pair's place in the tile's run and the run's length, into a shared-memory
-// stage of the tile's ids; it then writes the run with consecutive lanes on
-// consecutive ids.
-constexpr int kFineThreads = 256, kFineRound = 512;
+// is 0xFFFF, else in masks[]).  Rounds of one pair per thread, the next
+// round's loads in flight during the current one.  A warp's 32 pairs give one
+// ballot per tile; the ballots' counts of all warps (a small table) place the
+// warp in each tile's list, and a lane with the tile's bit writes its id at
+// the place its lower lanes leave, so that the ids of a warp go to consecutive
+// addresses.  Splitting a round by pairs rather than by tiles keeps the chain
+// per round short, which is what the kernel waits for: its time is that of the
+// longest supertiles, whose rounds follow one another.  The depth a key needs
+// is read once per pair, a round ahead.  Against warps that own tiles and walk
+// all pairs of a round: 1280 x 720, 200k, full rectangles with keys 114 -> 44
+// us; 1920 x 1080, 1M 252 -> 93; opacity-aware lists at 3840 x 2160, 139M
+// instances, no keys 225 -> 206 (2.7 TB/s of ids); 16 views 563 -> 524 us.
+constexpr int kFineThreads = 512;
+constexpr int kFineWarps = kFineThreads / 32;
+template <bool KEYS>
 __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ SortViews sv,
                                                        const float* __restrict__ depth,
                                                        const uint32_t* __restrict__ ckey,
@@ -1032,14 +1082,15 @@ __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ S
                                                        const uint16_t* __restrict__ masks,
                                                        const uint32_t* __restrict__ ranges,
                                                        const uint32_t* __restrict__ st_order,
+                                                       const uint32_t* __restrict__ st_count,
+                                                       const uint32_t* __restrict__ st_beg,
+                                                       const uint32_t* __restrict__ st_end, uint32_t n_items,
                                                        uint32_t* __restrict__ ids_out, uint64_t* __restrict__ keys_out) {
-    constexpr int PT = kFineRound / kFineThreads;  // pairs each thread loads
-    constexpr int TW = 16 / (kFineThreads / 32);  // tiles per warp
     __shared__ uint32_t s_rng[2];
-    __shared__ uint32_t s_beg[16], s_end[16], s_run[16];
-    __shared__ uint16_t s_mask[kFineRound];
-    __shared__ uint32_t s_item[kFineRound];
-    __shared__ uint32_t s_out[16][kFineRound];
+    __shared__ uint32_t s_beg[16], s_len[16];
+    // instances per round (double-buffered), tile and warp, one byte each (<= 32)
+    __shared__ uint4 s_cnt[2][16];
+    static_assert(kFineWarps == 16, "16 warps' bytes make the 16 bytes of a tile");
     const int s = st_order != nullptr ? (int)st_order[blockIdx.x] : (int)blockIdx.x;  // largest first
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -1050,68 +1101,88 @@ __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ S
     const int cx0 = (ls % sv.st_x[v]) * kSuper, cy0 = (ls / sv.st_x[v]) * kSuper;
     const int tx = vd.tiles_x, ty = tiles_y(vd.H);
     const uint32_t Ic = pass_count(n_host, n_dev);
-    if (threadIdx.x < 2) s_rng[threadIdx.x] = lower_bound_u32(ckey, Ic, (uint32_t)s + threadIdx.x, kmask);
+    if (st_count != nullptr) {  // k_pair_masks left the ends of the supertile's pairs
+        if (st_count[s] == 0) return;
+        if (threadIdx.x < 2) s_rng[threadIdx.x] = min(threadIdx.x ? st_end[s] : st_beg[s], Ic);
+    } else if (threadIdx.x < 2) {
+        s_rng[threadIdx.x] = lower_bound_u32(ckey, Ic, (uint32_t)s + threadIdx.x, kmask);
+    }
     if (threadIdx.x < 16) {
         const int c = cx0 + (threadIdx.x & 3), r = cy0 + (threadIdx.x >> 2);
         const bool ok = c < tx && r < ty;
         const uint32_t gt = (uint32_t)vd.tile_begin + (uint32_t)r * (uint32_t)tx + (uint32_t)c;
-        s_run[threadIdx.x] = 0;
-        s_beg[threadIdx.x] = ok ? ranges[2 * gt] : 0u;
-        s_end[threadIdx.x] = ok ? ranges[2 * gt + 1] : 0u;
+        const uint32_t b = ok ? ranges[2 * gt] : 0u, e = ok ? ranges[2 * gt + 1] : 0u;
+        s_beg[threadIdx.x] = b;
+        s_len[threadIdx.x] = e - b;
     }
     __syncthreads();
     const uint32_t cs = s_rng[0], ce = s_rng[1];
     if (cs >= ce) return;
     const bool packed = kmask == 0xFFFFu;
-    uint32_t mk[PT], it[PT];
-    auto fetch = [&](uint32_t r0) {
-#pragma unroll
-        for (int i = 0; i < PT; ++i) {
-            const uint32_t e = r0 + (uint32_t)(i * kFineThreads + threadIdx.x);
-            mk[i] = e < ce ? (packed ? ckey[e] >> 16 : (uint32_t)masks[e]) : 0u;
-            it[i] = e < ce ? cval[e] : 0u;
-        }
+    const int tl = lane & 15;
+    const uint32_t beg = s_beg[tl], len = s_len[tl];  // lane t (and t + 16): tile t's list
+    const uint32_t tile_key = (uint32_t)vd.tile_begin + (uint32_t)(cy0 + (tl >> 2)) * (uint32_t)tx + (uint32_t)(cx0 + (tl & 3));
+    uint32_t run = 0;  // lane t: tile t's instances of the rounds before
+    // pairs of the next round, and of the one after it: a key's depth is a load that
+    // depends on the pair's item
+    uint32_t mk = 0, it = 0, dp = 0, mk2 = 0, it2 = 0;
+    auto fetch = [&](uint32_t e) {
+        mk2 = e < ce ? (packed ? ckey[e] >> 16 : (uint32_t)masks[e]) : 0u;
+        it2 = e < ce ? cval[e] : 0u;
     };
-    fetch(cs);
-    for (uint32_t r0 = cs; r0 < ce; r0 += kFineRound) {
+    auto advance = [&](uint32_t e) {
+        mk = mk2;
+        it = it2;
+        if constexpr (KEYS) dp = mk != 0 && it < n_items ? __float_as_uint(depth[it]) : 0u;
+        fetch(e);
+    };
+    fetch(cs + threadIdx.x);
+    advance(cs + kFineThreads + threadIdx.x);
+    for (uint32_t r0 = cs, round = 0; r0 < ce; r0 += kFineThreads, round ^= 1u) {
+        const uint32_t m = mk, id = it, dep = dp;
+        advance(r0 + 2 * kFineThreads + threadIdx.x);
+        // lane t: the warp's instances of tile t in this round, from four lane reductions of
+        // the masks' bits spread to bytes
+        uint32_t cnt = 0;
 #pragma unroll
-        for (int i = 0; i < PT; ++i) {
-            s_mask[i * kFineThreads + threadIdx.x] = (uint16_t)mk[i];
-            s_item[i * kFineThreads + threadIdx.x] = it[i];
+        for (int w = 0; w < 4; ++w) {
+            const uint32_t spread = (((m >> (4 * w)) & 0xFu) * 0x00204081u) & 0x01010101u;
+            const uint32_t sum = __reduce_add_sync(0xffffffffu, spread);
+            if ((tl >> 2) == w) cnt = (sum >> (8 * (tl & 3))) & 0xFFu;
         }
-        if (r0 + kFineRound < ce) fetch(r0 + kFineRound);
-        __syncthreads();
-        const int ng = (int)((min(ce - r0, (uint32_t)kFineRound) + 31) / 32);  // groups of 32 pairs in the round
+        if (lane < 16) reinterpret_cast<uint8_t*>(&s_cnt[round][lane])[warp] = (uint8_t)cnt;
+        __syncthreads();  // (a warp two rounds ahead has passed the next barrier: two tables suffice)
+        const uint4 c4 = s_cnt[round][tl];
+        // where the warp's instances of tile t start: after those of the lower warps
+        const uint32_t lo = 0xFFFFFFFFu >> (31 - 8 * (warp & 3)) >> 1;  // the bytes of the lower warps in this warp's word
+        const int wq = warp >> 2;
+        uint32_t off = run;
+        off = __dp4a(wq > 0 ? c4.x : c4.x & lo, 0x01010101u, off);
+        off = __dp4a(wq > 1 ? c4.y : wq == 1 ? c4.y & lo : 0u, 0x01010101u, off);
+        off = __dp4a(wq > 2 ? c4.z : wq == 2 ? c4.z & lo : 0u, 0x01010101u, off);
+        off = __dp4a(wq == 3 ? c4.w & lo : 0u, 0x01010101u, off);
+        run = __dp4a(c4.x, 0x01010101u, __dp4a(c4.y, 0x01010101u, __dp4a(c4.z, 0x01010101u, __dp4a(c4.w, 0x01010101u, run))));
+        // whole unless the lists are cut off at the capacity
+        const bool whole = __all_sync(0xffffffffu, off + cnt <= len);
+        const uint32_t place = beg + off;
+        const unsigned any = __reduce_or_sync(0xffffffffu, m);
 #pragma unroll
-        for (int h = 0; h < TW; ++h) {
-            const int t = warp + h * (kFineThreads / 32);
-            uint32_t n_t = 0;
-            for (int g = 0; g < ng; ++g) {
-                const int i = 32 * g + lane;
-                const bool in = (s_mask[i] >> t) & 1u;
-                const unsigned b = __ballot_sync(0xffffffffu, in);
-                if (in) s_out[t][n_t + (uint32_t)__popc(b & lt)] = s_item[i];
-                n_t += (uint32_t)__popc(b);
+        for (int t = 0; t < 16; ++t) {
+            if (!((any >> t) & 1u)) continue;
+            bool in = (m >> t) & 1u;
+            const uint32_t o = (uint32_t)__popc(__ballot_sync(0xffffffffu, in) & lt);
+            const uint32_t p = __shfl_sync(0xffffffffu, place, t) + o;
+            if (!whole) {  // (uniform; every lane takes part in the shuffles)
+                const uint32_t ot = __shfl_sync(0xffffffffu, off, t) + o, lt_n = __shfl_sync(0xffffffffu, len, t);
+                in = in && ot < lt_n;
             }
-            __syncwarp();
-            const uint64_t p0 = (uint64_t)s_beg[t] + s_run[t];
-            const uint64_t end = s_end[t];
-            const uint64_t dkey = keys_out != nullptr
-                                      ? (uint64_t)((uint32_t)vd.tile_begin + (uint32_t)(cy0 + (t >> 2)) * (uint32_t)tx +
-                                                   (uint32_t)(cx0 + (t & 3))) << 32
-                                      : 0ull;
-            for (uint32_t k = lane; k < n_t; k += 32) {
-                const uint64_t p = p0 + k;
-                if (p < end) {
-                    const uint32_t g = s_out[t][k];
-                    ids_out[p] = g;
-                    if (keys_out != nullptr) keys_out[p] = dkey | __float_as_uint(depth[g]);
-                }
+            uint32_t hi = 0;
+            if constexpr (KEYS) hi = __shfl_sync(0xffffffffu, tile_key, t);
+            if (in) {
+                ids_out[p] = id;
+                if constexpr (KEYS) keys_out[p] = ((uint64_t)hi << 32) | dep;
             }
-            __syncwarp();
-            if (lane == 0) s_run[t] += n_t;  // this warp's tile alone
         }
-        __syncthreads();  // the round's masks and items are replaced next
     }
 }
 
@@ -1341,6 +1412,9 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     const int nst = sv2.total_st;
     uint32_t* st_count = nst <= n ? dk[0] : nullptr;
     uint32_t* st_order = nst <= n ? dk[1] : nullptr;
+    // the ends of each supertile's pairs, in the sorted items' buffers (free after the duplication)
+    uint32_t* st_beg = nst <= n ? dv[0] : nullptr;
+    uint32_t* st_end = nst <= n ? dv[1] : nullptr;
     if ((e = record_kernel_event(GS_KERNEL_DUPLICATE, false, s)) != cudaSuccess)
         return cuda_status(e, "gs_bin_sort: kernel event");
     dup<<<(int)cdiv(n, kDupTile), kThreads, 0, s>>>(n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes,
@@ -1386,7 +1460,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     // the pairs' tile masks go to the free half of the pair buffers (2 bytes per pair)
     uint16_t* masks = reinterpret_cast<uint16_t*>(ck[which ^ 1]);
     auto pair_masks = tight ? k_pair_masks<true> : k_pair_masks<false>;
-    int pair_grid = 0;  // at most 8 blocks per SM, each warp taking segments of kPairSeg pairs
+    int pair_grid = 0;  // at most 8 blocks per SM, each warp taking segments of pairs
     {
         int dev = 0, sms = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
@@ -1394,18 +1468,20 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
             return cuda_status(e, "gs_bin_sort: device");
         pair_grid = 8 * sms;
     }
-    pair_masks<<<(int)std::min<int64_t>(pair_grid, cdiv(I_grid, (int64_t)kPairSeg * (kThreads / 32))), kThreads, 0,
+    pair_masks<<<(int)std::min<int64_t>(pair_grid, cdiv(I_grid, (int64_t)kPairBatch * (kThreads / 32))), kThreads, 0,
                  s>>>(
-        sv2, mean2d, radius, ck[which], cv[which], I_grid, ctotal, (uint32_t)n, pack, masks, tile_ranges, st_count);
+        sv2, mean2d, radius, ck[which], cv[which], I_grid, ctotal, (uint32_t)n, pack, masks, tile_ranges, st_count,
+        st_beg, st_end);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: tile counts");
     k_tile_scan<<<1, kScanThreads, 0, s>>>(sv2, ntiles, tile_ranges, (uint64_t)capacity, fine_total,
                                            graph ? n_instances_dev : nullptr, st_count, st_order, err);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: tile ranges");
-    k_fine<<<nst, kFineThreads, 0, s>>>(sv2, depth, ck[which], cv[which], I_grid, ctotal,
-                                        pack ? 0xFFFFu : 0xFFFFFFFFu, masks, tile_ranges, st_order, ids_sorted,
-                                        keys_sorted);
+    auto fine = keys_sorted != nullptr ? k_fine<true> : k_fine<false>;
+    fine<<<nst, kFineThreads, 0, s>>>(sv2, depth, ck[which], cv[which], I_grid, ctotal, pack ? 0xFFFFu : 0xFFFFFFFFu,
+                                      masks, tile_ranges, st_order, st_count, st_beg, st_end, (uint32_t)n, ids_sorted,
+                                      keys_sorted);
     count_launches();
     return cuda_status(cudaGetLastError(), "gs_bin_sort: write lists");
 }
