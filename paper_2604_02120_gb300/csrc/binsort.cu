@@ -468,7 +468,6 @@ __device__ __forceinline__ uint32_t runs_mask(const Runs4& rr, int sx) {
 
 // The four tile-row runs of supertile row sy within the rectangle [x0, x1] x
 // [y0, y1], and in *fine their instance count.
-template <bool TIGHT>
 __device__ __forceinline__ Runs4 row_runs(const TightRows& t, int sy, int x0, int x1, int y0, int y1,
                                           uint32_t* fine) {
     Runs4 rr;
@@ -477,12 +476,7 @@ __device__ __forceinline__ Runs4 row_runs(const TightRows& t, int sy, int x0, in
         const int y = sy * kSuper + k;
         int f = 1, l = 0;
         if (y >= y0 && y <= y1) {
-            if constexpr (TIGHT) {
-                tight_row(t, y, x0, x1, f, l);
-            } else {
-                f = x0;
-                l = x1;
-            }
+            tight_row(t, y, x0, x1, f, l);
         }
         rr.f[k] = f;
         rr.l[k] = l;
@@ -631,8 +625,8 @@ __device__ __forceinline__ Runs4 unpack_runs(uint4 v) {
     return rr;
 }
 
-// Coarse duplication in depth order, with the supertile counts and their scan
-// folded in.  Tile t (from the ticket) holds the depth-ordered items
+// Coarse duplication in depth order of opacity-aware lists, with the supertile
+// counts and their scan folded in.  Tile t (from the ticket) holds the depth-ordered items
 // [t * kDupTile, (t + 1) * kDupTile).  Each warp deals its items' supertile
 // rows out to its lanes (warp_units) and evaluates every row's tile runs once,
 // keeping them in shared memory (the first kStashUnits of each warp; later
@@ -656,7 +650,6 @@ __device__ __forceinline__ Runs4 unpack_runs(uint4 v) {
 constexpr uint32_t kWideRow = 8;
 constexpr uint32_t kStashUnits = 128;  // per warp
 constexpr uint32_t kStagePairs = 2048;
-template <bool TIGHT>
 __global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint32_t* __restrict__ perm,
                                                          const __grid_constant__ SortViews sv,
                                                          const float2* __restrict__ mean2d,
@@ -705,8 +698,7 @@ __global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint
         vis = tile_rect(m.x, m.y, radius[item], vd.W, vd.H, x0, x1, y0, y1);
         stx = sv.st_x[v];
         stb = sv.st_begin[v];
-        if constexpr (TIGHT)
-            if (vis) t = item_tight_rows(sv, mean2d, item);
+        if (vis) t = item_tight_rows(sv, mean2d, item);
     }
     const uint32_t units = vis ? (uint32_t)(y1 / kSuper - y0 / kSuper + 1) : 0u;
     uint4* stash = s_runs + warp * kStashUnits;
@@ -720,10 +712,9 @@ __global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint
     warp_units(units, [&](bool act, int src, uint32_t u, uint32_t f) {
         const int bx0 = __shfl_sync(0xffffffffu, x0, src), bx1 = __shfl_sync(0xffffffffu, x1, src);
         const int by0 = __shfl_sync(0xffffffffu, y0, src), by1 = __shfl_sync(0xffffffffu, y1, src);
-        TightRows bt{};
-        if constexpr (TIGHT) bt = shfl_rows(t, src);
+        const TightRows bt = shfl_rows(t, src);
         if (act) {
-            const Runs4 rr = row_runs<TIGHT>(bt, by0 / kSuper + (int)u, bx0, bx1, by0, by1, &fine);
+            const Runs4 rr = row_runs(bt, by0 / kSuper + (int)u, bx0, bx1, by0, by1, &fine);
             const int n = runs_union(rr, [](int, int) {});
             atomicAdd(&s_c[wlane0 + src], (uint32_t)n);
             if (f < kStashUnits) {
@@ -786,14 +777,13 @@ __global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint
         const int sy = by0 / kSuper + (int)u;
         const bool again = act && f >= kStashUnits;  // beyond the stash: evaluated again
         TightRows bt{};
-        if constexpr (TIGHT)
-            if (__any_sync(0xffffffffu, again)) bt = shfl_rows(t, src);
+        if (__any_sync(0xffffffffu, again)) bt = shfl_rows(t, src);
         Runs4 rr{};
         uint32_t n = 0;
         if (act) {
             if (again) {
                 uint32_t fine2 = 0;
-                rr = row_runs<TIGHT>(bt, sy, bx0, bx1, by0, by1, &fine2);
+                rr = row_runs(bt, sy, bx0, bx1, by0, by1, &fine2);
                 n = (uint32_t)runs_union(rr, [](int, int) {});
             } else {
                 rr = unpack_runs(stash[f]);
@@ -873,6 +863,159 @@ __global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint
     }
     for (int i = threadIdx.x; i < (passes - 1) * 256; i += kThreads)
         if (s_h[i]) atomicAdd(&hist[256 + i], s_h[i]);
+}
+
+// The same for full rectangles.  An item's supertiles are then a rectangle too,
+// so nothing is evaluated per row: persistent blocks take tiles of kRectTile
+// depth-ordered items from the ticket (four consecutive items per thread),
+// scan their supertile counts, publish the sum, look back, and write the
+// tile's pairs with consecutive threads on consecutive pairs; a thread finds
+// its pair's item by a search over the items' first pairs and the supertile,
+// key and 16-bit tile mask from the rectangle.  The digit histograms stay in
+// shared memory over all tiles of a block.  It waits for its barriers and the
+// chain ticket, items, gather, look-back per tile (51% of the issue slots at 6
+// blocks per SM; 4 and 8 blocks, a look-back window of 128 tiles and fetching
+// the next tile's items ahead were all slower).  Against the per-row kernel
+// above, which full rectangles used to go through: 16 views of 1.5M splats 2.85
+// -> 0.87 ms; 1920 x 1080, 1M 128 -> 34 us; 1280 x 720, 200k 43 -> 18 us.
+// Counts beyond 32 bits: the starts saturate (no pair past the
+// capacity, below 2^32, is written).
+constexpr int kRectItems = 4;
+constexpr int kRectTile = kThreads * kRectItems;
+__global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uint32_t* __restrict__ perm,
+                                                          const __grid_constant__ SortViews sv,
+                                                          const float2* __restrict__ mean2d,
+                                                          const int* __restrict__ radius, uint64_t limit, int passes,
+                                                          bool pack, uint32_t* tickets, unsigned long long* status,
+                                                          uint32_t* __restrict__ ckey, uint32_t* __restrict__ cval,
+                                                          uint32_t* __restrict__ hist, uint64_t* __restrict__ total,
+                                                          unsigned long long* __restrict__ fine_total,
+                                                          unsigned long long* __restrict__ radix_status,
+                                                          uint32_t coarse_tile, uint32_t* __restrict__ st_zero, int st_n,
+                                                          unsigned* err) {
+    __shared__ uint64_t s_warp[kThreads / 32 + 1];
+    __shared__ uint64_t s_prefix;
+    __shared__ unsigned long long s_fine;
+    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_h[4 * 256];
+    __shared__ uint32_t s_start[kRectTile];  // each item's first pair within the tile
+    __shared__ uint2 s_rect[kRectTile];      // x0 | x1 << 16, y0 | y1 << 16 in tiles
+    __shared__ uint32_t s_item[kRectTile];
+    __shared__ uint8_t s_view[kRectTile];
+    if (st_zero != nullptr)  // the supertile counters of k_pair_masks
+        for (int i = blockIdx.x * kThreads + threadIdx.x; i < st_n; i += gridDim.x * kThreads) st_zero[i] = 0;
+    for (int i = threadIdx.x; i < passes * 256; i += kThreads) s_h[i] = 0;
+    if (threadIdx.x == 0) s_fine = 0;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = atomicAdd(&tickets[kMaxPasses], 1u);
+        __syncthreads();  // (also: the last tile's pairs have left shared memory)
+        const uint32_t tile = s_tile;
+        const int64_t base = (int64_t)tile * kRectTile;
+        if (base >= n_items) break;
+        uint32_t item[kRectItems];
+        float2 m[kRectItems];
+        int r[kRectItems];
+        const int64_t k0 = base + (int64_t)threadIdx.x * kRectItems;
+        if (k0 + kRectItems <= n_items) {
+            const uint4 q = *reinterpret_cast<const uint4*>(perm + k0);  // k0 is a multiple of 4, perm 256-byte aligned
+            item[0] = q.x;
+            item[1] = q.y;
+            item[2] = q.z;
+            item[3] = q.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < kRectItems; ++i) item[i] = k0 + i < n_items ? perm[k0 + i] : 0xffffffffu;
+        }
+#pragma unroll
+        for (int i = 0; i < kRectItems; ++i) {
+            const bool ok = item[i] < (uint32_t)n_items;  // always, unless a look-back gave up (timeout bit set)
+            r[i] = ok ? radius[item[i]] : 0;
+            m[i] = ok ? mean2d[item[i]] : make_float2(0.f, 0.f);
+        }
+        uint32_t c[kRectItems];
+        uint64_t sum = 0;
+        unsigned long long fine = 0;
+#pragma unroll
+        for (int i = 0; i < kRectItems; ++i) {
+            const int v = item[i] < (uint32_t)n_items ? (int)(item[i] / (uint32_t)sv.n_per_view) : 0;
+            int x0, x1, y0, y1;
+            c[i] = 0;
+            if (tile_rect(m[i].x, m[i].y, r[i], sv.views[v].W, sv.views[v].H, x0, x1, y0, y1)) {
+                c[i] = (uint32_t)(x1 / kSuper - x0 / kSuper + 1) * (uint32_t)(y1 / kSuper - y0 / kSuper + 1);
+                fine += (unsigned long long)(x1 - x0 + 1) * (unsigned long long)(y1 - y0 + 1);
+                const int at = threadIdx.x * kRectItems + i;
+                s_rect[at] = make_uint2((uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16));
+                s_item[at] = item[i];
+                s_view[at] = (uint8_t)v;
+            }
+            sum += c[i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fine += __shfl_xor_sync(0xffffffffu, fine, o);
+        if (lane == 0 && fine) atomicAdd(&s_fine, fine);
+        uint64_t tile_sum;
+        uint64_t at = block_excl_scan<uint64_t, kThreads>(sum, tile_sum, s_warp);
+        if (threadIdx.x == 0) st_status(status + tile, tile == 0 ? 2u : 1u, tile_sum);
+#pragma unroll
+        for (int i = 0; i < kRectItems; ++i) {
+            s_start[threadIdx.x * kRectItems + i] = (uint32_t)min(at, (uint64_t)0xffffffffu);
+            at += c[i];
+        }
+        if (warp == 0) {
+            uint64_t prefix = 0;
+            if (tile > 0) {
+                prefix = lookback_warp(status, tile, 1u, err);
+                if (lane == 0) st_status(status + tile, 2u, prefix + tile_sum);
+            }
+            if (lane == 0) {
+                s_prefix = prefix;
+                if (base + kRectTile >= n_items) *total = prefix + tile_sum;  // the last tile: the total
+            }
+        }
+        __syncthreads();
+        const uint64_t g0 = s_prefix;
+        if (coarse_tile > 0) {  // the sort takes at most `limit` pairs: its tiles start below it
+            const uint64_t hi = min(g0 + tile_sum, limit);
+            for (uint64_t ct = (g0 + coarse_tile - 1) / coarse_tile; ct * coarse_tile < hi; ++ct)
+                radix_status[ct * 256 + threadIdx.x] = 0ull;
+        }
+        const uint64_t room = g0 < limit ? min(tile_sum, limit - g0) : 0;  // below 2^32
+        for (uint64_t p64 = threadIdx.x; p64 < room; p64 += kThreads) {
+            const uint32_t p = (uint32_t)p64;
+            // the last item whose first pair is at or before p
+            int i = 0;
+#pragma unroll
+            for (int d = kRectTile / 2; d > 0; d >>= 1)
+                if (s_start[i + d] <= p) i += d;
+            const uint2 q = s_rect[i];
+            const int v = s_view[i];
+            const uint32_t x0 = q.x & 0xFFFFu, x1 = q.x >> 16, y0 = q.y & 0xFFFFu, y1 = q.y >> 16;
+            const uint32_t w = x1 / kSuper - x0 / kSuper + 1, j = p - s_start[i];
+            // below 2^21 the rounded product cannot cross an integer ((j + 1/2) / w is at least
+            // 1 / (2 w) away from one)
+            const uint32_t row = j < (1u << 21) ? (uint32_t)(((float)j + 0.5f) * __frcp_rn((float)w)) : j / w;
+            const uint32_t sx = x0 / kSuper + (j - row * w), sy = y0 / kSuper + row;
+            uint32_t key = (uint32_t)sv.st_begin[v] + sy * (uint32_t)sv.st_x[v] + sx;
+            for (int d = 0; d < passes; ++d) {
+                const uint32_t bin = (key >> (8 * d)) & 0xFFu;
+                atomicAdd(&s_h[d * 256 + bin], 1u);
+            }
+            if (pack) {  // bit 4 k + c: tile (4 sx + c, 4 sy + k) within the rectangle
+                const uint32_t cx = sx * kSuper, cy = sy * kSuper;
+                const uint32_t a = max(x0, cx) - cx, b = min(x1, cx + kSuper - 1) - cx;
+                const uint32_t e = max(y0, cy) - cy, f = min(y1, cy + kSuper - 1) - cy;
+                const uint32_t cols = ((2u << b) - (1u << a)) * 0x1111u;
+                key |= (cols & ((16u << (4 * f)) - (1u << (4 * e)))) << 16;
+            }
+            ckey[g0 + p] = key;
+            cval[g0 + p] = s_item[i];
+        }
+    }
+    // every thread left the loop through its barrier: the histograms are complete
+    if (threadIdx.x == 0 && s_fine) atomicAdd(fine_total, s_fine);
+    for (int i = threadIdx.x; i < passes * 256; i += kThreads)
+        if (s_h[i]) atomicAdd(&hist[i], s_h[i]);
 }
 
 // First position of key >= want in keys[0, n), ascending in (key & kmask).
@@ -1405,7 +1548,6 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     uint32_t* cv[2] = {U32(L.tv0), U32(L.tv1)};
     // up to 2^16 supertiles the pairs' tile masks ride in the key's high half
     const bool pack = st_bits <= 16;
-    auto dup = tight ? k_dup_coarse<true> : k_dup_coarse<false>;
     const uint32_t coarse_tile = graph ? (uint32_t)(kThreads * pass_items((uint64_t)capacity)) : 0u;
     // per-supertile instance counts and their order, largest first, in the depth keys'
     // buffers (free once the depth sort is done), when they fit
@@ -1417,9 +1559,21 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     uint32_t* st_end = nst <= n ? dv[1] : nullptr;
     if ((e = record_kernel_event(GS_KERNEL_DUPLICATE, false, s)) != cudaSuccess)
         return cuda_status(e, "gs_bin_sort: kernel event");
-    dup<<<(int)cdiv(n, kDupTile), kThreads, 0, s>>>(n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes,
-                                                    pack, tickets, dup_status, ck[0], cv[0], hist + 256 * 4, ctotal,
-                                                    fine_total, status, coarse_tile, st_count, nst, err);
+    int dev_sms = 0;
+    {
+        int dev = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&dev_sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+            return cuda_status(e, "gs_bin_sort: device");
+    }
+    if (tight)
+        k_dup_coarse<<<(int)cdiv(n, kDupTile), kThreads, 0, s>>>(
+            n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
+            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, err);
+    else
+        k_dup_rect<<<(int)std::min<int64_t>(cdiv(n, kRectTile), 6 * (int64_t)dev_sms), kThreads, 0, s>>>(
+            n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
+            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, err);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: duplicate");
     if ((e = record_kernel_event(GS_KERNEL_DUPLICATE, true, s)) != cudaSuccess)
@@ -1460,14 +1614,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     // the pairs' tile masks go to the free half of the pair buffers (2 bytes per pair)
     uint16_t* masks = reinterpret_cast<uint16_t*>(ck[which ^ 1]);
     auto pair_masks = tight ? k_pair_masks<true> : k_pair_masks<false>;
-    int pair_grid = 0;  // at most 8 blocks per SM, each warp taking segments of pairs
-    {
-        int dev = 0, sms = 0;
-        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
-            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
-            return cuda_status(e, "gs_bin_sort: device");
-        pair_grid = 8 * sms;
-    }
+    const int pair_grid = 8 * dev_sms;  // at most 8 blocks per SM, each warp taking segments of pairs
     pair_masks<<<(int)std::min<int64_t>(pair_grid, cdiv(I_grid, (int64_t)kPairBatch * (kThreads / 32))), kThreads, 0,
                  s>>>(
         sv2, mean2d, radius, ck[which], cv[which], I_grid, ctotal, (uint32_t)n, pack, masks, tile_ranges, st_count,
