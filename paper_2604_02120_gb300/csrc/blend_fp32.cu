@@ -2,6 +2,17 @@
 // 16 x 16 tile, one thread per pixel; the tile's list is staged through shared
 // memory in batches of 256 splats (Sec. 2.1 (d)).  The exponent is evaluated
 // per pixel as the quadratic of Eq. 3 in FP32.
+//
+// Both kernels are bound by the instructions of a (splat, warp) pair: 20 to 25
+// forward, about 100 backward with its sums over the warp.  So a warp holds an
+// 8 x 4 block (a square reaches fewer splats than a strip of 16 x 2), its lanes
+// test 32 staged splats at a time against that block (warp_reaches, about one
+// instruction per pair) and only the splats that can contribute are walked, in
+// list order and with their list positions: the same decisions and the same
+// values as the walk over all.  Full rectangles, forward and backward:
+// 641 x 479, 50k splats 107 -> 61 us and 225 -> 154 us; 1920 x 1080, 1M
+// clustered 994 -> 398 us and 2207 -> 1238 us (issue slots 86% and 75% busy).
+#include "blend_tc.cuh"
 #include "internal.h"
 
 namespace gs {
@@ -15,7 +26,7 @@ constexpr float kTMin = 1e-4f;
 struct SplatSm {
     float4 geo;  // mx, my, A, B
     float4 oc;   // C, o, r, g
-    float b;
+    float2 bl;   // b, log2 o
 };
 
 // alpha of a splat at a pixel; `e` receives exp(min(power, 0)) and `pw` power.
@@ -35,12 +46,23 @@ __device__ __forceinline__ void load_splat(const BlendArgs& a, uint32_t g, uint3
     const float2 m = a.mean2d[g];
     s.geo = make_float4(m.x, m.y, a.conic[3 * g], a.conic[3 * g + 1]);
     s.oc = make_float4(a.conic[3 * g + 2], a.opac[g - opac_off], a.rgb[3 * g], a.rgb[3 * g + 1]);
-    s.b = a.rgb[3 * g + 2];
+    s.bl = make_float2(a.rgb[3 * g + 2], __log2f(s.oc.y));
+}
+
+// Whether the splat may reach alpha >= 1/255 at a pixel of the warp's 8 x 4
+// block, whose first pixel centre is (x, y).  splat_alpha's own error is within
+// 2^-20 of the magnitude sum; the test leaves it eight times that.
+__device__ __forceinline__ bool warp_reaches(const float4& geo, const float4& oc, float l2o, float x, float y) {
+    const float x1 = geo.x - x, x0 = x1 - 7.0f, y1 = geo.y - y, y0 = y1 - 3.0f;
+    const float ax = fmaxf(fabsf(x0), fabsf(x1)), ay = fmaxf(fabsf(y0), fabsf(y1));
+    const float S = fmaf(0.5f * fabsf(geo.z) * ax, ax, fmaf(fabsf(geo.w) * ax, ay, 0.5f * fabsf(oc.x) * ay * ay));
+    return tc::box_reaches(geo.z, geo.w, oc.x, l2o, x0, x1, y0, y1, S, 1.0f / 131072);
 }
 
 // Geometry of the block's tile (blockIdx.x is a global tile id).
 struct TileGeo {
     int W, H, px, py;
+    float bx, by;  // first pixel centre of the warp's 8 x 4 block
     long long pix_off;
     uint32_t opac_off;
 };
@@ -52,8 +74,12 @@ __device__ __forceinline__ TileGeo tile_geo(const BlendArgs& a, int tile) {
     TileGeo t;
     t.W = vd.W;
     t.H = vd.H;
-    t.px = (lt % vd.tiles_x) * kTile + (threadIdx.x & 15);
-    t.py = (lt / vd.tiles_x) * kTile + (threadIdx.x >> 4);
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int x = (lt % vd.tiles_x) * kTile + 8 * (w & 1), y = (lt / vd.tiles_x) * kTile + 4 * (w >> 1);
+    t.px = x + (lane & 7);
+    t.py = y + (lane >> 3);
+    t.bx = x + 0.5f;
+    t.by = y + 0.5f;
     t.pix_off = vd.pix_off;
     t.opac_off = (uint32_t)(v * a.n_per_view);
     return t;
@@ -62,12 +88,13 @@ __device__ __forceinline__ TileGeo tile_geo(const BlendArgs& a, int tile) {
 __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant__ BlendArgs a) {
     __shared__ float4 s_geo[kBatch];
     __shared__ float4 s_oc[kBatch];
-    __shared__ float s_b[kBatch];
+    __shared__ float2 s_bl[kBatch];
     const int tile = tile_at(a, blockIdx.x * a.shard_count + a.shard_index);
     const TileGeo tg = tile_geo(a, tile);
     const int px = tg.px, py = tg.py;
     const bool inside = px < tg.W && py < tg.H;
     const float xp = px + 0.5f, yp = py + 0.5f;
+    const int lane = threadIdx.x & 31;
     const uint32_t start = a.ranges[2 * tile], end = a.ranges[2 * tile + 1];
     const int len = end > start ? (int)(end - start) : 0;
 
@@ -82,26 +109,33 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
             load_splat(a, a.ids[start + i], tg.opac_off, s);
             s_geo[threadIdx.x] = s.geo;
             s_oc[threadIdx.x] = s.oc;
-            s_b[threadIdx.x] = s.b;
+            s_bl[threadIdx.x] = s.bl;
         }
         __syncthreads();
         const int nb = min(kBatch, len - base);
-        for (int j = 0; !done && j < nb; ++j) {
-            const float4 geo = s_geo[j], oc = s_oc[j];
-            float e, pw, dx, dy;
-            const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
-            if (alpha < kAlphaMin) continue;
-            const float tT = T * (1.0f - alpha);
-            if (tT < kTMin) {
-                done = true;
-                break;
+        for (int c = 0; c < nb; c += 32) {
+            if (__all_sync(0xffffffffu, done)) break;
+            const int t = c + lane;
+            unsigned hits =
+                __ballot_sync(0xffffffffu, t < nb && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
+            for (; hits; hits &= hits - 1) {
+                const int j = c + __ffs(hits) - 1;
+                const float4 geo = s_geo[j], oc = s_oc[j];
+                float e, pw, dx, dy;
+                const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
+                if (done || alpha < kAlphaMin) continue;
+                const float tT = T * (1.0f - alpha);
+                if (tT < kTMin) {
+                    done = true;
+                    continue;
+                }
+                const float w = alpha * T;
+                cr = __fmaf_rn(oc.z, w, cr);
+                cg = __fmaf_rn(oc.w, w, cg);
+                cb = __fmaf_rn(s_bl[j].x, w, cb);
+                T = tT;
+                last = base + j + 1;
             }
-            const float w = alpha * T;
-            cr = __fmaf_rn(oc.z, w, cr);
-            cg = __fmaf_rn(oc.w, w, cg);
-            cb = __fmaf_rn(s_b[j], w, cb);
-            T = tT;
-            last = base + j + 1;
         }
     }
     if (inside) {
@@ -160,7 +194,7 @@ __device__ __forceinline__ float* grad_slot(const GradArgs& gr, uint32_t g, uint
 __global__ void __launch_bounds__(kBatch) k_blend_fp32_bwd(const __grid_constant__ BlendArgs a, GradArgs gr) {
     __shared__ float4 s_geo[kBatch];
     __shared__ float4 s_oc[kBatch];
-    __shared__ float s_b[kBatch];
+    __shared__ float2 s_bl[kBatch];
     __shared__ uint32_t s_id[kBatch];
     __shared__ int s_max;
     const int tile = tile_at(a, blockIdx.x * a.shard_count + a.shard_index);
@@ -202,60 +236,65 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_bwd(const __grid_constant
             load_splat(a, g, tg.opac_off, s);
             s_geo[threadIdx.x] = s.geo;
             s_oc[threadIdx.x] = s.oc;
-            s_b[threadIdx.x] = s.b;
+            s_bl[threadIdx.x] = s.bl;
             s_id[threadIdx.x] = g;
         }
         __syncthreads();
         // this warp only needs list positions below its largest n_contrib
-        for (int j = min(hi, wmax) - 1; j >= lo; --j) {
-            const int k = j - lo;
-            const float4 geo = s_geo[k], oc = s_oc[k];
-            const float cb = s_b[k];
-            float v[9];
+        for (int top = min(hi, wmax); top > lo; top -= 32) {
+            const int t = top - 1 - lane - lo;
+            unsigned hits =
+                __ballot_sync(0xffffffffu, t >= 0 && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
+            for (; hits; hits &= hits - 1) {
+                const int j = top - __ffs(hits), k = j - lo;
+                const float4 geo = s_geo[k], oc = s_oc[k];
+                const float cb = s_bl[k].x;
+                float v[9];
 #pragma unroll
-            for (int q = 0; q < 9; ++q) v[q] = 0.f;
-            bool contrib = false;
-            if (j < nc) {
-                float e, pw, dx, dy;
-                const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
-                if (alpha >= kAlphaMin) {
-                    contrib = true;
-                    const float Ti = __fdividef(T, 1.0f - alpha);
-                    const float wgt = alpha * Ti;
-                    v[6] = wgt * g0;
-                    v[7] = wgt * g1;
-                    v[8] = wgt * g2;
-                    const float dL_dalpha = Ti * ((oc.z - S0) * g0 + (oc.w - S1) * g1 + (cb - S2) * g2);
-                    S0 = fmaf(alpha, oc.z - S0, S0);
-                    S1 = fmaf(alpha, oc.w - S1, S1);
-                    S2 = fmaf(alpha, cb - S2, S2);
-                    T = Ti;
-                    if (oc.y * e <= kAlphaMax) {  // not clamped
-                        v[5] = dL_dalpha * e;
-                        if (pw <= 0.0f) {
-                            const float dp = dL_dalpha * alpha;
-                            v[0] = -dp * (geo.z * dx + geo.w * dy);
-                            v[1] = -dp * (geo.w * dx + oc.x * dy);
-                            v[2] = -0.5f * dp * dx * dx;
-                            v[3] = -dp * dx * dy;
-                            v[4] = -0.5f * dp * dy * dy;
+                for (int q = 0; q < 9; ++q) v[q] = 0.f;
+                bool contrib = false;
+                if (j < nc) {
+                    float e, pw, dx, dy;
+                    const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
+                    if (alpha >= kAlphaMin) {
+                        contrib = true;
+                        const float Ti = __fdividef(T, 1.0f - alpha);
+                        const float wgt = alpha * Ti;
+                        v[6] = wgt * g0;
+                        v[7] = wgt * g1;
+                        v[8] = wgt * g2;
+                        const float dL_dalpha = Ti * ((oc.z - S0) * g0 + (oc.w - S1) * g1 + (cb - S2) * g2);
+                        S0 = fmaf(alpha, oc.z - S0, S0);
+                        S1 = fmaf(alpha, oc.w - S1, S1);
+                        S2 = fmaf(alpha, cb - S2, S2);
+                        T = Ti;
+                        if (oc.y * e <= kAlphaMax) {  // not clamped
+                            v[5] = dL_dalpha * e;
+                            if (pw <= 0.0f) {
+                                const float dp = dL_dalpha * alpha;
+                                v[0] = -dp * (geo.z * dx + geo.w * dy);
+                                v[1] = -dp * (geo.w * dx + oc.x * dy);
+                                v[2] = -0.5f * dp * dx * dx;
+                                v[3] = -dp * dx * dy;
+                                v[4] = -0.5f * dp * dy * dy;
+                            }
                         }
                     }
                 }
-            }
-            const unsigned who = __ballot_sync(0xffffffffu, contrib);
-            if (who == 0u) continue;
-            const uint32_t g = s_id[k];
-            if (__popc(who) <= 3) {
-                if (contrib) {
+                const unsigned who = __ballot_sync(0xffffffffu, contrib);
+                if (who == 0u) continue;
+                const uint32_t g = s_id[k];
+                if (__popc(who) <= 3) {
+                    if (contrib) {
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) atomicAdd(grad_slot(gr, g, tg.opac_off, q), v[q]);
+                        for (int q = 0; q < 9; ++q) atomicAdd(grad_slot(gr, g, tg.opac_off, q), v[q]);
+                    }
+                } else {
+                    float vk, v8;
+                    warp_reduce9(v, lane, vk, v8);
+                    if ((lane & 3) == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, lane >> 2), vk);
+                    if (lane == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, 8), v8);
                 }
-            } else {
-                float vk, v8;
-                warp_reduce9(v, lane, vk, v8);
-                if ((lane & 3) == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, lane >> 2), vk);
-                if (lane == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, 8), v8);
             }
         }
     }

@@ -127,7 +127,7 @@ __device__ __forceinline__ float from_op(uint16_t b) {
     else return __bfloat162float(__ushort_as_bfloat16(b));
 }
 
-// Per-splat record of the backward and the fused small-scene kernels: colour
+// Per-splat record of the fused small-scene kernel: colour
 // duplicated for both pixels of a lane and the exponent ceiling min(log2 0.99, log2 o).
 // (The forward's epilogue reads (r, g, b, cap) as one float4: a warp-wide broadcast
 // of 16 bytes costs four cycles of the SM's shared-memory pipe.)
@@ -230,23 +230,15 @@ constexpr float reach_rel() {
            : V == GS_BLEND_TC_FP8_SPLIT ? 1.0f / 256 : 1.0f / 131072;
 }
 
-// False only if the splat's alpha, in the variant's own arithmetic, is below
-// 1/255 at every pixel of the tile; such a splat changes no pixel (the skip
-// rule of Alg. 1) and its MMA columns and compositing can be left out.  The
-// largest quadratic over the box of pixel offsets is compared with the
-// threshold, lowered by 0.3 in base-2 units (more than coeff_row's own test of
-// far splats allows) and by reach_rel of the magnitude sum S at offsets
-// enlarged by 24 px (which covers either reference pixel).  A sum that is not
-// finite keeps the splat.  (xh, yh): splat centre minus the upper half's
-// reference; bx0..by1: the offsets of that half's pixels from it.
-template <int V>
-__device__ __forceinline__ bool splat_reaches(float A, float B, float C, float l2o, float xh, float yh, float bx0,
-                                              float bx1, float by0, float by1) {
-    const float ax = fabsf(xh) + 24.f, ay = fabsf(yh) + 24.f;
-    const float S = fmaf(0.5f * fabsf(A) * ax, ax, fmaf(fabsf(B) * ax, ay, 0.5f * fabsf(C) * ay * ay));
+// False only if a splat's alpha is below 1/255 at every pixel of a box; x0..x1
+// and y0..y1 are the pixels' offsets from the splat's centre.  The largest
+// quadratic over the box is compared with the threshold, lowered by 0.3 in
+// base-2 units and by `rel` of the magnitude sum S of Eq. 3's terms (what the
+// caller's arithmetic may be off).  A sum that is not finite keeps the splat.
+__device__ __forceinline__ bool box_reaches(float A, float B, float C, float l2o, float x0, float x1, float y0,
+                                            float y1, float S, float rel) {
     // the maximum over the box lies on the two lines nearest to the splat's centre
     // (a definite form; a nearly singular or indefinite one is kept)
-    const float x0 = xh + bx0, x1 = xh + bx1, y0 = yh + by0 - 8.0f, y1 = yh + by1;
     const float ex = fminf(fmaxf(0.f, x0), x1), ey = fminf(fmaxf(0.f, y0), y1);
     const float dy = fminf(fmaxf(__fdividef(-B * ex, C), y0), y1);
     const float dx = fminf(fmaxf(__fdividef(-B * ey, A), x0), x1);
@@ -254,8 +246,22 @@ __device__ __forceinline__ bool splat_reaches(float A, float B, float C, float l
     const float qy = fmaf(A * dx, dx, fmaf(2.f * B * dx, ey, C * ey * ey));
     const float p = fmaf(-0.5f * kLog2e, fminf(qx, qy), l2o);
     const bool definite = A > 0.f && C > 0.f && A * C > B * B;
-    return !(S < 1e30f && ((definite && fmaf(reach_rel<V>(), S, p) < kLog2AlphaMin - 0.3f) ||
-                           l2o < kLog2AlphaMin - 0.3f));
+    return !(S < 1e30f && ((definite && fmaf(rel, S, p) < kLog2AlphaMin - 0.3f) || l2o < kLog2AlphaMin - 0.3f));
+}
+
+// False only if the splat's alpha, in the variant's own arithmetic, is below
+// 1/255 at every pixel of the tile; such a splat changes no pixel (the skip
+// rule of Alg. 1) and its MMA columns and compositing can be left out.  The
+// margin (0.3 in base-2 units) is more than coeff_row's own test of far splats
+// allows; S is taken at offsets enlarged by 24 px (which covers either
+// reference pixel).  (xh, yh): splat centre minus the upper half's reference;
+// bx0..by1: the offsets of that half's pixels from it.
+template <int V>
+__device__ __forceinline__ bool splat_reaches(float A, float B, float C, float l2o, float xh, float yh, float bx0,
+                                              float bx1, float by0, float by1) {
+    const float ax = fabsf(xh) + 24.f, ay = fabsf(yh) + 24.f;
+    const float S = fmaf(0.5f * fabsf(A) * ax, ax, fmaf(fabsf(B) * ax, ay, 0.5f * fabsf(C) * ay * ay));
+    return box_reaches(A, B, C, l2o, xh + bx0, xh + bx1, yh + by0 - 8.0f, yh + by1, S, reach_rel<V>());
 }
 
 // Coefficient row of Eq. 6 for one splat and one reference pixel, in base-2
