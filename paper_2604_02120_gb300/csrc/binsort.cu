@@ -28,7 +28,8 @@
 // for blocks that started before it, so the waits always end; each is still
 // bounded in time and sets the timeout bit of the error word if it gives up.
 // The scan of coarse counts in depth order is done the same way inside the
-// duplication kernel, so the whole stage is
+// duplication kernels (k_dup_rect for full rectangles, k_dup_coarse for
+// opacity-aware lists), so the whole stage is
 //   memset, keys, 4 depth passes, coarse duplicate, ceil(bits / 8) supertile
 //   passes, tile counts, tile scan, fine write.
 #include <algorithm>
@@ -41,8 +42,7 @@ namespace {
 
 constexpr int kThreads = 256;
 constexpr uint32_t kSmallPass = 1u << 20;  // passes up to this size use 1024-item tiles, larger ones 4096
-constexpr int kDupItems = 1;                // items per thread of the duplication kernel
-constexpr int kDupTile = kThreads * kDupItems;
+constexpr int kDupTile = kThreads;          // items per tile of the opacity-aware duplication
 constexpr int kMaxPasses = 8;               // 4 depth passes + up to 4 tile-id passes
 constexpr uint64_t kLookbackLimitNs = 2000000000ull;
 
@@ -474,13 +474,12 @@ __device__ __forceinline__ Runs4 row_runs(const TightRows& t, int sy, int x0, in
 #pragma unroll
     for (int k = 0; k < kSuper; ++k) {
         const int y = sy * kSuper + k;
-        int f = 1, l = 0;
-        if (y >= y0 && y <= y1) {
-            tight_row(t, y, x0, x1, f, l);
-        }
+        int f, l;
+        tight_row(t, y, x0, x1, f, l);
+        if (y < y0 || y > y1) l = f - 1;
         rr.f[k] = f;
         rr.l[k] = l;
-        if (f <= l) *fine += (uint32_t)(l - f + 1);
+        *fine += (uint32_t)max(l - f + 1, 0);
     }
     return rr;
 }
@@ -494,54 +493,6 @@ __device__ __forceinline__ int runs_union(const Runs4& rr, F emit) {
     for (int k = 0; k < kSuper; ++k)
         r[k] = rr.f[k] <= rr.l[k] ? Iv{rr.f[k] / kSuper, rr.l[k] / kSuper} : Iv{0x7fffffff, -1};
     return iv_union4(r[0], r[1], r[2], r[3], emit);
-}
-
-// Deals the work units of a warp's items (lane l's item has units[l] of
-// them: its supertile rows) out to the lanes, 32 per round, in lane-then-unit
-// order, so that every lane evaluates one supertile row whatever the spread
-// of the items' heights.  body(active, src, u, f) runs on every lane each
-// round: src is the lane whose item the unit belongs to, u the unit's index
-// within that item, f its index among the warp's units; active is false on
-// the idle lanes of the last round.
-template <class F>
-__device__ __forceinline__ void warp_units(uint32_t units, F body) {
-    const int lane = threadIdx.x & 31;
-    uint32_t incl = units;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
-        if (lane >= d) incl += v;
-    }
-    const uint32_t excl = incl - units, total = __shfl_sync(0xffffffffu, incl, 31);
-    for (uint32_t r0 = 0; r0 < total; r0 += 32) {
-        const uint32_t f = r0 + (uint32_t)lane;
-        // the last lane whose first unit is at or before f (the first units are nondecreasing)
-        int src = 0;
-        uint32_t start = 0;
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-            const uint32_t v = __shfl_sync(0xffffffffu, excl, src + d);
-            if (v <= f) {
-                src += d;
-                start = v;
-            }
-        }
-        body(f < total, src, f - start, f);
-    }
-}
-
-__device__ __forceinline__ TightRows shfl_rows(const TightRows& t, int src) {
-    TightRows b;
-    b.mode = __shfl_sync(0xffffffffu, t.mode, src);
-    b.mx = __shfl_sync(0xffffffffu, t.mx, src);
-    b.my = __shfl_sync(0xffffffffu, t.my, src);
-    b.nB = __shfl_sync(0xffffffffu, t.nB, src);
-    b.det = __shfl_sync(0xffffffffu, t.det, src);
-    b.Atau = __shfl_sync(0xffffffffu, t.Atau, src);
-    b.rA = __shfl_sync(0xffffffffu, t.rA, src);
-    b.ymax = __shfl_sync(0xffffffffu, t.ymax, src);
-    b.dyr = __shfl_sync(0xffffffffu, t.dyr, src);
-    return b;
 }
 
 // Per item: its depth key and index (the depth sort's input) and the keys'
@@ -584,28 +535,6 @@ __global__ void __launch_bounds__(kThreads) k_keys(int n_items, const float* __r
         if (s_h[i]) atomicAdd(&hist[i], s_h[i]);
 }
 
-// Digit histograms of the tile ids [a, a + w) of one rectangle row, by runs:
-// a run inside one aligned block of 256 ids has constant digits 1..3, and its
-// digit-0 values form a contiguous range, added to the difference array s_d0
-// (the histogram of digit 0 is its prefix sum).
-__device__ __forceinline__ void row_hist(uint32_t a, uint32_t w, int passes, int* s_d0, uint32_t* s_h) {
-    while (w > 0) {
-        const uint32_t lo = a & 0xFFu, len = min(w, 256u - lo);
-        atomicAdd(&s_d0[lo], 1);
-        atomicSub(&s_d0[lo + len], 1);
-        for (int p = 1; p < passes; ++p) atomicAdd(&s_h[(p - 1) * 256 + ((a >> (8 * p)) & 0xFFu)], len);
-        a += len;
-        w -= len;
-    }
-}
-
-// Digit histograms of one tile id (the wide-row path: one id per lane).
-__device__ __forceinline__ void key_hist(uint32_t a, int passes, int* s_d0, uint32_t* s_h) {
-    atomicAdd(&s_d0[a & 0xFFu], 1);
-    atomicSub(&s_d0[(a & 0xFFu) + 1], 1);
-    for (int p = 1; p < passes; ++p) hist_add(s_h, (p - 1) * 256 + ((a >> (8 * p)) & 0xFFu));
-}
-
 // A unit's runs in four words (16 bits per end; an empty run as (1, 0)).
 __device__ __forceinline__ uint4 pack_runs(const Runs4& rr) {
     uint32_t w[kSuper];
@@ -626,243 +555,280 @@ __device__ __forceinline__ Runs4 unpack_runs(uint4 v) {
 }
 
 // Coarse duplication in depth order of opacity-aware lists, with the supertile
-// counts and their scan folded in.  Tile t (from the ticket) holds the depth-ordered items
-// [t * kDupTile, (t + 1) * kDupTile).  Each warp deals its items' supertile
-// rows out to its lanes (warp_units) and evaluates every row's tile runs once,
-// keeping them in shared memory (the first kStashUnits of each warp; later
-// ones are evaluated again when written): the items' supertile counts and the
-// instance count, added into *fine_total.  The tile's pair count goes out for
-// the decoupled look-back over the tiles before it.  Each item then emits one
-// (global supertile id, item) pair per supertile it touches, supertile rows in
-// order, placed by a warp scan of the rows' pair counts; a row of more than
-// kWideRow supertiles is emitted by the whole warp, one supertile column per
-// lane.  A tile of at most kStagePairs pairs emits them into shared memory
-// before its look-back (so the predecessors' prefixes are usually there by
-// then) and copies them out with consecutive threads on consecutive pairs; a
-// larger tile looks back first and writes them directly.  With `pack` the
-// key's high half holds the pair's 16-bit tile mask (runs_mask).  Writes stop
-// at `limit`; the pair total goes to *total.  The digit histograms of the
-// written pairs' supertile ids go to hist (passes of them), so a truncated
-// list still sorts into a permutation of what was written.  With coarse_tile
-// > 0 the block also clears the look-back status words (256 per radix tile,
-// at radix_status) of the pair sort's tiles that start within its pairs
-// (below `limit`), and the blocks together zero st_zero[0, st_n).
-constexpr uint32_t kWideRow = 8;
-constexpr uint32_t kStashUnits = 128;  // per warp
-constexpr uint32_t kStagePairs = 2048;
-__global__ void __launch_bounds__(kThreads) k_dup_coarse(int n_items, const uint32_t* __restrict__ perm,
-                                                         const __grid_constant__ SortViews sv,
-                                                         const float2* __restrict__ mean2d,
-                                                         const int* __restrict__ radius, uint64_t limit, int passes,
-                                                         bool pack, uint32_t* tickets, unsigned long long* status,
-                                                         uint32_t* __restrict__ ckey, uint32_t* __restrict__ cval,
-                                                         uint32_t* __restrict__ hist, uint64_t* __restrict__ total,
-                                                         unsigned long long* __restrict__ fine_total,
-                                                         unsigned long long* __restrict__ radix_status,
-                                                         uint32_t coarse_tile, uint32_t* __restrict__ st_zero,
-                                                         int st_n, unsigned* err) {
-    __shared__ uint64_t s_warp[kThreads / 32 + 1];
+// counts and their scan folded in.  Persistent blocks take tiles of kDupTile
+// depth-ordered items from the ticket.  A unit is one supertile row of an item:
+// the block deals the tile's units out to its threads (a run of consecutive
+// ones each, found by a search over the items' first units), evaluates each
+// one's four tile runs once into shared memory with its supertile count, scans
+// the counts and publishes the sum.  It then makes one (global supertile id,
+// item) pair per supertile touched, supertile rows in order, consecutive
+// threads on consecutive pairs: a search over the units' first pairs names the
+// unit, and with `pack` the key's high half holds the pair's 16-bit tile mask.
+// Up to kStagePairs pairs are made into shared memory, then the look-back
+// gives their place and they are copied out; a tile of more looks back first.
+// A tile of more than kStash units goes in batches, evaluated once for the
+// count and once more for the pairs.  Writes stop at `limit`; the pair total
+// goes to *total and the instance count to *fine_total.  The digit histograms
+// of the written pairs' supertile ids go to hist (passes of them), so a
+// truncated list still sorts into a permutation of what was written; they stay
+// in shared memory over all tiles of a block.  With coarse_tile > 0 the block
+// also clears the look-back status words (256 per radix tile, at radix_status)
+// of the pair sort's tiles that start within its pairs (below `limit`), and
+// the blocks together zero st_zero[0, st_n).
+//
+// Bound by issue slots (55%) and by waits of every kind in a tile's chain of
+// about 34000 cycles: 20% the gathers of the items, 20% evaluating, 17% making
+// pairs, 17% the look-back.  Nothing may wait between a tile's ticket and its
+// sum: drawing the next ticket before the look-back's end (to load its items
+// early) made the look-backs wait for one another, 469 us.  3840 x 2160, 3M
+// splats, 7.2M units, 14.1M pairs: one block per tile with a row's pairs
+// written by its lane 674 us; this kernel 308 us, without the staged pairs 320,
+// with 3 / 5 blocks per SM 333 / 370 us.
+__device__ __forceinline__ uint32_t pack16(int lo, int hi) { return __byte_perm((uint32_t)lo, (uint32_t)hi, 0x5410); }
+// Byte k: table[min(max(v[k] + add, 0), 4)] of the 16-bit values v[0..3] in a and b
+// (entry 4 is 0).
+__device__ __forceinline__ uint32_t nibbles(uint32_t table, uint32_t a, uint32_t b, uint32_t add) {
+    const uint32_t x = __viaddmin_s16x2_relu(a, add, 0x00040004u) | __viaddmin_s16x2_relu(b, add, 0x00040004u) << 8;
+    return __byte_perm(table, 0u, x | x >> 12);
+}
+constexpr uint32_t kStash = 832;
+constexpr uint32_t kStagePairs = 1536;
+constexpr int kDupBlocks = 4;  // per SM
+constexpr uint32_t kMaxSpan = 8000;  // supertiles of a unit whose relative runs fit 16 bits
+__global__ void __launch_bounds__(kThreads, kDupBlocks)
+    k_dup_coarse(int n_items, const uint32_t* __restrict__ perm, const __grid_constant__ SortViews sv,
+                 const float2* __restrict__ mean2d, const int* __restrict__ radius, uint64_t limit, int passes,
+                 bool pack, uint32_t* tickets, unsigned long long* status, uint32_t* __restrict__ ckey,
+                 uint32_t* __restrict__ cval, uint32_t* __restrict__ hist, uint64_t* __restrict__ total,
+                 unsigned long long* __restrict__ fine_total, unsigned long long* __restrict__ radix_status,
+                 uint32_t coarse_tile, uint32_t* __restrict__ st_zero, int st_n, unsigned* err) {
+    __shared__ uint32_t s_warp[kThreads / 32 + 1];
     __shared__ uint64_t s_prefix;
-    __shared__ unsigned long long s_fine;
+    __shared__ uint32_t s_tile;
+    __shared__ uint32_t s_h[4 * 256];
+    // per item of the tile
+    __shared__ uint32_t s_u[kDupTile + 1];  // its first unit
+    __shared__ uint2 s_rect[kDupTile];      // x0 | x1 << 16, y0 | y1 << 16 in tiles
+    __shared__ float4 s_ta[kDupTile], s_tb[kDupTile];  // its TightRows
+    __shared__ uint32_t s_item[kDupTile];
+    __shared__ uint32_t s_row[kDupTile], s_stx[kDupTile];  // id of supertile 0 in its first row, ids per row
+    __shared__ uint8_t s_mode[kDupTile];
+    // per unit of the batch
+    __shared__ uint4 s_runs[kStash];     // relative to the first supertile (general: pack_runs)
+    __shared__ uint32_t s_p[1024];       // its first pair
+    __shared__ uint32_t s_key[kStash];   // id of its first supertile (general: of its row's supertile 0)
+    __shared__ uint16_t s_who[kStash];   // item | general << 15
+    static_assert(kDupTile <= 256 && kStash <= 1024);
+    // the tile's pairs, made before the look-back (up to kStagePairs)
+    __shared__ uint32_t s_pk[kStagePairs];
+    __shared__ uint8_t s_pv[kStagePairs];
     if (st_zero != nullptr)  // the supertile counters of k_pair_masks
         for (int i = blockIdx.x * kThreads + threadIdx.x; i < st_n; i += gridDim.x * kThreads) st_zero[i] = 0;
-    __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_h[3 * 256];  // digits 1..3
-    __shared__ int s_d0[257];          // digit 0, as a difference array
-    __shared__ int s_warp_i[kThreads / 32 + 1];
-    __shared__ uint32_t s_c[kThreads];  // per lane: its item's supertile count
-    __shared__ uint4 s_runs[(kThreads / 32) * kStashUnits];
-    __shared__ uint8_t s_n[(kThreads / 32) * kStashUnits];
-    __shared__ uint32_t s_pk[kStagePairs], s_pv[kStagePairs];
+    for (int i = threadIdx.x; i < passes * 256; i += kThreads) s_h[i] = 0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) {
-        s_tile = atomicAdd(&tickets[kMaxPasses], 1u);
-        s_fine = 0;
-    }
-    for (int i = threadIdx.x; i < 3 * 256; i += kThreads) s_h[i] = 0;
-    for (int i = threadIdx.x; i < 257; i += kThreads) s_d0[i] = 0;
-    __syncthreads();
-    const uint32_t tile = s_tile;
-    const int64_t base = (int64_t)tile * kDupTile;
-    if (base >= n_items) return;
-
-    const int64_t k = base + threadIdx.x;
-    const uint32_t item = k < n_items ? perm[k] : 0u;
-    int x0 = 0, x1 = -1, y0 = 0, y1 = -1, stx = 0, stb = 0;
-    bool vis = false;
-    TightRows t{};
-    if (k < n_items) {
-        const int v = (int)(item / (uint32_t)sv.n_per_view);
-        const ViewDesc& vd = sv.views[v];
-        const float2 m = mean2d[item];
-        vis = tile_rect(m.x, m.y, radius[item], vd.W, vd.H, x0, x1, y0, y1);
-        stx = sv.st_x[v];
-        stb = sv.st_begin[v];
-        if (vis) t = item_tight_rows(sv, mean2d, item);
-    }
-    const uint32_t units = vis ? (uint32_t)(y1 / kSuper - y0 / kSuper + 1) : 0u;
-    uint4* stash = s_runs + warp * kStashUnits;
-    uint8_t* stash_n = s_n + warp * kStashUnits;
-    const int wlane0 = threadIdx.x & ~31;
-
-    // every unit's runs once: the items' supertile counts and the instance count
-    s_c[threadIdx.x] = 0;
-    __syncwarp();
-    uint32_t fine = 0;
-    warp_units(units, [&](bool act, int src, uint32_t u, uint32_t f) {
-        const int bx0 = __shfl_sync(0xffffffffu, x0, src), bx1 = __shfl_sync(0xffffffffu, x1, src);
-        const int by0 = __shfl_sync(0xffffffffu, y0, src), by1 = __shfl_sync(0xffffffffu, y1, src);
-        const TightRows bt = shfl_rows(t, src);
-        if (act) {
-            const Runs4 rr = row_runs(bt, by0 / kSuper + (int)u, bx0, bx1, by0, by1, &fine);
-            const int n = runs_union(rr, [](int, int) {});
-            atomicAdd(&s_c[wlane0 + src], (uint32_t)n);
-            if (f < kStashUnits) {
-                stash[f] = pack_runs(rr);
-                stash_n[f] = (uint8_t)min(n, 255);
-            }
-        }
-    });
-    __syncwarp();
-    const uint32_t c = s_c[threadIdx.x];
-    if (fine) atomicAdd(&s_fine, (unsigned long long)fine);
-
-    uint64_t tile_sum;
-    const uint64_t local = block_excl_scan<uint64_t, kThreads>((uint64_t)c, tile_sum, s_warp);
-    unsigned long long* mine = status + tile;
-    const bool staged = tile_sum <= kStagePairs;  // uniform over the block
-    if (warp == 0 && lane == 0) st_status(mine, tile == 0 ? 2u : 1u, tile_sum);
-    // the tile's offset among all pairs: the look-back, then the clears that need it
-    auto resolve = [&]() {
-        if (warp == 0) {
-            uint64_t prefix = 0;
-            if (tile > 0) {
-                prefix = lookback_warp(status, tile, 1u, err);
-                if (lane == 0) st_status(mine, 2u, prefix + tile_sum);
-            }
-            if (lane == 0) {
-                s_prefix = prefix;
-                if (base + kDupTile >= n_items) *total = prefix + tile_sum;  // the last tile: the total
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x == 0 && s_fine) atomicAdd(fine_total, s_fine);
-        if (coarse_tile > 0) {
-            // the sort takes at most `limit` pairs: its tiles start below it
-            const uint64_t lo = s_prefix, hi = min(s_prefix + tile_sum, limit);
-            for (uint64_t ct = (lo + coarse_tile - 1) / coarse_tile; ct * coarse_tile < hi; ++ct)
-                radix_status[ct * 256 + threadIdx.x] = 0ull;
-        }
+    unsigned long long fine = 0;
+    auto count = [&](uint32_t key) {  // into the digit histograms (with `pack` the id is the low half)
+        for (int d = 0; d < passes; ++d) atomicAdd(&s_h[d * 256 + ((key >> (8 * d)) & 0xFFu)], 1u);
     };
-    if (!staged) resolve();
-    const uint64_t gbase = staged ? 0 : s_prefix;  // where block offset 0 goes
-    // one pair at block offset p: staged, or written below `limit` (histograms counted)
-    auto put = [&](uint64_t p, uint32_t key, uint32_t val) {
-        if (staged) {
-            s_pk[p] = key;
-            s_pv[p] = val;
-        } else if (gbase + p < limit) {
-            ckey[gbase + p] = key;
-            cval[gbase + p] = val;
-        }
-    };
-
-    uint64_t p_warp = __shfl_sync(0xffffffffu, local, 0);  // the warp's pairs start at its lane 0's item
-    const unsigned lt = (1u << lane) - 1u;
-    warp_units(units, [&](bool act, int src, uint32_t u, uint32_t f) {
-        const int bx0 = __shfl_sync(0xffffffffu, x0, src), bx1 = __shfl_sync(0xffffffffu, x1, src);
-        const int by0 = __shfl_sync(0xffffffffu, y0, src), by1 = __shfl_sync(0xffffffffu, y1, src);
-        const int bstx = __shfl_sync(0xffffffffu, stx, src), bstb = __shfl_sync(0xffffffffu, stb, src);
-        const uint32_t bi = __shfl_sync(0xffffffffu, item, src);
-        const int sy = by0 / kSuper + (int)u;
-        const bool again = act && f >= kStashUnits;  // beyond the stash: evaluated again
-        TightRows bt{};
-        if (__any_sync(0xffffffffu, again)) bt = shfl_rows(t, src);
-        Runs4 rr{};
-        uint32_t n = 0;
-        if (act) {
-            if (again) {
-                uint32_t fine2 = 0;
-                rr = row_runs(bt, sy, bx0, bx1, by0, by1, &fine2);
-                n = (uint32_t)runs_union(rr, [](int, int) {});
-            } else {
-                rr = unpack_runs(stash[f]);
-                n = stash_n[f];
-                if (n == 255) n = (uint32_t)runs_union(rr, [](int, int) {});
-            }
-        }
-        uint32_t incl = n;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t v = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += v;
-        }
-        uint64_t p = p_warp + (incl - n);
-        p_warp += __shfl_sync(0xffffffffu, incl, 31);
-        const uint32_t krow = (uint32_t)bstb + (uint32_t)sy * (uint32_t)bstx;  // the row's supertile 0
-        const bool wide = n > kWideRow;
-        if (act && !wide)
-            runs_union(rr, [&](int lo, int hi) {
-                const uint32_t len = (uint32_t)(hi - lo + 1);
-                for (uint32_t j = 0; j < len; ++j)
-                    put(p + j, (krow + (uint32_t)lo + j) | (pack ? runs_mask(rr, lo + (int)j) << 16 : 0u), bi);
-                if (!staged && gbase + p < limit)
-                    row_hist(krow + (uint32_t)lo, (uint32_t)min((uint64_t)len, limit - (gbase + p)), passes, s_d0,
-                             s_h);
-                p += len;
-            });
-        unsigned wides = __ballot_sync(0xffffffffu, act && wide);
-        while (wides) {  // a wide row: the whole warp, supertile column lo + j on lane j
-            const int w = __ffs(wides) - 1;
-            wides &= wides - 1;
-            Runs4 wr;
-#pragma unroll
-            for (int q = 0; q < kSuper; ++q) {
-                wr.f[q] = __shfl_sync(0xffffffffu, rr.f[q], w);
-                wr.l[q] = __shfl_sync(0xffffffffu, rr.l[q], w);
-            }
-            uint64_t wp = __shfl_sync(0xffffffffu, p, w);
-            const uint32_t wk = __shfl_sync(0xffffffffu, krow, w), wi = __shfl_sync(0xffffffffu, bi, w);
-            int lo = 0x7fffffff, hi = -1;
-#pragma unroll
-            for (int q = 0; q < kSuper; ++q)
-                if (wr.f[q] <= wr.l[q]) {
-                    lo = min(lo, wr.f[q] / kSuper);
-                    hi = max(hi, wr.l[q] / kSuper);
+    for (;;) {
+        if (threadIdx.x == 0) s_tile = atomicAdd(&tickets[kMaxPasses], 1u);
+        __syncthreads();  // (also: the last tile's pairs have left shared memory)
+        const uint32_t tile = s_tile;
+        const int64_t base = (int64_t)tile * kDupTile;
+        if (base >= n_items) break;
+        {
+            const int64_t k = base + threadIdx.x;
+            const uint32_t item = k < n_items ? perm[k] : 0xffffffffu;
+            uint32_t units = 0;
+            if (item < (uint32_t)n_items) {  // always, unless a look-back gave up (timeout bit set)
+                const int v = (int)(item / (uint32_t)sv.n_per_view);
+                // all of the item's loads at once
+                const float2 m = mean2d[item];
+                const int r = radius[item];
+                const float ca = sv.conic[3 * (size_t)item], cb = sv.conic[3 * (size_t)item + 1],
+                            cc = sv.conic[3 * (size_t)item + 2];
+                const float pmin = sv.power_min[item - (uint32_t)v * (uint32_t)sv.n_per_view];
+                int x0, x1, y0, y1;
+                if (tile_rect(m.x, m.y, r, sv.views[v].W, sv.views[v].H, x0, x1, y0, y1)) {
+                    const TightRows t = tight_rows(m.x, m.y, ca, cb, cc, pmin);
+                    // rows beyond the ellipse's height hold nothing: leave them out (one pixel of slack)
+                    if (t.mode == 2 && fabsf(t.my) + t.ymax < 1048576.f) {
+                        y0 = max(y0, (int)floorf((t.my - t.ymax - 17.f) * 0.0625f));
+                        y1 = min(y1, (int)floorf((t.my + t.ymax + 1.f) * 0.0625f));
+                    }
+                    if (t.mode != 1 && y0 <= y1) units = (uint32_t)(y1 / kSuper - y0 / kSuper + 1);
+                    s_rect[threadIdx.x] =
+                        make_uint2((uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16));
+                    s_ta[threadIdx.x] = make_float4(t.mx, t.my, t.nB, t.det);
+                    s_tb[threadIdx.x] = make_float4(t.Atau, t.rA, t.ymax, t.dyr);
+                    s_item[threadIdx.x] = item;
+                    s_mode[threadIdx.x] = (uint8_t)t.mode;
+                    s_row[threadIdx.x] =
+                        (uint32_t)sv.st_begin[v] + (uint32_t)(max(y0, 0) / kSuper) * (uint32_t)sv.st_x[v];
+                    s_stx[threadIdx.x] = (uint32_t)sv.st_x[v];
                 }
-            for (int sx0 = lo; sx0 <= hi; sx0 += 32) {
-                const int sx = sx0 + lane;
-                const uint32_t m = sx <= hi ? runs_mask(wr, sx) : 0u;
-                const unsigned nz = __ballot_sync(0xffffffffu, m != 0u);
-                const uint64_t q = wp + (uint64_t)__popc(nz & lt);
-                if (m != 0u) {
-                    put(q, (wk + (uint32_t)sx) | (pack ? m << 16 : 0u), wi);
-                    if (!staged && gbase + q < limit) key_hist(wk + (uint32_t)sx, passes, s_d0, s_h);
-                }
-                wp += (uint64_t)__popc(nz);
             }
+            uint32_t all;
+            s_u[threadIdx.x] = block_excl_scan<uint32_t, kThreads>(units, all, s_warp);
+            if (threadIdx.x == 0) s_u[kDupTile] = all;
+            __syncthreads();
         }
-    });
-    if (staged) {
-        resolve();  // (its barrier also orders the staging before the copy)
-        const uint64_t g0 = s_prefix;
-        for (uint32_t i = threadIdx.x; i < (uint32_t)tile_sum; i += kThreads) {
-            if (g0 + i >= limit) break;
-            const uint32_t key = s_pk[i];
-            ckey[g0 + i] = key;
-            cval[g0 + i] = s_pv[i];
-            key_hist(pack ? key & 0xFFFFu : key, passes, s_d0, s_h);
+        const uint32_t n_units = s_u[kDupTile];
+        const uint32_t batches = max(1u, (n_units + kStash - 1) / kStash);
+        uint64_t tile_sum = 0, at = 0;  // `at`: where the batch's pairs go
+        for (uint32_t it = 0; it < (batches == 1 ? 1u : 2 * batches); ++it) {
+            const bool counting = it < batches, writing = batches == 1 || !counting;
+            const uint32_t b0 = (counting ? it : it - batches) * kStash, nu = min(kStash, n_units - b0);
+            const uint32_t per = (nu + kThreads - 1) / kThreads;
+            const uint32_t f0 = min(threadIdx.x * per, nu), f1 = min(f0 + per, nu);
+            uint32_t sum = 0;
+            int i = 0;  // the last item whose first unit is at or before b0 + f0
+#pragma unroll
+            for (int d = kDupTile / 2; d > 0; d >>= 1)
+                if (s_u[i + d] <= b0 + f0) i += d;
+            for (uint32_t r = 0; r < per; ++r) {
+                const uint32_t f = f0 + r;
+                if (f < f1)
+                    while (s_u[i + 1] <= b0 + f) ++i;  // (ends: s_u[kDupTile] is above every unit)
+                __syncwarp();                          // the lanes step apart: together again for the row's work
+                if (f < f1) {
+                    const uint2 q = s_rect[i];
+                    const float4 ta = s_ta[i], tb = s_tb[i];
+                    const TightRows t{(int)s_mode[i], ta.x, ta.y, ta.z, ta.w, tb.x, tb.y, tb.z, tb.w};
+                    const int y0 = (int)(q.y & 0xFFFFu), u = (int)(b0 + f - s_u[i]), sy = y0 / kSuper + u;
+                    uint32_t inst = 0;
+                    const Runs4 rr =
+                        row_runs(t, sy, (int)(q.x & 0xFFFFu), (int)(q.x >> 16), y0, (int)(q.y >> 16), &inst);
+                    // the runs of a convex shape join up; any gap between them takes the general union
+                    // (selects, no branches: the lanes' patterns of empty rows differ)
+                    int lo = 0x3fffffff, hi = -1;
+                    bool gap = false;
+#pragma unroll
+                    for (int k = 0; k < kSuper; ++k) {
+                        const bool some = rr.f[k] <= rr.l[k];
+                        const int a = some ? rr.f[k] / kSuper : 0x3fffffff, b = some ? rr.l[k] / kSuper : -1;
+                        gap |= some & (hi >= 0) & ((a > hi + 1) | (b < lo - 1));
+                        lo = min(lo, a);
+                        hi = max(hi, b);
+                    }
+                    uint32_t n = (uint32_t)max(hi - lo + 1, 0), key = s_row[i] + (uint32_t)u * s_stx[i];
+                    uint4 runs;
+                    const bool general = gap || n > kMaxSpan;
+                    if (general) {
+                        n = (uint32_t)runs_union(rr, [](int, int) {});
+                        runs = pack_runs(rr);
+                    } else {
+                        int fr[kSuper], lr[kSuper];  // first column, 3 - last column; an empty run as 0, 4
+#pragma unroll
+                        for (int k = 0; k < kSuper; ++k) {
+                            const bool some = rr.f[k] <= rr.l[k];
+                            fr[k] = some ? rr.f[k] - lo * kSuper : 0;
+                            lr[k] = some ? 3 + lo * kSuper - rr.l[k] : 4;
+                        }
+                        runs = make_uint4(pack16(fr[0], fr[1]), pack16(fr[2], fr[3]), pack16(lr[0], lr[1]),
+                                          pack16(lr[2], lr[3]));
+                        key += (uint32_t)lo;
+                    }
+                    s_runs[f] = runs;
+                    s_key[f] = key;
+                    s_who[f] = (uint16_t)((uint32_t)i | (general ? 0x8000u : 0u));
+                    s_p[f] = n;
+                    sum += n;
+                    if (counting) fine += inst;
+                }
+            }
+            uint32_t batch_sum;
+            uint32_t p0 = block_excl_scan<uint32_t, kThreads>(sum, batch_sum, s_warp);
+            for (uint32_t f = f0; f < f1; ++f) {
+                const uint32_t n = s_p[f];
+                s_p[f] = p0;
+                p0 += n;
+            }
+            for (uint32_t f = nu + threadIdx.x; f < 1024; f += kThreads) s_p[f] = 0xffffffffu;
+            if (counting) tile_sum += batch_sum;
+            __syncthreads();
+            const bool staged = batches == 1 && batch_sum <= kStagePairs;
+            if (it == batches - 1 && threadIdx.x == 0) st_status(status + tile, tile == 0 ? 2u : 1u, tile_sum);
+            // the pairs are made into shared memory before the look-back, while the tiles before
+            // this one publish their sums; a tile of more pairs looks back first
+#pragma unroll 1
+            for (int ph = 0; ph < 2; ++ph) {
+                if (writing && (ph == 0) == staged) {
+                    const uint32_t room =
+                        staged ? batch_sum : at < limit ? (uint32_t)min((uint64_t)batch_sum, limit - at) : 0u;
+                    for (uint32_t p = threadIdx.x; p < room; p += kThreads) {
+                        uint32_t f = 0;  // the last unit whose first pair is at or before p
+#pragma unroll
+                        for (uint32_t d = 512; d > 0; d >>= 1)
+                            if (s_p[f + d] <= p) f += d;
+                        const uint4 runs = s_runs[f];
+                        const uint32_t who = s_who[f];
+                        uint32_t j = p - s_p[f], key = s_key[f], mask = 0;  // mask: row k's 4 columns in byte k
+                        if (who >> 15) {
+                            const Runs4 rr = unpack_runs(runs);
+                            int left = (int)j;
+                            runs_union(rr, [&](int lo, int hi) {
+                                if (left >= 0 && left <= hi - lo) j = (uint32_t)(lo + left);
+                                left -= hi - lo + 1;
+                            });
+                            const uint32_t m = runs_mask(rr, (int)j);
+                            mask = (m & 0xFu) | (m & 0xF0u) << 4 | (m & 0xF00u) << 8 | (m & 0xF000u) << 12;
+                        } else if (pack) {
+                            const uint32_t up = kSuper * j * 0x10001u, dn = ((0u - kSuper * j) & 0xFFFFu) * 0x10001u;
+                            mask = nibbles(0x080C0E0Fu, runs.x, runs.y, dn) & nibbles(0x0103070Fu, runs.z, runs.w, up);
+                        }
+                        key += j;
+                        if (pack) key = __byte_perm(key, mask | mask >> 4, 0x6410);  // the four nibbles above the id
+                        if (staged) {
+                            s_pk[p] = key;
+                            s_pv[p] = (uint8_t)who;
+                        } else {
+                            ckey[at + p] = key;
+                            cval[at + p] = s_item[who & 0xFFu];
+                            count(key);
+                        }
+                    }
+                }
+                if (ph == 0 && it == batches - 1) {
+                    if (warp == 0) {
+                        uint64_t prefix = 0;
+                        if (tile > 0) {
+                            prefix = lookback_warp(status, tile, 1u, err);
+                            if (lane == 0) st_status(status + tile, 2u, prefix + tile_sum);
+                        }
+                        if (lane == 0) {
+                            s_prefix = prefix;
+                            if (base + kDupTile >= n_items) *total = prefix + tile_sum;  // the last tile: the total
+                        }
+                    }
+                    __syncthreads();
+                    at = s_prefix;
+                    if (coarse_tile > 0) {  // the sort takes at most `limit` pairs: its tiles start below it
+                        const uint64_t hi = min(at + tile_sum, limit);
+                        for (uint64_t ct = (at + coarse_tile - 1) / coarse_tile; ct * coarse_tile < hi; ++ct)
+                            radix_status[ct * 256 + threadIdx.x] = 0ull;
+                    }
+                }
+            }
+            if (staged) {
+                const uint32_t room = at < limit ? (uint32_t)min((uint64_t)batch_sum, limit - at) : 0u;
+                for (uint32_t p = threadIdx.x; p < room; p += kThreads) {
+                    const uint32_t key = s_pk[p];
+                    ckey[at + p] = key;
+                    cval[at + p] = s_item[s_pv[p]];
+                    count(key);
+                }
+            }
+            if (writing) at += batch_sum;
+            if (batches > 1) __syncthreads();  // the batch has left shared memory
         }
     }
-    __syncthreads();
-    {
-        int tot;
-        const int v = s_d0[threadIdx.x];
-        const int d0 = block_excl_scan<int, kThreads>(v, tot, s_warp_i) + v;  // count of digit-0 value threadIdx.x
-        if (d0) atomicAdd(&hist[threadIdx.x], (uint32_t)d0);
-    }
-    for (int i = threadIdx.x; i < (passes - 1) * 256; i += kThreads)
-        if (s_h[i]) atomicAdd(&hist[256 + i], s_h[i]);
+    // every thread left the loop through its barrier: the histograms are complete
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) fine += __shfl_xor_sync(0xffffffffu, fine, o);
+    if (lane == 0 && fine) atomicAdd(fine_total, fine);
+    for (int i = threadIdx.x; i < passes * 256; i += kThreads)
+        if (s_h[i]) atomicAdd(&hist[i], s_h[i]);
 }
 
 // The same for full rectangles.  An item's supertiles are then a rectangle too,
@@ -1567,7 +1533,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
             return cuda_status(e, "gs_bin_sort: device");
     }
     if (tight)
-        k_dup_coarse<<<(int)cdiv(n, kDupTile), kThreads, 0, s>>>(
+        k_dup_coarse<<<(int)std::min<int64_t>(cdiv(n, kDupTile), kDupBlocks * (int64_t)dev_sms), kThreads, 0, s>>>(
             n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
             hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, err);
     else

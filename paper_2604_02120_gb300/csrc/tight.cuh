@@ -77,28 +77,24 @@ __device__ __forceinline__ float tight_end(const TightRows& t, float y, float si
 }
 
 // The kept tiles [first, last] of row ty within [x0, x1] (first > last: none).
+// Selects in place of early returns: neighbouring lanes hold different splats.
 __device__ __forceinline__ void tight_row(const TightRows& t, int ty, int x0, int x1, int& first, int& last) {
-    first = x0;
-    last = x1;
-    if (t.mode == 0) return;
-    last = x0 - 1;
-    if (t.mode == 1) return;
     const float lo = fmaxf(__fsub_rn(t.my, __fadd_rn((float)(16 * ty), 15.5f)), -t.ymax);
     const float hi = fminf(__fsub_rn(t.my, __fadd_rn((float)(16 * ty), 0.5f)), t.ymax);
-    if (!(lo <= hi)) return;
-    float xr, xl;
-    if (t.mode == 2) {
-        xr = tight_end(t, fminf(fmaxf(t.dyr, lo), hi), 1.f);
-        xl = tight_end(t, fminf(fmaxf(-t.dyr, lo), hi), -1.f);
-    } else {
+    float xr = tight_end(t, fminf(fmaxf(t.dyr, lo), hi), 1.f);
+    float xl = tight_end(t, fminf(fmaxf(-t.dyr, lo), hi), -1.f);
+    if (t.mode == 3) {
         xr = fmaxf(tight_end(t, lo, 1.f), tight_end(t, hi, 1.f));
         xl = fminf(tight_end(t, lo, -1.f), tight_end(t, hi, -1.f));
     }
     // tile tx has offsets [mx - 16 tx - 15.5, mx - 16 tx - 0.5]
     const float flo = __fmul_rn(__fsub_rn(__fsub_rn(t.mx, 15.5f), xr), 0.0625f);
     const float fhi = __fmul_rn(__fsub_rn(__fsub_rn(t.mx, 0.5f), xl), 0.0625f);
-    first = (int)ceilf(fminf(fmaxf(flo, (float)x0), (float)(x1 + 1)));
-    last = (int)floorf(fminf(fmaxf(fhi, (float)(x0 - 1)), (float)x1));
+    const int a = (int)ceilf(fminf(fmaxf(flo, (float)x0), (float)(x1 + 1)));
+    const int b = (int)floorf(fminf(fmaxf(fhi, (float)(x0 - 1)), (float)x1));
+    const bool strip = t.mode >= 2 && lo <= hi;
+    first = strip ? a : x0;
+    last = strip ? b : t.mode == 0 ? x1 : x0 - 1;
 }
 
 }  // namespace gs
