@@ -41,15 +41,19 @@ namespace gs {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr uint32_t kSmallPass = 1u << 20;  // passes up to this size use 1024-item tiles, larger ones 4096
+constexpr uint32_t kSmallPass = 1u << 20;
+// Items per thread of a radix pass: tiles of 1024 up to 2^18 items, so that a
+// small pass reaches all SMs; of 2048 up to 9 x 2^17, one wave of 4 blocks per
+// SM (a pass of 1M: 13.5 us, in tiles of 1024 17.4); of 4096 beyond, which
+// halves the look-back.
 constexpr int kDupTile = kThreads;          // items per tile of the opacity-aware duplication
 constexpr int kMaxPasses = 8;               // 4 depth passes + up to 4 tile-id passes
 constexpr uint64_t kLookbackLimitNs = 2000000000ull;
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
-inline int pass_items(uint64_t n) { return n <= kSmallPass ? 4 : 16; }
-// Most radix tiles a pass over at most m items can have.
+inline int pass_items(uint64_t n) { return n <= 1u << 18 ? 4 : n <= 9u << 17 ? 8 : 16; }
+// An upper bound of the radix tiles of a pass over at most m items.
 inline int64_t radix_tiles_max(int64_t m) {
     return std::max(cdiv(std::min<int64_t>(m, kSmallPass), kThreads * 4), cdiv(m, kThreads * pass_items(m)));
 }
@@ -107,13 +111,13 @@ __device__ __forceinline__ unsigned long long ld_status(const unsigned long long
     return w;
 }
 
-// Sum of the counts of tiles [0, tile) for one digit, walking back from
-// tile - 1 until an inclusive prefix is found.  Eight predecessors are read
-// per round trip; the ready ones nearest to this tile are consumed, up to the
-// first inclusive prefix.
+// Sum of the counts of groups [0, g) for one digit, walking back from g - 1
+// until an inclusive prefix is found.  W predecessors are read per round trip;
+// the ready ones nearest to this group are consumed, up to the first inclusive
+// prefix.
 __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* status, int64_t tile, int stride,
                                                     int d, uint32_t tag_agg, unsigned* err) {
-    constexpr int W = 8;
+    constexpr int W = 4;
     uint64_t prefix = 0, t0 = 0;
     int64_t j = tile - 1;
     while (j >= 0) {
@@ -139,6 +143,7 @@ __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* st
         if (done) break;
         j -= used;
         if (blocked) {
+            __nanosleep(100);
             const uint64_t now = globaltimer_ns();
             if (t0 == 0) {
                 t0 = now;
@@ -149,6 +154,49 @@ __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* st
         }
     }
     return prefix;
+}
+
+// The radix passes look back over two levels.  A tile publishes its digit
+// counts once (rows: 256 words of 32 bits, tag in bits [27, 32)) and adds up
+// the rows before it in its group of kGroup tiles; the group's last tile
+// publishes the group's counts and, after its own look-back, their inclusive
+// prefix (64-bit words as above), and everybody looks back over groups.  With
+// one level a tile walked over 150 rows (600 tiles are in flight, and rows turn
+// inclusive only as walks end) and the reading, not the waiting, took longer
+// than the tile's own work: windows of 16 or 32 rows were slower than 8.  Per
+// pass, 200k / 1M / 3M / 14M items: 10.9 / 23.4 / 32 / 120 us with one level,
+// 8.9 / 17.7 / 31 / 115 with two (16 tiles in a group, windows of 4), 25.5 and
+// 77 for the large ones with the ranking below and groups of 8.
+constexpr int kGroup = 8;
+constexpr int kRowTagBit = 27;
+__device__ __forceinline__ uint32_t group_sum(const uint32_t* rows, int64_t tile, int d, uint32_t tag, unsigned* err) {
+    const int m = (int)(tile % kGroup);
+    const uint32_t* p = rows + (size_t)(tile - m) * 256 + d;
+    uint64_t t0 = 0;
+    for (;;) {
+        uint32_t w[kGroup - 1];
+#pragma unroll
+        for (int q = 0; q < kGroup - 1; ++q) {
+            w[q] = tag << kRowTagBit;
+            if (q < m) asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(w[q]) : "l"(p + q * 256) : "memory");
+        }
+        uint32_t sum = 0;
+        bool ready = true;
+#pragma unroll
+        for (int q = 0; q < kGroup - 1; ++q) {
+            ready = ready && (w[q] >> kRowTagBit) == tag;
+            sum += w[q] & ((1u << kRowTagBit) - 1);
+        }
+        if (ready) return sum;
+        __nanosleep(100);
+        const uint64_t now = globaltimer_ns();
+        if (t0 == 0) {
+            t0 = now;
+        } else if (now - t0 > kLookbackLimitNs) {
+            atomicOr(err, kErrTimeout);
+            return 0;
+        }
+    }
 }
 
 // The same for a single count per tile, by one warp over windows of 32
@@ -187,25 +235,6 @@ __device__ __forceinline__ uint64_t lookback_warp(const unsigned long long* stat
     return prefix;
 }
 
-// The lanes of the warp whose digit equals this lane's, among the valid lanes
-// (an invalid lane gets only itself).  FULL: one ballot per bit of the 8-bit
-// digit, a cost that does not grow with the number of distinct digits in the
-// warp (random digits: up to 32); otherwise __match_any_sync, the cheaper when
-// the digit has at most 4 significant bits (the last pass over a short key).
-template <bool FULL>
-__device__ __forceinline__ unsigned digit_peers(uint32_t d, bool valid) {
-    const unsigned lane_bit = 1u << (threadIdx.x & 31);
-    if constexpr (!FULL) return __match_any_sync(0xffffffffu, valid ? d : 0x100u + (threadIdx.x & 31));
-    unsigned m = __ballot_sync(0xffffffffu, valid);
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const bool bit = (d >> b) & 1u;
-        const unsigned bal = __ballot_sync(0xffffffffu, bit);
-        m &= bit ? bal : ~bal;
-    }
-    return valid ? m : lane_bit;
-}
-
 // s_h[bin] += 1 for every active lane: one atomic when the lanes agree on the
 // bin (the high digits of nearby keys usually do, and same-address shared
 // atomics serialise), else one per lane.
@@ -233,8 +262,12 @@ __device__ __forceinline__ uint32_t pass_count(uint32_t n_host, const uint64_t* 
 // of TILE items from the ticket; warp w owns the contiguous items
 // [w * 32 ITEMS, (w + 1) * 32 ITEMS) walked in rounds of 32, so lane order is
 // input order, and each item's rank among equal digits comes from the lanes
-// with the same digit (digit_peers; FULL: ballots, for digits of more than
-// 4 significant bits).  The ranking runs once: it keeps each item's rank among
+// with the same digit: FULL, for digits of more than 4 significant bits, ors the
+// lane's bit into a word per warp and digit in shared memory and reads it back
+// (14M items 117 -> 77 us against eight ballots, whose bit tests filled 69% of
+// the ALU); else __match_any_sync, cheaper while few digits occur (the last
+// pass over a short key: 70 us, with the shared words 86, as lanes then collide
+// on them).  The ranking runs once: it keeps each item's rank among
 // its warp's items of the same digit, so placing an item needs only its warp's
 // start of the digit.  Items are placed in shared memory in digit order, then
 // written so that consecutive threads write consecutive addresses of each
@@ -252,7 +285,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
     __shared__ uint32_t s_goff[256];               // global start of each digit's run
     __shared__ uint32_t s_warp[kThreads / 32 + 1];
     __shared__ uint32_t s_tile;
-    __shared__ uint32_t s_key[TILE], s_val[TILE];
+    __shared__ uint32_t s_buf[2 * TILE];
+    uint32_t *s_key = s_buf, *s_val = s_buf + TILE;
+    uint32_t* s_peers = s_buf;  // while ranking: per warp and digit, the lanes of the round that have it
+    static_assert(2 * TILE >= kThreads / 32 * 256);
     const uint32_t n = pass_count(n_host, n_dev);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     // persistent: the block takes tiles until the pass is done (a tile's
@@ -260,7 +296,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
     // already processing)
     for (;;) {
         if (threadIdx.x == 0) s_tile = atomicAdd(&tickets[pass_id], 1u);
-        for (int i = threadIdx.x; i < (kThreads / 32) * 256; i += kThreads) (&s_w[0][0])[i] = 0;
+        for (int i = threadIdx.x; i < (kThreads / 32) * 256; i += kThreads) {
+            (&s_w[0][0])[i] = 0;
+            if constexpr (FULL) s_peers[i] = 0;
+        }
         __syncthreads();
         const uint32_t tile = s_tile;
         const int64_t bbase = (int64_t)tile * TILE;
@@ -282,10 +321,21 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
         for (int r = 0; r < ITEMS; ++r) {
             const bool valid = wbase + r * 32 + lane < cnt;
             const uint32_t d = (k[r] >> shift) & 0xFFu;
-            const unsigned peers = digit_peers<FULL>(d, valid);
-            const uint32_t before = valid ? s_w[warp][d] : 0u;
+            uint32_t* slot = s_peers + warp * 256 + d;
+            uint32_t peers;
+            if constexpr (FULL) {
+                if (valid) atomicOr(slot, 1u << lane);
+                __syncwarp();
+                peers = *slot;
+            } else {
+                peers = __match_any_sync(0xffffffffu, valid ? d : 0x100u + lane);
+            }
+            const uint32_t before = s_w[warp][d];
             __syncwarp();
-            if (valid && (peers & lt) == 0) s_w[warp][d] = before + __popc(peers);
+            if (valid && (peers & lt) == 0) {
+                s_w[warp][d] = before + __popc(peers);
+                if constexpr (FULL) *slot = 0;
+            }
             __syncwarp();
             const uint32_t rk = before + __popc(peers & lt);
             if (r & 1)
@@ -299,16 +349,24 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
             uint32_t c = 0;
 #pragma unroll
             for (int w = 0; w < kThreads / 32; ++w) c += s_w[w][d];
-            unsigned long long* mine = status + (size_t)tile * 256 + d;
+            // rows of 32 bits, then the full groups' rows: within the 256 64-bit words per tile
+            uint32_t* rows = reinterpret_cast<uint32_t*>(status);
+            unsigned long long* groups = status + ((size_t)n + TILE - 1) / TILE * 128;
             const uint32_t tag_agg = 2u * pass_id + 1u;
-            st_status(mine, tile == 0 ? tag_agg + 1 : tag_agg, c);  // publish first, successors may be waiting
+            asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(rows + (size_t)tile * 256 + d),
+                         "r"(tag_agg << kRowTagBit | c)
+                         : "memory");  // publish first, successors may be waiting
             uint32_t total;
             const uint32_t db = block_excl_scan<uint32_t, kThreads>(c, total, s_warp);
             const uint32_t gstart = block_excl_scan<uint32_t, kThreads>(hist[d], total, s_warp);
             uint32_t prefix = 0;
-            if (tile > 0) {
-                prefix = (uint32_t)lookback_serial(status, tile, 256, d, tag_agg, err);
-                st_status(mine, tag_agg + 1, prefix + c);
+            const int64_t g = tile / kGroup;
+            const bool closes = tile % kGroup == kGroup - 1;
+            if (tile % kGroup) prefix = group_sum(rows, tile, d, tag_agg, err);
+            if (closes) st_status(groups + (size_t)g * 256 + d, g == 0 ? tag_agg + 1 : tag_agg, prefix + c);
+            if (g > 0) {
+                prefix += (uint32_t)lookback_serial(groups, g, 256, d, tag_agg, err);
+                if (closes) st_status(groups + (size_t)g * 256 + d, tag_agg + 1, prefix + c);
             }
             s_dbase[d] = db;
             s_goff[d] = gstart + prefix;
@@ -375,10 +433,10 @@ cudaError_t radix_sort(uint32_t* k[2], uint32_t* v[2], uint32_t n_host, const ui
     const int nblk = (int)std::min<int64_t>(cdiv(n_host, (int64_t)kThreads * items), 4 * (int64_t)sms);
     for (int p = 0, shift = 0; shift < bits; ++p, shift += 8) {
         const int id = first_pass + p;
-        // ballots unless the digit has at most 4 significant bits (match_any is cheaper then)
-        const bool full = bits - shift > 4;
-        auto kern = items == 4 ? (full ? k_onesweep<4, true> : k_onesweep<4, false>)
-                               : (full ? k_onesweep<16, true> : k_onesweep<16, false>);
+        const bool full = bits - shift > 4;  // k_onesweep: how equal digits are found
+        auto kern = items == 4   ? (full ? k_onesweep<4, true> : k_onesweep<4, false>)
+                    : items == 8 ? (full ? k_onesweep<8, true> : k_onesweep<8, false>)
+                                 : (full ? k_onesweep<16, true> : k_onesweep<16, false>);
         kern<<<nblk, kThreads, 0, s>>>(k[cur], v[cur], n_host, n_dev, shift, id, ps.hist + 256 * id, ps.tickets,
                                        ps.status, k[cur ^ 1], v[cur ^ 1], ps.err);
         count_launches();
@@ -857,8 +915,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
                                                           uint32_t* __restrict__ hist, uint64_t* __restrict__ total,
                                                           unsigned long long* __restrict__ fine_total,
                                                           unsigned long long* __restrict__ radix_status,
-                                                          uint32_t coarse_tile, uint32_t* __restrict__ st_zero, int st_n,
-                                                          unsigned* err) {
+                                                          uint32_t coarse_tile, uint32_t* __restrict__ st_zero,
+                                                          int st_n, unsigned* err) {
     __shared__ uint64_t s_warp[kThreads / 32 + 1];
     __shared__ uint64_t s_prefix;
     __shared__ unsigned long long s_fine;
@@ -1064,7 +1122,8 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
     const uint64_t warp_id = ((uint64_t)blockIdx.x * kThreads + threadIdx.x) >> 5;
     const uint64_t warps = ((uint64_t)gridDim.x * kThreads) >> 5;
     const uint64_t want = (Ic + warps - 1) / warps;
-    const uint64_t seg = min((uint64_t)kPairSegMax, max((want + kPairBatch - 1) / kPairBatch, (uint64_t)1) * kPairBatch);
+    const uint64_t seg =
+        min((uint64_t)kPairSegMax, max((want + kPairBatch - 1) / kPairBatch, (uint64_t)1) * kPairBatch);
     constexpr int U = kPairBatch / 32;
     for (uint64_t s0 = warp_id * seg; s0 < Ic; s0 += warps * seg) {
         const uint64_t s1 = min(s0 + seg, (uint64_t)Ic);
@@ -1079,7 +1138,8 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
             acc = 0;
         };
         const uint32_t kmask = pack ? 0xFFFFu : 0xFFFFFFFFu;
-        uint32_t last = st_beg != nullptr && s0 > 0 ? ckey[s0 - 1] & kmask : 0xffffffffu;  // the pair before the group's
+        // the supertile of the pair before the group's
+        uint32_t last = st_beg != nullptr && s0 > 0 ? ckey[s0 - 1] & kmask : 0xffffffffu;
         uint32_t kn[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
