@@ -10,9 +10,14 @@
 //   dM += r0^T du0 + r1^T du1 and dr = du M^T for the rows r0, r1 of J R,
 // and J's entries are functions of the camera-space point p = R mean + t.
 // A block's SH coefficients and their gradients go through shared memory
-// (coalesced loads and stores, one odd-stride row per Gaussian so the
-// threads' row reads are free of bank conflicts), which keeps the registers,
-// and with them the resident warps, at what the latency of HBM needs.
+// (coalesced copies and stores, one odd-stride row per Gaussian so the
+// threads' row reads are free of bank conflicts).  The kernel is bound by HBM
+// latency, by how many bytes the resident blocks have in flight: the
+// coefficients are copied by cp.async, which holds no registers meanwhile, and
+// with one view (ONE) the gradients overwrite them in place, which halves the
+// shared memory and leaves out clearing and re-reading the sums.  One view, 1M
+// Gaussians, degree 3 (453 MB): 103 -> 83 us, 5.4 TB/s; with 4 / 6 / 8 blocks per
+// SM instead of 5 85 / 89 / 101 us (6 and 8 spill).
 #include "internal.h"
 #include "sh.cuh"
 
@@ -42,12 +47,18 @@ __device__ __forceinline__ ViewIn load_view(size_t item, const int* radius_all, 
     return in;
 }
 
+// 4 bytes from global to shared memory without a register in between.
+__device__ __forceinline__ void copy_word_async(float* dst, const float* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
 // Floats per Gaussian row of the shared coefficient arrays (odd).
 template <int SH_DEGREE>
 __host__ __device__ constexpr int sh_row() { return (3 * (SH_DEGREE + 1) * (SH_DEGREE + 1)) | 1; }
 
-template <int SH_DEGREE>
-__global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const float* __restrict__ means,
+template <int SH_DEGREE, bool ONE>
+__global__ void __launch_bounds__(kProjBwdThreads, ONE ? 5 : 4) k_project_bwd(int n, const float* __restrict__ means,
                                                                  const float* __restrict__ scales,
                                                                  const float* __restrict__ quats,
                                                                  const float* __restrict__ sh,
@@ -59,9 +70,10 @@ __global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const
                                                                  float* __restrict__ dmeans, float* __restrict__ dscales,
                                                                  float* __restrict__ dquats, float* __restrict__ dsh) {
     constexpr int K = (SH_DEGREE + 1) * (SH_DEGREE + 1), KC = 3 * K, ROW = sh_row<SH_DEGREE>();
-    extern __shared__ float s_sh[];  // [kProjBwdThreads][ROW] coefficients, then as many gradients
+    // [kProjBwdThreads][ROW] coefficients, then as many gradients (ONE: in the coefficients' place)
+    extern __shared__ float s_sh[];
     float* s_cf = s_sh;
-    float* s_dcf = s_sh + kProjBwdThreads * ROW;
+    float* s_dcf = ONE ? s_sh : s_sh + kProjBwdThreads * ROW;
     const int g0 = blockIdx.x * kProjBwdThreads;
     const int nb = min(kProjBwdThreads, n - g0);
     // every global load before the first barrier, so that a block waits for HBM once
@@ -70,20 +82,15 @@ __global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const
     const float s[3] = {scales[3 * gc], scales[3 * gc + 1], scales[3 * gc + 2]};
     const float q0 = quats[4 * gc], q1 = quats[4 * gc + 1], q2 = quats[4 * gc + 2], q3 = quats[4 * gc + 3];
     const ViewIn first = load_view((size_t)gc, radius_all, dmean2d_all, dconic_all, drgb_all);
-    if (nb == kProjBwdThreads) {  // a full block: a fixed trip count, many loads in flight
+    const float* src = sh + (size_t)g0 * KC;
 #pragma unroll 12
-        for (int j = 0; j < KC; ++j) {
-            const int i = threadIdx.x + j * kProjBwdThreads, r = i / KC, q = i - r * KC;
-            s_cf[r * ROW + q] = __ldg(sh + (size_t)g0 * KC + i);
-            s_dcf[r * ROW + q] = 0.f;
-        }
-    } else {
-        for (int i = threadIdx.x; i < nb * KC; i += kProjBwdThreads) {
-            const int r = i / KC, q = i - r * KC;
-            s_cf[r * ROW + q] = __ldg(sh + (size_t)g0 * KC + i);
-            s_dcf[r * ROW + q] = 0.f;
-        }
+    for (int j = 0; j < KC; ++j) {
+        const int i = threadIdx.x + j * kProjBwdThreads, r = i / KC, q = i - r * KC;
+        if (i < nb * KC) copy_word_async(s_cf + r * ROW + q, src + i);
     }
+    if constexpr (!ONE)
+        for (int i = threadIdx.x; i < kProjBwdThreads * ROW; i += kProjBwdThreads) s_dcf[i] = 0.f;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     if (g < n) {
     const float* cf = s_cf + threadIdx.x * ROW;
@@ -102,7 +109,10 @@ __global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const
 
     float dmw[3] = {0.f, 0.f, 0.f}, dM[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
 
-    for (int v = 0; v < views.num_views; ++v) {
+    if (ONE && first.radius <= 0)
+#pragma unroll
+        for (int i = 0; i < KC; ++i) dcf[i] = 0.f;
+    for (int v = 0; v < (ONE ? 1 : views.num_views); ++v) {
         const ViewIn in =
             v == 0 ? first : load_view((size_t)v * n + g, radius_all, dmean2d_all, dconic_all, drgb_all);
         if (in.radius <= 0) continue;
@@ -209,8 +219,8 @@ __global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const
             wk[k] = 0.f;
 #pragma unroll
             for (int ch = 0; ch < 3; ++ch) {
-                dcf[3 * k + ch] += Y[k] * dacc[ch];
                 wk[k] += cf[3 * k + ch] * dacc[ch];
+                dcf[3 * k + ch] = ONE ? Y[k] * dacc[ch] : dcf[3 * k + ch] + Y[k] * dacc[ch];
             }
         }
         if constexpr (SH_DEGREE > 0) {
@@ -257,24 +267,24 @@ __global__ void __launch_bounds__(kProjBwdThreads, 4) k_project_bwd(int n, const
     }
 }
 
-template <int D>
+template <int D, bool ONE>
 cudaError_t launch_deg(int n, cudaStream_t s, const float* means, const float* scales, const float* quats,
                        const float* sh, const CamViews& cams, const int* radius, const float* dmean2d,
                        const float* dconic, const float* drgb, float* dmeans, float* dscales, float* dquats,
                        float* dsh) {
-    const size_t smem = 2 * sizeof(float) * kProjBwdThreads * sh_row<D>();
+    const size_t smem = (ONE ? 1 : 2) * sizeof(float) * kProjBwdThreads * sh_row<D>();
     static std::mutex mu;  // the attribute is set once per process, as for the blend kernels
     static bool attr = false;
     {
         std::lock_guard<std::mutex> lock(mu);
         if (!attr) {
             const cudaError_t e =
-                cudaFuncSetAttribute(k_project_bwd<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                cudaFuncSetAttribute(k_project_bwd<D, ONE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
             attr = true;
         }
     }
-    k_project_bwd<D><<<(n + kProjBwdThreads - 1) / kProjBwdThreads, kProjBwdThreads, smem, s>>>(
+    k_project_bwd<D, ONE><<<(n + kProjBwdThreads - 1) / kProjBwdThreads, kProjBwdThreads, smem, s>>>(
         n, means, scales, quats, sh, cams, radius, reinterpret_cast<const float2*>(dmean2d), dconic, drgb, dmeans,
         dscales, dquats, dsh);
     return cudaSuccess;
@@ -287,15 +297,15 @@ cudaError_t launch_project_bwd(int n, const float* means, const float* scales, c
                                const float* dconic, const float* drgb, float* dmeans, float* dscales, float* dquats,
                                float* dsh, cudaStream_t s) {
     cudaError_t e;
+    auto run = [&](auto one, auto many) {
+        return (cams.num_views == 1 ? one : many)(n, s, means, scales, quats, sh, cams, radius, dmean2d, dconic, drgb,
+                                                  dmeans, dscales, dquats, dsh);
+    };
     switch (sh_degree) {
-        case 0: e = launch_deg<0>(n, s, means, scales, quats, sh, cams, radius, dmean2d, dconic, drgb, dmeans,
-                                  dscales, dquats, dsh); break;
-        case 1: e = launch_deg<1>(n, s, means, scales, quats, sh, cams, radius, dmean2d, dconic, drgb, dmeans,
-                                  dscales, dquats, dsh); break;
-        case 2: e = launch_deg<2>(n, s, means, scales, quats, sh, cams, radius, dmean2d, dconic, drgb, dmeans,
-                                  dscales, dquats, dsh); break;
-        default: e = launch_deg<3>(n, s, means, scales, quats, sh, cams, radius, dmean2d, dconic, drgb, dmeans,
-                                   dscales, dquats, dsh); break;
+        case 0: e = run(launch_deg<0, true>, launch_deg<0, false>); break;
+        case 1: e = run(launch_deg<1, true>, launch_deg<1, false>); break;
+        case 2: e = run(launch_deg<2, true>, launch_deg<2, false>); break;
+        default: e = run(launch_deg<3, true>, launch_deg<3, false>); break;
     }
     if (e != cudaSuccess) return e;
     count_launches();

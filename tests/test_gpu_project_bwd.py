@@ -214,3 +214,27 @@ def test_project_backward_sh1_without_lowpass():
     report("project_bwd_rel_sh1_no_lowpass", rel)
     for key, e in rel.items():
         assert e < 1e-4, f"{key}: relative error {e:.2e}"
+
+
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 1000])
+def test_one_view_equals_the_sum_over_views(degree, n):
+    """One camera has a kernel of its own; with a second camera that sees
+    nothing (radius 0) the general one adds nothing to the same values."""
+    rng = np.random.default_rng(10 * n + degree)
+    t = lambda *shape: torch.from_numpy(rng.normal(size=shape).astype(np.float32)).cuda()  # noqa: E731
+    cam = scenes.look_at_camera((0, 0, -3), (0, 0, 0), 200, 120)
+    means, quats, sh = t(n, 3) * 0.5, t(n, 4), t(n, (degree + 1) ** 2, 3)
+    scales = torch.exp(t(n, 3) * 0.5 - 3)
+    quats[0] = 0.0  # no rotation: the forward skips it
+    proj = gs.project(means, scales, quats, sh, degree, cam)
+    dm, dc, dr = t(n, 2), t(n, 3), t(n, 3)
+    one = gs.project_backward(means, scales, quats, sh, degree, cam, proj["radius"], dm, dc, dr)
+    twice = [torch.cat([a, torch.zeros_like(b)]) for a, b in ((proj["radius"], proj["radius"]), (dm, dm), (dc, dc),
+                                                              (dr, dr))]
+    two = gs.project_backward(means, scales, quats, sh, degree, [cam, cam], *twice)
+    assert gs.gs_sync_status() == gs.GS_OK
+    assert n == 1 or (proj["radius"] > 0).any()
+    for k in one:
+        assert torch.isfinite(one[k]).all()
+        np.testing.assert_array_equal(one[k].cpu().numpy(), two[k].cpu().numpy(), err_msg=k)
