@@ -134,12 +134,11 @@ def _ptr(t):
         return None
     if not t.is_contiguous():
         raise ValueError("tensor must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()  # ctypes converts by the declared c_void_p: no object per pointer
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return (stream if stream is not None else torch.cuda.current_stream()).cuda_stream
 
 
 def make_camera(cam) -> gs_camera:
@@ -567,8 +566,8 @@ def blend_backward(width, height, bs, proj, opacity, opts, fwd, dL_dimage, strea
     n = opacity.shape[0]
     # the four outputs accumulate by atomics: views of one buffer, zeroed by one fill
     buf = torch.zeros(9 * n, device=opacity.device)
-    g = dict(mean2d=buf[:2 * n].view(n, 2), conic=buf[2 * n:5 * n].view(n, 3), opacity=buf[5 * n:6 * n],
-             rgb=buf[6 * n:].view(n, 3))
+    g = dict(mean2d=buf.as_strided((n, 2), (2, 1)), conic=buf.as_strided((n, 3), (3, 1), 2 * n),
+             opacity=buf.as_strided((n,), (1,), 5 * n), rgb=buf.as_strided((n, 3), (3, 1), 6 * n))
     gs_blend_backward(width, height, bs["tile_ranges"], _list_ids(bs), proj["mean2d"], proj["conic"], opacity,
                       proj["rgb"], opts, fwd["T_final"], fwd["n_contrib"], dL_dimage.contiguous(), g["mean2d"],
                       g["conic"], g["opacity"], g["rgb"], stream)
@@ -582,11 +581,14 @@ class BlendFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, mean2d, conic, opacity, rgb, tile_ranges, ids, width, height, opts):
         proj = dict(mean2d=mean2d.contiguous(), conic=conic.contiguous(), rgb=rgb.contiguous())
+        opacity = opacity.contiguous()
         bs = dict(tile_ranges=tile_ranges, ids=ids)
-        out = blend_forward(width, height, bs, proj, opacity.contiguous(), opts)
-        ctx.save_for_backward(proj["mean2d"], proj["conic"], opacity.contiguous(), proj["rgb"], tile_ranges, ids,
+        out = blend_forward(width, height, bs, proj, opacity, opts)
+        ctx.save_for_backward(proj["mean2d"], proj["conic"], opacity, proj["rgb"], tile_ranges, ids,
                               out["T_final"], out["n_contrib"])
         ctx.meta = (width, height, opts)
+        # no zero-filled gradients for T_final and n_contrib, which backward does not read
+        ctx.set_materialize_grads(False)
         ctx.mark_non_differentiable(out["T_final"], out["n_contrib"])
         return out["image"], out["T_final"], out["n_contrib"]
 
@@ -594,6 +596,8 @@ class BlendFunction(torch.autograd.Function):
     def backward(ctx, dimage, _dT, _dn):
         mean2d, conic, opacity, rgb, ranges, ids, T, nc = ctx.saved_tensors
         width, height, opts = ctx.meta
+        if dimage is None:
+            dimage = torch.zeros(3, height, width, device=T.device)
         g = blend_backward(width, height, dict(tile_ranges=ranges, ids=ids),
                            dict(mean2d=mean2d, conic=conic, rgb=rgb), opacity, opts,
                            dict(T_final=T, n_contrib=nc), dimage)
