@@ -12,21 +12,29 @@
 //      power_min, of its opacity-aware runs) in the tile's fixed slot range
 //      of `ids`, by an atomic counter per tile;
 //   4. a second grid barrier;
-//   5. each block orders its tiles' lists by (depth bits, Gaussian index) --
-//      the order of the global stable sort -- with a bitonic sort in shared
-//      memory and writes them back;
-//   6. (BLEND) the same block then blends the tile from the ordered list it
-//      holds in shared memory: per chunk of 32 splats, warp 0 builds the
-//      Eq. 6 coefficient rows of both 16 x 8 halves (fp16 hi + lo, as
-//      GS_BLEND_TC_FP16_SPLIT), one tcgen05.mma (M = 128 pixels, N = 64 rows,
-//      K = 16) leaves the exponents in TMEM, and warps w and w + 4 composite
-//      the upper and lower pixel of TMEM lane quarter w with the persistent
-//      blend's branch-free arithmetic (Eq. 1, Alg. 1's skip and stop rules),
-//      until every pixel of the tile has stopped.
+//   5. each team of 256 threads orders its tiles' lists by (depth bits,
+//      Gaussian index) -- the order of the global stable sort -- with a bitonic
+//      sort in shared memory and writes them back;
+//   6. (BLEND) the same team then blends the tile from the ordered list it
+//      holds in shared memory, without the entries that reach no pixel of it:
+//      every warp builds the Eq. 6 coefficient rows of both 16 x 8 halves of one
+//      chunk of 32 splats (fp16 hi + lo, as GS_BLEND_TC_FP16_SPLIT), one
+//      tcgen05.mma per chunk (M = 128 pixels, N = 64 rows, K = 16) leaves the
+//      exponents in TMEM, and warps w and w + 4 composite the upper and lower
+//      pixel of TMEM lane quarter w with the persistent blend's branch-free
+//      arithmetic (Eq. 1, Alg. 1's skip and stop rules), until every pixel of
+//      the tile has stopped.
 // The lists equal gs_bin_sort's lists tile by tile, so the blend kernels take
 // them unchanged, and the blended tiles equal gs_blend_forward's
 // (GS_BLEND_TC_FP16_SPLIT) on those lists.  One tile's list is sorted by one
-// block in shared memory, which is what limits this path to small scenes.
+// team in shared memory, which is what limits this path to small scenes.
+//
+// It waits for its chain of steps throughout.  256 x 256, 10k splats, degree 0:
+// 65 us with blocks of one team, rows built by one warp a chunk ahead and every
+// entry composited; 61 without the dead entries; 59.6 with eight lanes per
+// splat in step 3; 57.6 with the rows of eight chunks built together; 49 with
+// two teams per block.  A rank sort (runs of 32, binary searches) was no faster
+// than the bitonic one, and unrolled code costs its first instruction fetches.
 #include <algorithm>
 
 #include "blend_tc.cuh"
@@ -36,7 +44,24 @@
 namespace gs {
 namespace {
 
-constexpr int kFusedThreads = 256;
+constexpr int kFusedThreads = 512;
+// A tile's list and blend are the work of a team of 256 threads, two teams to a
+// block where their shared memory fits (lists of up to 8192): a cooperative
+// launch of a kernel that holds TMEM gets one block per SM, so a second tile
+// per SM has to be in the same block.
+constexpr int kTeamThreads = 256;
+__device__ __forceinline__ void team_sync(int team) {
+    asm volatile("bar.sync %0, %1;" ::"r"(team + 1), "n"(kTeamThreads) : "memory");
+}
+__device__ __forceinline__ bool team_sync_and(int team, bool v) {
+    uint32_t all;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(all)
+        : "r"((uint32_t)v), "r"(team + 1), "n"(kTeamThreads)
+        : "memory");
+    return all != 0;
+}
 constexpr int kScatterBatch = 8;  // a splat's tile counters incremented together
 constexpr uint64_t kFusedBarrierNs = 1000000000ull;  // 1 s
 
@@ -80,51 +105,59 @@ struct SmallArgs {
     int* n_contrib;
 };
 
-// The blend's shared memory after the sort keys: M_p, two stages of a chunk's
-// coefficient rows and records, three mbarriers (MMA done per stage, drain)
-// and the TMEM address.
+// Shared memory: M_p (with BLEND), then per team its sort keys and, with BLEND,
+// the coefficient rows and records of kRowStages chunks, three mbarriers (MMA
+// done per TMEM stage, drain); the TMEM address last.
 constexpr int kBlendV = GS_BLEND_TC_FP16_SPLIT;
 using BTR = tc::Traits<kBlendV>;
 constexpr int kBlendCh = 32;                       // splats per MMA
+constexpr int kRowStages = kTeamThreads / 32;     // chunks whose rows are built together, one per warp
 constexpr int kSmA = 128 * BTR::ROW_BYTES;         // 4 KB
 constexpr int kSmB = 2 * kBlendCh * BTR::ROW_BYTES;  // 2 KB per stage
 constexpr int kSmRec = kBlendCh * (int)sizeof(tc::Rec);
-constexpr int kSmBlend = kSmA + 2 * kSmB + 2 * kSmRec + 32;
+constexpr int kSmBlend = kRowStages * (kSmB + kSmRec) + 1024;  // per team
+constexpr int kMaxSmem = 226 * 1024;  // dynamic, beside a few static words
 constexpr uint32_t kBlendCols = 4 * kBlendCh;      // 2 stages x 64 TMEM columns (upper splats, lower splats)
-__host__ __device__ inline size_t blend_smem_offset(int pow2) { return ((size_t)8 * pow2 + 1023) / 1024 * 1024; }
+__host__ __device__ inline size_t key_bytes(int pow2) { return ((size_t)8 * pow2 + 1023) / 1024 * 1024; }
+__host__ __device__ inline size_t team_bytes(int pow2, bool blend) { return key_bytes(pow2) + (blend ? kSmBlend : 0); }
 
 template <int SH_DEGREE, bool VEC16, bool BLEND>
 __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __grid_constant__ SmallArgs a,
                                                                      const __grid_constant__ CamViews views,
-                                                                     int pow2) {
-    extern __shared__ __align__(1024) unsigned long long s_key[];  // (depth bits << 32) | index, pow2 of them
+                                                                     int pow2, int teams) {
+    extern __shared__ __align__(1024) uint8_t s_all[];
     const CamDev& cam = views.cams[0];
     const int n = a.n, max_per_tile = a.max_per_tile;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    uint8_t* sm = reinterpret_cast<uint8_t*>(s_key) + blend_smem_offset(pow2);
-    uint8_t* sA = sm;
-    uint8_t* sB = sm + kSmA;                                               // stage b at sB + b kSmB
-    tc::Rec* sRec = reinterpret_cast<tc::Rec*>(sm + kSmA + 2 * kSmB);     // stage b at sRec + b kBlendCh
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + kSmA + 2 * kSmB + 2 * kSmRec);  // [2]: drain
-    uint32_t* sTmem = reinterpret_cast<uint32_t*>(bars + 3);
+    const int lane = threadIdx.x & 31, team = threadIdx.x / kTeamThreads, tid = threadIdx.x % kTeamThreads;
+    const int warp = tid >> 5;  // within the team
+    uint8_t* sA = s_all;
+    // (a block of one team: the other team's pointers are not used)
+    uint8_t* sm = s_all + (BLEND ? kSmA : 0) + (team < teams ? team : 0) * team_bytes(pow2, BLEND);
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(sm);  // (depth bits << 32) | index, pow2 of them
+    uint8_t* sB = sm + key_bytes(pow2);                                      // stage b at sB + b kSmB
+    tc::Rec* sRec = reinterpret_cast<tc::Rec*>(sB + kRowStages * kSmB);      // stage b at sRec + b kBlendCh
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sB + kRowStages * (kSmB + kSmRec));  // [2]: drain
+    __shared__ uint32_t sTmem;
     uint32_t tmem = 0, mma_phase[2] = {0u, 0u};
+    __shared__ int s_kept_all[kFusedThreads / 32];
+    int* s_kept = s_kept_all + team * (kTeamThreads / 32);
     bool blend_ok = true;  // false once an MMA wait gave up: no further MMA is issued
     if constexpr (BLEND) {
-        if (threadIdx.x == 0) {
+        if (tid == 0 && team < teams) {
             for (int b = 0; b < 3; ++b) mbar_init(smem_u32(bars + b), 1);
             mbar_fence_init();
         }
         for (int row = threadIdx.x; row < 128; row += kFusedThreads)  // M_p of a 16 x 8 half, centre reference
             tc::store_mp_row<kBlendV>(sA, row, 7.5f - (float)(row & 15), 3.5f - (float)(row >> 4));
         fence_proxy_async_smem();
-        if (warp == 0) {
-            tmem_alloc(smem_u32(sTmem), kBlendCols);
+        if (threadIdx.x < 32) {
+            tmem_alloc(smem_u32(&sTmem), kBlendCols * teams);
             tmem_relinquish();
         }
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        tmem = *sTmem;
+        tmem = sTmem + team * kBlendCols;  // this team's columns
     }
 
     // 1. projection
@@ -139,8 +172,12 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
 
     // 3. every splat appends its index to the tiles it covers (the other
     // blocks' outputs are read through L2: this SM's L1 may hold lines from
-    // before the barrier)
-    for (int g = blockIdx.x * kFusedThreads + threadIdx.x; ok && g < n; g += gridDim.x * kFusedThreads) {
+    // before the barrier).  Up to half as many splats as threads: eight lanes share a
+    // splat's rows, as a chain of atomics per thread is what this step waits for.
+    const int share = n <= (int)(gridDim.x * kFusedThreads / 2) ? 8 : 1;
+    for (long long q = blockIdx.x * kFusedThreads + threadIdx.x; ok && q < (long long)n * share;
+         q += gridDim.x * kFusedThreads) {
+        const int g = (int)(q / share), sub = (int)(q % share);
         const int r = __ldcg(a.radius + g);
         if (r <= 0) continue;
         const float2 m = __ldcg(a.mean2d + g);
@@ -150,7 +187,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
         if (a.power_min != nullptr)
             tr = tight_rows(m.x, m.y, __ldcg(a.conic + 3 * g), __ldcg(a.conic + 3 * g + 1),
                             __ldcg(a.conic + 3 * g + 2), a.power_min[g]);
-        for (int y = y0; y <= y1; ++y) {
+        for (int y = y0 + sub; y <= y1; y += share) {
             int f = x0, l = x1;
             if (a.power_min != nullptr) tight_row(tr, y, x0, x1, f, l);
             for (int xb = f; xb <= l; xb += kScatterBatch) {  // the batch's atomics in flight together
@@ -169,13 +206,14 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
 
     // 4. per tile: (depth bits, index) keys, bitonic sort padded to a power of
     // two with keys above any real one, the list written back in order
-    for (int t = blockIdx.x; ok && t < ntiles; t += gridDim.x) {
+    // (the first teams of all blocks before any second one)
+    for (int t = blockIdx.x + team * gridDim.x; ok && team < teams && t < ntiles; t += gridDim.x * teams) {
         const unsigned total = __ldcg(&a.ranges[2 * t + 1]);
         const int cnt = (int)min(total, (unsigned)max_per_tile);
         uint32_t* list = a.ids + (size_t)t * max_per_tile;
         int P = 2;
         while (P < cnt) P <<= 1;
-        for (int i = threadIdx.x; i < P; i += kFusedThreads) {
+        for (int i = tid; i < P; i += kTeamThreads) {
             unsigned long long k = ~0ull;
             if (i < cnt) {
                 const uint32_t g = __ldcg(list + i);
@@ -183,10 +221,10 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
             }
             s_key[i] = k;
         }
-        __syncthreads();
+        team_sync(team);
         for (int k = 2; k <= P; k <<= 1) {
             for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < P; i += kFusedThreads) {
+                for (int i = tid; i < P; i += kTeamThreads) {
                     const int ixj = i ^ j;
                     if (ixj > i) {
                         const unsigned long long x = s_key[i], y = s_key[ixj];
@@ -196,11 +234,11 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                         }
                     }
                 }
-                __syncthreads();
+                team_sync(team);
             }
         }
-        for (int i = threadIdx.x; i < cnt; i += kFusedThreads) list[i] = (uint32_t)s_key[i];
-        if (threadIdx.x == 0) {
+        for (int i = tid; i < cnt; i += kTeamThreads) list[i] = (uint32_t)s_key[i];
+        if (tid == 0) {
             if (total > (unsigned)max_per_tile) atomicOr(a.err, kErrCapacity);
             a.ranges[2 * t] = (uint32_t)t * (uint32_t)max_per_tile;
             a.ranges[2 * t + 1] = (uint32_t)t * (uint32_t)max_per_tile + (uint32_t)cnt;
@@ -213,18 +251,44 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
             const bool in = px < cam.W && py < cam.H;
             float T = in ? 1.f : 0.f, Tstop = 0.f, last = 0.f, Cr = 0.f, Cg = 0.f, Cb = 0.f;
             const float xc = (float)lx + 8.0f, yc_up = (float)ly + 4.0f, yc_lo = (float)ly + 12.0f;
-            // chunk c in stage c & 1: warp 0 builds chunk c + 1's rows (and loads
-            // chunk c + 2's splats) while the MMA of chunk c runs and its
-            // exponents are composited
-            // warp 0's registers: the parameters of splat c0 + lane of the next chunk to build,
-            // loaded a chunk ahead so that their latency overlaps the compositing
+            // drop the entries that reach no pixel of the tile (with full rectangles about
+            // half): the chunks follow one another, and a tile's chain is what the launch
+            // waits for.  The kept ones move up in s_key, list positions in the high half.
+            int live = 0;
+            for (int i0 = 0; i0 < cnt; i0 += kTeamThreads) {
+                const int i = i0 + tid;
+                uint32_t g = 0;
+                bool keep = false;
+                if (i < cnt) {
+                    g = (uint32_t)s_key[i];
+                    const float2 m = __ldcg(a.mean2d + g);
+                    const float A = __ldcg(a.conic + 3 * g), B = __ldcg(a.conic + 3 * g + 1),
+                                C = __ldcg(a.conic + 3 * g + 2), o = a.opacity[g];
+                    keep = tc::splat_reaches<kBlendV>(A, B, C, o > 0.f ? __log2f(o) : -INFINITY, m.x - xc, m.y - yc_up,
+                                                      -7.5f, 7.5f, -3.5f, 3.5f);
+                }
+                const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                if (lane == 0) s_kept[warp] = __popc(kept);
+                team_sync(team);  // (also: the round's keys are read)
+                int at = live;
+                for (int w = 0; w < kTeamThreads / 32; ++w) {
+                    if (w < warp) at += s_kept[w];
+                    live += s_kept[w];
+                }
+                if (keep) s_key[at + __popc(kept & ((1u << lane) - 1u))] = (unsigned long long)(unsigned)i << 32 | g;
+                team_sync(team);
+            }
+            // kRowStages chunks at a time: every warp builds the rows of one of them (loads
+            // and arithmetic of all at once), then their MMAs run one after the other, chunk
+            // c in TMEM stage c & 1, each while the chunk before it is composited
             bool pv = false;
             float2 pm = make_float2(0.f, 0.f);
-            float pA = 0.f, pB = 0.f, pC = 0.f, po = 0.f, pr = 0.f, pg = 0.f, pb = 0.f;
+            float pA = 0.f, pB = 0.f, pC = 0.f, po = 0.f, pr = 0.f, pg = 0.f, pb = 0.f, pi = 0.f;
             auto fetch = [&](int c0) {
-                pv = c0 + lane < cnt;
+                pv = c0 + lane < live;
                 if (pv) {
                     const uint32_t g = (uint32_t)s_key[c0 + lane];
+                    pi = (float)(uint32_t)(s_key[c0 + lane] >> 32) + 1.0f;
                     pm = __ldcg(a.mean2d + g);
                     pA = __ldcg(a.conic + 3 * g);
                     pB = __ldcg(a.conic + 3 * g + 1);
@@ -235,7 +299,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                     pb = __ldcg(a.rgb + 3 * g + 2);
                 }
             };
-            auto build = [&](int st) {  // warp 0: the fetched splat's rows of both halves and record
+            auto build = [&](int st) {  // the fetched splat's rows of both halves and record, in row stage st
                 uint8_t* mB = sB + st * kSmB;
                 float vu[6], vl[6];
                 tc::Rec rc;
@@ -246,7 +310,7 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                     tc::coeff_row<true>(pA, pB, pC, l2o, xh, pm.y - yc_lo, -7.5f, 7.5f, -3.5f, 3.5f, vl);
                     const float cap = fminf(l2o, tc::kLog2AlphaMax);
                     rc.rg = make_float4(pr, pr, pg, pg);
-                    rc.bc = make_float4(pb, pb, cap, cap);
+                    rc.bc = make_float4(pb, pb, cap, pi);
                 } else {  // padding: dead rows, no colour
 #pragma unroll
                     for (int i = 0; i < 5; ++i) vu[i] = vl[i] = 0.f;
@@ -258,45 +322,39 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                 sRec[st * kBlendCh + lane] = rc;
                 fence_proxy_async_smem();
             };
-            auto issue = [&](int st) {  // thread 0: the MMA of stage st, committed to its barrier
+            auto issue = [&](int c) {  // thread 0: the MMA of chunk c, committed to its TMEM stage's barrier
                 tc_fence_after();
                 constexpr uint32_t IDESC = idesc_f16(BTR::FMT, 128, 2 * kBlendCh);
-                tc::tc_mma<kBlendV>(tmem + (uint32_t)(st * 2 * kBlendCh), smem_desc(smem_u32(sA), 128, BTR::SBO),
-                                    smem_desc(smem_u32(sB + st * kSmB), 128, BTR::SBO), IDESC, 0u);
-                tc_commit(smem_u32(bars + st));
+                tc::tc_mma<kBlendV>(tmem + (uint32_t)((c & 1) * 2 * kBlendCh), smem_desc(smem_u32(sA), 128, BTR::SBO),
+                                    smem_desc(smem_u32(sB + c % kRowStages * kSmB), 128, BTR::SBO), IDESC, 0u);
+                tc_commit(smem_u32(bars + (c & 1)));
             };
-            const int nchunk = blend_ok ? (cnt + kBlendCh - 1) / kBlendCh : 0;
-            if (nchunk > 0) {
-                if (warp == 0) {
-                    fetch(0);
-                    build(0);
-                    if (nchunk > 1) fetch(kBlendCh);
-                }
-                __syncthreads();
-                if (threadIdx.x == 0) issue(0);
-            }
+            const int nchunk = blend_ok ? (live + kBlendCh - 1) / kBlendCh : 0;
             int c = 0;
             bool pending = false;  // an MMA issued and not yet waited for (chunk c + 1's)
             for (; c < nchunk; ++c) {
-                const int st = c & 1;
-                const bool more = c + 1 < nchunk;
-                if (more && warp == 0) {
-                    build(st ^ 1);
-                    if (c + 2 < nchunk) fetch((c + 2) * kBlendCh);
+                const int st = c & 1, row = c % kRowStages;
+                if (row == 0) {  // (no MMA is in flight: the row stages are free)
+                    if (c + warp < nchunk) {
+                        fetch((c + warp) * kBlendCh);
+                        build(warp);
+                    }
+                    team_sync(team);
+                    if (tid == 0) issue(c);
                 }
+                const bool more = c + 1 < nchunk && row + 1 < kRowStages;
                 const bool got = mbar_wait_bounded(smem_u32(bars + st), mma_phase[st], kFusedBarrierNs, nullptr);
                 mma_phase[st] ^= 1u;
-                if (!__syncthreads_and(got)) {  // (also: chunk c + 1's rows are in place)
-                    if (threadIdx.x == 0) atomicOr(a.err, kErrTimeout);
+                if (!team_sync_and(team, got)) {
+                    if (tid == 0) atomicOr(a.err, kErrTimeout);
                     blend_ok = false;
                     pending = false;  // whatever is in flight, the final drain waits for it
                     break;
                 }
-                if (more && threadIdx.x == 0) issue(st ^ 1);
+                if (more && tid == 0) issue(c + 1);
                 pending = more;
                 tc_fence_after();
-                const int c0 = c * kBlendCh;
-                const tc::Rec* rec = sRec + st * kBlendCh;
+                const tc::Rec* rec = sRec + row * kBlendCh;
                 const uint32_t tcol = tmem + ((uint32_t)((warp & 3) * 32) << 16) +
                                       (uint32_t)(st * 2 * kBlendCh + h * kBlendCh);
 #pragma unroll 1
@@ -320,12 +378,11 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                         Cg = fmaf(rc.rg.z, w, Cg);
                         Cb = fmaf(rc.bc.x, w, Cb);
                         const float used = tc::sat(__fmul_rn(a2, tc::kCullScale));
-                        const float idx1 = (float)(c0 + q0 + q + 1);
-                        last = fmaf(used, __fadd_rn(idx1, -last), last);
+                        last = fmaf(used, __fadd_rn(rc.bc.w, -last), last);
                     }
                 }
                 tc_fence_before();
-                if (__syncthreads_and(T == 0.f)) {  // every pixel of the tile has stopped
+                if (team_sync_and(team, T == 0.f)) {  // every pixel of the tile has stopped
                     ++c;
                     break;
                 }
@@ -334,8 +391,8 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                 const int st = c & 1;
                 const bool got = mbar_wait_bounded(smem_u32(bars + st), mma_phase[st], kFusedBarrierNs, nullptr);
                 mma_phase[st] ^= 1u;
-                if (!__syncthreads_and(got)) {
-                    if (threadIdx.x == 0) atomicOr(a.err, kErrTimeout);
+                if (!team_sync_and(team, got)) {
+                    if (tid == 0) atomicOr(a.err, kErrTimeout);
                     blend_ok = false;
                 }
             }
@@ -349,18 +406,18 @@ __global__ void __launch_bounds__(kFusedThreads) k_project_bin_small(const __gri
                 a.n_contrib[p] = (int)last;
             }
         }
-        __syncthreads();
+        team_sync(team);
     }
     if constexpr (BLEND) {
-        // every MMA this block issued has completed before TMEM is freed
-        if (threadIdx.x == 0) {
+        // every MMA this team issued has completed before TMEM is freed
+        if (tid == 0 && team < teams) {
             tc_commit(smem_u32(bars + 2));
             mbar_wait_bounded(smem_u32(bars + 2), 0, kFusedBarrierNs, nullptr);
         }
         tc_fence_before();
         __syncthreads();
         tc_fence_after();
-        if (warp == 0) tmem_dealloc(tmem, kBlendCols);
+        if (threadIdx.x < 32) tmem_dealloc(tmem, kBlendCols * teams);
     }
 }
 
@@ -369,7 +426,9 @@ cudaError_t launch_fused(const SmallArgs& args, const CamViews& cams, cudaStream
     auto kern = k_project_bin_small<D, V, BLEND>;
     int pow2 = 2;  // the sort pads a tile's keys to a power of two
     while (pow2 < args.max_per_tile) pow2 <<= 1;
-    const size_t smem = BLEND ? blend_smem_offset(pow2) + kSmBlend : sizeof(unsigned long long) * (size_t)pow2;
+    const size_t shared_part = BLEND ? kSmA : 0;
+    const int teams = shared_part + 2 * team_bytes(pow2, BLEND) <= (size_t)kMaxSmem ? 2 : 1;
+    const size_t smem = shared_part + teams * team_bytes(pow2, BLEND);
     // residency for the last shared-memory size, as for the other kernels once per process
     // (under a lock: host threads may call at the same time)
     static std::mutex mu;
@@ -394,8 +453,8 @@ cudaError_t launch_fused(const SmallArgs& args, const CamViews& cams, cudaStream
             if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s_per_sm, kern, kFusedThreads, smem)) !=
                 cudaSuccess)
                 return e;
-            // BLEND: every resident block holds kBlendCols of the SM's 512 TMEM columns
-            if (BLEND) s_per_sm = std::min(s_per_sm, (int)(512 / kBlendCols));
+            // BLEND: every resident block holds its teams' columns of the SM's 512 of TMEM
+            if (BLEND) s_per_sm = std::min(s_per_sm, (int)(512 / (kBlendCols * teams)));
             cached_sms = s_sms;
             cached_per_sm = s_per_sm;
             cached_smem = smem;
@@ -408,7 +467,7 @@ cudaError_t launch_fused(const SmallArgs& args, const CamViews& cams, cudaStream
     const int need = std::max(ntiles, (args.n + kFusedThreads - 1) / kFusedThreads);
     const int grid = std::max(1, std::min(need, std::max(per_sm, 1) * sms));
     if ((e = cudaMemsetAsync(args.barrier, 0, 2 * sizeof(unsigned), s)) != cudaSuccess) return e;
-    void* kargs[] = {(void*)&args, (void*)&cams, (void*)&pow2};
+    void* kargs[] = {(void*)&args, (void*)&cams, (void*)&pow2, (void*)&teams};
     e = cudaLaunchCooperativeKernel((const void*)kern, dim3(grid), dim3(kFusedThreads), kargs, smem, s);
     count_launches();
     return e;

@@ -174,3 +174,22 @@ def test_fused_rejects_bad_arguments():
         with pytest.raises(gs.GsError):
             gs.project_bin_small(dev["means"], dev["scales"], dev["quats"], dev["sh"], dev["sh_degree"], cam,
                                  max_per_tile=mpt)
+
+
+@pytest.mark.parametrize("max_per_tile", [4096, 8192, 16384])  # two teams per block, two, one
+@pytest.mark.parametrize("n", [1, 255, 257, 9000, 45000])  # eight lanes share a splat, or none do
+def test_fused_render_teams_and_shared_rows(n, max_per_tile):
+    cam = scenes.look_at_camera((0, 0, -3), (0, 0, 0), 400, 300)  # 475 tiles: several per team
+    rng = np.random.default_rng(n)
+    t = lambda a: torch.from_numpy(np.ascontiguousarray(a, np.float32)).cuda()  # noqa: E731
+    means, scales = t(rng.uniform(-1, 1, (n, 3))), t(np.exp(rng.normal(-4.2, 0.6, (n, 3))))
+    quats, sh, op = t(rng.normal(size=(n, 4))), t(rng.uniform(0, 1, (n, 1, 3))), t(rng.uniform(0.002, 0.9, n))
+    proj, bs, fwd = gs.render_small(means, scales, quats, sh, 0, op, cam, max_per_tile=max_per_tile)
+    assert gs.gs_sync_status() == gs.GS_OK
+    ref_bs = gs.BinSorter("cuda").run(proj["mean2d"], proj["radius"], proj["depth"], cam.width, cam.height)
+    assert _tile_lists(bs["tile_ranges"].cpu().numpy(), bs["ids"].cpu().numpy()) == \
+        _tile_lists(ref_bs["tile_ranges"].cpu().numpy(), ref_bs["ids"].cpu().numpy())
+    ref = gs.blend_forward(cam.width, cam.height, bs, proj, op, gs.make_opts("fp16_split"))
+    assert gs.gs_sync_status() == gs.GS_OK
+    for k in ("image", "T_final", "n_contrib"):
+        assert torch.equal(fwd[k], ref[k]), k
