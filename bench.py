@@ -59,7 +59,7 @@ KNOWN_TRAFFIC = {}
 #  - bytes per instance a blend touches: the id and the splat's record
 #    (mean2d 8, conic 12, opacity 4, rgb 12); per pixel written or read:
 #    image 12, T_final 4, n_contrib 4 (forward), plus dL/dimage 12 (backward);
-#    the backward adds 9 gradient floats per (instance, tile half);
+#    the backward adds 9 gradient floats per instance;
 #  - bin/sort: per Gaussian its inputs (mean2d, radius, depth, conic,
 #    power_min: 32 bytes) and per instance the sorted id (4 bytes), per tile
 #    its range (8 bytes): the least a binning must move.
@@ -314,8 +314,9 @@ def _timed(torch, flush, stream, fn, reps):
 
 
 def backward_issued_pairs(torch, n_contrib, chunk=16):
-    """Pairs the tensor-core backward evaluates: every pixel of a tile, in
-    chunks of 16 splats, up to the tile's longest n_contrib."""
+    """Pairs the tensor-core backward may evaluate: every pixel of a tile, in
+    chunks of 16 splats, up to the tile's longest n_contrib (an upper bound: it
+    drops the entries that reach no pixel of the tile)."""
     H, W = n_contrib.shape
     ty, tx = (H + 15) // 16, (W + 15) // 16
     nc = torch.zeros(ty * 16, tx * 16, dtype=torch.int32, device=n_contrib.device)
@@ -339,7 +340,7 @@ def blend_roofline(kind, variant, t_ms, evals, issued, pixels, peaks):
     else:
         terms["mufu"] = {"per_s": 1.0 / (1.0 / ex2 + 1.0 / rcp), "note": "1 ex2 + 1 rcp per evaluated pair"}
         ops = FP32_OPS["backward"]
-        bytes_ = issued / 256 * (REC_BYTES + 2 * 36) + pixels * 32
+        bytes_ = issued / 256 * (REC_BYTES + 36) + pixels * 32
         flops_pair = (256 + 2 * K_OF.get(variant, 0)) * issued / max(evals, 1)
     terms["fp32_issue"] = {"per_s": fma / ops, "note": f"{ops} FP32 operations per evaluated pair at the measured "
                                                        f"FMA rate {fma / 1e12:.1f} T/s"}
@@ -633,7 +634,7 @@ def run_ours(args):
                     "frac": round(ach / hbm, 4) if hbm else None, "traffic": None, "launch_ms": round(dup_ms, 5),
                     "algorithmic_bytes": dup_bytes, "pairs": n_pairs,
                     "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst) of measured",
-                    "note": "bound by instruction issue and latency, not by HBM (ncu: issue 56% busy, 4 blocks "
+                    "note": "bound by instruction issue and latency, not by HBM (ncu: issue 55% busy, 4 blocks "
                             "per SM); algorithmic bytes: 32 per Gaussian read, 8 per supertile pair written"}
     else:
         r = rf if dom == "blend_forward" else rb
@@ -713,7 +714,8 @@ def run_ours(args):
         "forward_pairs": {"evaluated_per_frame": evals_fwd, "issued_per_frame": issued_fwd,
                           "backward_issued_per_frame": issued_bwd,
                           "note": "evaluated = sum of n_contrib (the metric's pairs); issued = 256 x the splats of "
-                                  "every chunk the tensor-core kernels evaluate before a tile's exit"},
+                                  "every chunk the forward evaluates before a tile's exit, entries that reach no "
+                                  "pixel of the tile left out; backward: an upper bound that counts them"},
         **({"projection_backward": pb_line} if pb_line else {}),
         **({"small_scene_fused": small_line} if small_line else {}),
         **({"batched_views": batched_line} if batched_line else {}),

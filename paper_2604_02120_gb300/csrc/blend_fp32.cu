@@ -9,9 +9,10 @@
 // test 32 staged splats at a time against that block (warp_reaches, about one
 // instruction per pair) and only the splats that can contribute are walked, in
 // list order and with their list positions: the same decisions and the same
-// values as the walk over all.  Full rectangles, forward and backward:
-// 641 x 479, 50k splats 107 -> 61 us and 225 -> 154 us; 1920 x 1080, 1M
-// clustered 994 -> 398 us and 2207 -> 1238 us (issue slots 86% and 75% busy).
+// values as the walk over all.  Forward and backward against the walk over all:
+// full rectangles, 641 x 479, 50k splats 105 -> 60 us and 217 -> 152 us; 1920 x
+// 1080, 1M clustered 995 -> 410 us and 2209 -> 1256 us; opacity-aware lists there
+// 379 -> 321 us and 1228 -> 1101 us; 1280 x 720, 200k 99 -> 86 us and 281 -> 262 us.
 #include "blend_tc.cuh"
 #include "internal.h"
 
@@ -58,6 +59,13 @@ __device__ __forceinline__ bool warp_reaches(const float4& geo, const float4& oc
     const float S = fmaf(0.5f * fabsf(geo.z) * ax, ax, fmaf(fabsf(geo.w) * ax, ay, 0.5f * fabsf(oc.x) * ay * ay));
     return tc::box_reaches(geo.z, geo.w, oc.x, l2o, x0, x1, y0, y1, S, 1.0f / 131072);
 }
+
+// A batch whose first 32 splats include four in five that the warp needs is walked
+// whole, by the plain loop: it costs less per splat than one over set bits, and
+// what the tests would spare there does not pay for them.  Opacity-aware lists of
+// large splats (3840 x 2160, 3M, heavy tails), forward / backward: without any
+// test 636 / 2266 us, with this rule 660 / 2317, with every group tested 793 / 2482.
+__device__ __forceinline__ bool dense_group(unsigned hits, int n) { return 5 * __popc(hits) >= 4 * n; }
 
 // Geometry of the block's tile (blockIdx.x is a global tile id).
 struct TileGeo {
@@ -113,21 +121,38 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
         }
         __syncthreads();
         const int nb = min(kBatch, len - base);
-        for (int c = 0; c < nb; c += 32) {
-            if (__all_sync(0xffffffffu, done)) break;
+        auto step = [&](int j) {
+            const float4 geo = s_geo[j], oc = s_oc[j];
+            float e, pw, dx, dy;
+            const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
+            if (done || alpha < kAlphaMin) return;
+            const float tT = T * (1.0f - alpha);
+            if (tT < kTMin) {
+                done = true;
+                return;
+            }
+            const float w = alpha * T;
+            cr = __fmaf_rn(oc.z, w, cr);
+            cg = __fmaf_rn(oc.w, w, cg);
+            cb = __fmaf_rn(s_bl[j].x, w, cb);
+            T = tT;
+            last = base + j + 1;
+        };
+        auto test = [&](int c) {
             const int t = c + lane;
-            unsigned hits =
-                __ballot_sync(0xffffffffu, t < nb && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
-            for (; hits; hits &= hits - 1) {
-                const int j = c + __ffs(hits) - 1;
+            return __ballot_sync(0xffffffffu, t < nb && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
+        };
+        unsigned hits = test(0);
+        if (dense_group(hits, min(32, nb))) {
+            for (int j = 0; !done && j < nb; ++j) {
                 const float4 geo = s_geo[j], oc = s_oc[j];
                 float e, pw, dx, dy;
                 const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
-                if (done || alpha < kAlphaMin) continue;
+                if (alpha < kAlphaMin) continue;
                 const float tT = T * (1.0f - alpha);
                 if (tT < kTMin) {
                     done = true;
-                    continue;
+                    break;
                 }
                 const float w = alpha * T;
                 cr = __fmaf_rn(oc.z, w, cr);
@@ -135,6 +160,13 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
                 cb = __fmaf_rn(s_bl[j].x, w, cb);
                 T = tT;
                 last = base + j + 1;
+            }
+        } else {
+            for (int c = 0;;) {
+                for (; hits; hits &= hits - 1) step(c + __ffs(hits) - 1);
+                c += 32;
+                if (c >= nb || __all_sync(0xffffffffu, done)) break;
+                hits = test(c);
             }
         }
     }
@@ -240,60 +272,73 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_bwd(const __grid_constant
             s_id[threadIdx.x] = g;
         }
         __syncthreads();
-        // this warp only needs list positions below its largest n_contrib
-        for (int top = min(hi, wmax); top > lo; top -= 32) {
-            const int t = top - 1 - lane - lo;
-            unsigned hits =
-                __ballot_sync(0xffffffffu, t >= 0 && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
-            for (; hits; hits &= hits - 1) {
-                const int j = top - __ffs(hits), k = j - lo;
-                const float4 geo = s_geo[k], oc = s_oc[k];
-                const float cb = s_bl[k].x;
-                float v[9];
+        auto step = [&](int j) {
+            const int k = j - lo;
+            const float4 geo = s_geo[k], oc = s_oc[k];
+            const float cb = s_bl[k].x;
+            float v[9];
 #pragma unroll
-                for (int q = 0; q < 9; ++q) v[q] = 0.f;
-                bool contrib = false;
-                if (j < nc) {
-                    float e, pw, dx, dy;
-                    const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
-                    if (alpha >= kAlphaMin) {
-                        contrib = true;
-                        const float Ti = __fdividef(T, 1.0f - alpha);
-                        const float wgt = alpha * Ti;
-                        v[6] = wgt * g0;
-                        v[7] = wgt * g1;
-                        v[8] = wgt * g2;
-                        const float dL_dalpha = Ti * ((oc.z - S0) * g0 + (oc.w - S1) * g1 + (cb - S2) * g2);
-                        S0 = fmaf(alpha, oc.z - S0, S0);
-                        S1 = fmaf(alpha, oc.w - S1, S1);
-                        S2 = fmaf(alpha, cb - S2, S2);
-                        T = Ti;
-                        if (oc.y * e <= kAlphaMax) {  // not clamped
-                            v[5] = dL_dalpha * e;
-                            if (pw <= 0.0f) {
-                                const float dp = dL_dalpha * alpha;
-                                v[0] = -dp * (geo.z * dx + geo.w * dy);
-                                v[1] = -dp * (geo.w * dx + oc.x * dy);
-                                v[2] = -0.5f * dp * dx * dx;
-                                v[3] = -dp * dx * dy;
-                                v[4] = -0.5f * dp * dy * dy;
-                            }
+            for (int q = 0; q < 9; ++q) v[q] = 0.f;
+            bool contrib = false;
+            if (j < nc) {
+                float e, pw, dx, dy;
+                const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
+                if (alpha >= kAlphaMin) {
+                    contrib = true;
+                    const float Ti = __fdividef(T, 1.0f - alpha);
+                    const float wgt = alpha * Ti;
+                    v[6] = wgt * g0;
+                    v[7] = wgt * g1;
+                    v[8] = wgt * g2;
+                    const float dL_dalpha = Ti * ((oc.z - S0) * g0 + (oc.w - S1) * g1 + (cb - S2) * g2);
+                    S0 = fmaf(alpha, oc.z - S0, S0);
+                    S1 = fmaf(alpha, oc.w - S1, S1);
+                    S2 = fmaf(alpha, cb - S2, S2);
+                    T = Ti;
+                    if (oc.y * e <= kAlphaMax) {  // not clamped
+                        v[5] = dL_dalpha * e;
+                        if (pw <= 0.0f) {
+                            const float dp = dL_dalpha * alpha;
+                            v[0] = -dp * (geo.z * dx + geo.w * dy);
+                            v[1] = -dp * (geo.w * dx + oc.x * dy);
+                            v[2] = -0.5f * dp * dx * dx;
+                            v[3] = -dp * dx * dy;
+                            v[4] = -0.5f * dp * dy * dy;
                         }
                     }
                 }
-                const unsigned who = __ballot_sync(0xffffffffu, contrib);
-                if (who == 0u) continue;
-                const uint32_t g = s_id[k];
-                if (__popc(who) <= 3) {
-                    if (contrib) {
+            }
+            const unsigned who = __ballot_sync(0xffffffffu, contrib);
+            if (who == 0u) return;
+            const uint32_t g = s_id[k];
+            if (__popc(who) <= 3) {
+                if (contrib) {
 #pragma unroll
-                        for (int q = 0; q < 9; ++q) atomicAdd(grad_slot(gr, g, tg.opac_off, q), v[q]);
-                    }
-                } else {
-                    float vk, v8;
-                    warp_reduce9(v, lane, vk, v8);
-                    if ((lane & 3) == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, lane >> 2), vk);
-                    if (lane == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, 8), v8);
+                    for (int q = 0; q < 9; ++q) atomicAdd(grad_slot(gr, g, tg.opac_off, q), v[q]);
+                }
+            } else {
+                float vk, v8;
+                warp_reduce9(v, lane, vk, v8);
+                if ((lane & 3) == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, lane >> 2), vk);
+                if (lane == 0) atomicAdd(grad_slot(gr, g, tg.opac_off, 8), v8);
+            }
+        };
+        // this warp only needs list positions below its largest n_contrib
+        int top = min(hi, wmax);
+        if (top > lo) {
+            auto test = [&]() {
+                const int t = top - 1 - lane - lo;
+                return __ballot_sync(0xffffffffu, t >= 0 && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
+            };
+            unsigned hits = test();
+            if (dense_group(hits, min(32, top - lo))) {
+                for (int j = top - 1; j >= lo; --j) step(j);
+            } else {
+                for (;;) {
+                    for (; hits; hits &= hits - 1) step(top - __ffs(hits));
+                    top -= 32;
+                    if (top <= lo) break;
+                    hits = test();
                 }
             }
         }

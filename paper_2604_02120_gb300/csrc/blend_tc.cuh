@@ -6,7 +6,7 @@
 // half; M_p (A operand, 128 x K) holds the monomials
 // [xb^2, yb^2, xb yb, xb, yb, 1] of the 128 pixels of a half relative to the
 // half's reference pixel and is built once per CTA.  For every chunk of CH
-// splats of a tile the producer writes 2 CH coefficient rows v_g (Eq. 6):
+// splats of a tile the builder writes 2 CH coefficient rows v_g (Eq. 6):
 // rows [0, CH) referred to the upper half's reference, rows [CH, 2 CH) to the
 // lower half's (8 pixels further down).  One tcgen05.mma (M = 128, N = 2 CH,
 // K = 16 or 32) then leaves in TMEM lane r, column j the exponent of splat j
@@ -66,10 +66,10 @@ namespace gs {
 namespace tc {
 
 constexpr int kEpiWarps = 4;
-constexpr int kThreads = 192;     // backward: epilogue warps, producer, MMA
+constexpr int kThreads = 192;     // 4 epilogue warps, scanner, row builder
 constexpr int kFwdThreads = 192;  // forward: epilogue warps, scanner, row builder
 constexpr int kTStages = 2;
-constexpr int kDoneRing = 16;  // tiles in flight between producer and epilogue < kDoneRing
+constexpr int kDoneRing = 16;  // tiles in flight between scanner and epilogue < kDoneRing
 constexpr float kAlphaMin = 1.0f / 255.0f;
 constexpr float kTMin = 1e-4f;
 constexpr float kLog2e = 1.4426950408889634f;
