@@ -26,7 +26,11 @@
 // start, publish their per-digit counts, then add up their predecessors'
 // published counts until one carries an inclusive prefix.  A block only waits
 // for blocks that started before it, so the waits always end; each is still
-// bounded in time and sets the timeout bit of the error word if it gives up.
+// bounded in time.  One that gives up sets the timeout bit of the error word and
+// the call's own flag (GiveUp): its kernel goes on with a prefix too small, so
+// everything after it holds holes and stale words, which every kernel up to the
+// pair sort bounds before it writes, and the tile counts are left at zero: every
+// list comes out empty, and nothing is read through ids that were never written.
 // The scan of coarse counts in depth order is done the same way inside the
 // duplication kernels (k_dup_rect for full rectangles, k_dup_coarse for
 // opacity-aware lists), so the whole stage is
@@ -48,7 +52,20 @@ constexpr uint32_t kSmallPass = 1u << 20;
 // halves the look-back.
 constexpr int kDupTile = kThreads;          // items per tile of the opacity-aware duplication
 constexpr int kMaxPasses = 8;               // 4 depth passes + up to 4 tile-id passes
-constexpr uint64_t kLookbackLimitNs = 2000000000ull;
+#ifndef GS_LOOKBACK_LIMIT_NS
+#define GS_LOOKBACK_LIMIT_NS 2000000000ull  // 2 s; a test builds the file with 0
+#endif
+constexpr uint64_t kLookbackLimitNs = GS_LOOKBACK_LIMIT_NS;
+
+// Where a look-back that gives up says so: the device's error word and the flag
+// of this call, in its workspace (k_pair_masks reads it).
+struct GiveUp {
+    unsigned *err, *call;
+    __device__ __forceinline__ void set() const {
+        atomicOr(err, kErrTimeout);
+        atomicOr(call, 1u);
+    }
+};
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -116,7 +133,7 @@ __device__ __forceinline__ unsigned long long ld_status(const unsigned long long
 // the ready ones nearest to this group are consumed, up to the first inclusive
 // prefix.
 __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* status, int64_t tile, int stride,
-                                                    int d, uint32_t tag_agg, unsigned* err) {
+                                                    int d, uint32_t tag_agg, const GiveUp& gu) {
     constexpr int W = 4;
     uint64_t prefix = 0, t0 = 0;
     int64_t j = tile - 1;
@@ -148,7 +165,7 @@ __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* st
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > kLookbackLimitNs) {
-                atomicOr(err, kErrTimeout);
+                gu.set();
                 break;
             }
         }
@@ -169,7 +186,7 @@ __device__ __forceinline__ uint64_t lookback_serial(const unsigned long long* st
 // 77 for the large ones with the ranking below and groups of 8.
 constexpr int kGroup = 8;
 constexpr int kRowTagBit = 27;
-__device__ __forceinline__ uint32_t group_sum(const uint32_t* rows, int64_t tile, int d, uint32_t tag, unsigned* err) {
+__device__ __forceinline__ uint32_t group_sum(const uint32_t* rows, int64_t tile, int d, uint32_t tag, const GiveUp& gu) {
     const int m = (int)(tile % kGroup);
     const uint32_t* p = rows + (size_t)(tile - m) * 256 + d;
     uint64_t t0 = 0;
@@ -193,7 +210,7 @@ __device__ __forceinline__ uint32_t group_sum(const uint32_t* rows, int64_t tile
         if (t0 == 0) {
             t0 = now;
         } else if (now - t0 > kLookbackLimitNs) {
-            atomicOr(err, kErrTimeout);
+            gu.set();
             return 0;
         }
     }
@@ -202,7 +219,7 @@ __device__ __forceinline__ uint32_t group_sum(const uint32_t* rows, int64_t tile
 // The same for a single count per tile, by one warp over windows of 32
 // predecessors (lane l reads tile j - l).  Every lane returns the prefix.
 __device__ __forceinline__ uint64_t lookback_warp(const unsigned long long* status, int64_t tile, uint32_t tag_agg,
-                                                  unsigned* err) {
+                                                  const GiveUp& gu) {
     const int lane = threadIdx.x & 31;
     uint64_t prefix = 0, t0 = 0;
     int64_t j = tile - 1;
@@ -220,7 +237,7 @@ __device__ __forceinline__ uint64_t lookback_warp(const unsigned long long* stat
             if (t0 == 0) {
                 t0 = now;
             } else if (now - t0 > kLookbackLimitNs) {
-                if (lane == 0) atomicOr(err, kErrTimeout);
+                if (lane == 0) gu.set();
                 break;
             }
             continue;
@@ -278,7 +295,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
                                                        const uint64_t* __restrict__ n_dev, int shift, int pass_id,
                                                        const uint32_t* __restrict__ hist, uint32_t* tickets,
                                                        unsigned long long* status, uint32_t* __restrict__ kout,
-                                                       uint32_t* __restrict__ vout, unsigned* err) {
+                                                       uint32_t* __restrict__ vout, GiveUp gu) {
     constexpr int TILE = kThreads * ITEMS;
     __shared__ uint32_t s_w[kThreads / 32][256];  // per-warp digit counts, then local bases
     __shared__ uint32_t s_dbase[256];              // block-local start of each digit's run
@@ -362,10 +379,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_onesweep(const uint32_t* __rest
             uint32_t prefix = 0;
             const int64_t g = tile / kGroup;
             const bool closes = tile % kGroup == kGroup - 1;
-            if (tile % kGroup) prefix = group_sum(rows, tile, d, tag_agg, err);
+            if (tile % kGroup) prefix = group_sum(rows, tile, d, tag_agg, gu);
             if (closes) st_status(groups + (size_t)g * 256 + d, g == 0 ? tag_agg + 1 : tag_agg, prefix + c);
             if (g > 0) {
-                prefix += (uint32_t)lookback_serial(groups, g, 256, d, tag_agg, err);
+                prefix += (uint32_t)lookback_serial(groups, g, 256, d, tag_agg, gu);
                 if (closes) st_status(groups + (size_t)g * 256 + d, tag_agg + 1, prefix + c);
             }
             s_dbase[d] = db;
@@ -414,7 +431,7 @@ struct PassScratch {
     const uint32_t* hist;  // [kMaxPasses][256] digit counts
     uint32_t* tickets;     // [kMaxPasses]
     unsigned long long* status;
-    unsigned* err;
+    GiveUp gu;
 };
 
 // Stable LSD sort of (k[0], v[0]) on bits [0, bits) with pass ids
@@ -438,7 +455,7 @@ cudaError_t radix_sort(uint32_t* k[2], uint32_t* v[2], uint32_t n_host, const ui
                     : items == 8 ? (full ? k_onesweep<8, true> : k_onesweep<8, false>)
                                  : (full ? k_onesweep<16, true> : k_onesweep<16, false>);
         kern<<<nblk, kThreads, 0, s>>>(k[cur], v[cur], n_host, n_dev, shift, id, ps.hist + 256 * id, ps.tickets,
-                                       ps.status, k[cur ^ 1], v[cur ^ 1], ps.err);
+                                       ps.status, k[cur ^ 1], v[cur ^ 1], ps.gu);
         count_launches();
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
@@ -659,7 +676,7 @@ __global__ void __launch_bounds__(kThreads, kDupBlocks)
                  bool pack, uint32_t* tickets, unsigned long long* status, uint32_t* __restrict__ ckey,
                  uint32_t* __restrict__ cval, uint32_t* __restrict__ hist, uint64_t* __restrict__ total,
                  unsigned long long* __restrict__ fine_total, unsigned long long* __restrict__ radix_status,
-                 uint32_t coarse_tile, uint32_t* __restrict__ st_zero, int st_n, unsigned* err) {
+                 uint32_t coarse_tile, uint32_t* __restrict__ st_zero, int st_n, GiveUp gu) {
     __shared__ uint32_t s_warp[kThreads / 32 + 1];
     __shared__ uint64_t s_prefix;
     __shared__ uint32_t s_tile;
@@ -851,7 +868,7 @@ __global__ void __launch_bounds__(kThreads, kDupBlocks)
                     if (warp == 0) {
                         uint64_t prefix = 0;
                         if (tile > 0) {
-                            prefix = lookback_warp(status, tile, 1u, err);
+                            prefix = lookback_warp(status, tile, 1u, gu);
                             if (lane == 0) st_status(status + tile, 2u, prefix + tile_sum);
                         }
                         if (lane == 0) {
@@ -916,7 +933,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
                                                           unsigned long long* __restrict__ fine_total,
                                                           unsigned long long* __restrict__ radix_status,
                                                           uint32_t coarse_tile, uint32_t* __restrict__ st_zero,
-                                                          int st_n, unsigned* err) {
+                                                          int st_n, GiveUp gu) {
     __shared__ uint64_t s_warp[kThreads / 32 + 1];
     __shared__ uint64_t s_prefix;
     __shared__ unsigned long long s_fine;
@@ -989,7 +1006,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
         if (warp == 0) {
             uint64_t prefix = 0;
             if (tile > 0) {
-                prefix = lookback_warp(status, tile, 1u, err);
+                prefix = lookback_warp(status, tile, 1u, gu);
                 if (lane == 0) st_status(status + tile, 2u, prefix + tile_sum);
             }
             if (lane == 0) {
@@ -1107,7 +1124,9 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
                                                          const uint64_t* __restrict__ n_dev, uint32_t n_items,
                                                          bool pack, uint16_t* __restrict__ masks,
                                                          uint32_t* __restrict__ ranges, uint32_t* st_count,
-                                                         uint32_t* __restrict__ st_beg, uint32_t* __restrict__ st_end) {
+                                                         uint32_t* __restrict__ st_beg, uint32_t* __restrict__ st_end,
+                                                         const unsigned* __restrict__ gave_up) {
+    if (*gave_up != 0) return;  // the pairs are not what the sort was to leave: every list stays empty
     const uint32_t Ic = pass_count(n_host, n_dev);
     const int lane = threadIdx.x & 31;
     // tile j of supertile key (global id) as a global tile index
@@ -1438,7 +1457,7 @@ __global__ void __launch_bounds__(kScanThreads) k_tile_scan(const __grid_constan
 // histograms, tickets, counts), the look-back status words (cleared by
 // k_keys), and the pair key/value double buffers.
 struct Layout {
-    size_t dk0, dk1, dv0, dv1, hdr, hist, tickets, total, ctotal, hdr_bytes, status, status_bytes, tk0, tk1, tv0,
+    size_t dk0, dk1, dv0, dv1, hdr, hist, tickets, total, ctotal, gave_up, hdr_bytes, status, status_bytes, tk0, tk1, tv0,
         tv1, total_bytes;
 };
 
@@ -1458,8 +1477,9 @@ Layout make_layout(int n, int64_t capacity) {
     L.hdr = o;
     L.hist = take(4 * 256 * kMaxPasses);
     L.tickets = take(4 * (kMaxPasses + 1));
-    L.total = take(16);  // instances, then supertile pairs (k_dup_coarse)
+    L.total = take(24);  // instances, then supertile pairs (the duplication), then the give-up flag
     L.ctotal = L.total + 8;
+    L.gave_up = L.total + 16;
     L.hdr_bytes = o - L.hdr;
     // status words: 256 per radix tile (the largest tile count of either sort)
     // plus one per duplication tile
@@ -1529,7 +1549,9 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     unsigned long long* status = reinterpret_cast<unsigned long long*>(base + L.status);
     const int64_t radix_status_words = (int64_t)(L.status_bytes / 8) - cdiv(n, kDupTile);
     unsigned long long* dup_status = status + radix_status_words;
-    const PassScratch ps{hist, tickets, status, err};
+    unsigned* gave_up = reinterpret_cast<unsigned*>(base + L.gave_up);
+    const GiveUp gu{err, gave_up};
+    const PassScratch ps{hist, tickets, status, gu};
 
     // supertiles of every view
     SortViews sv2 = sv;
@@ -1595,11 +1617,11 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     if (tight)
         k_dup_coarse<<<(int)std::min<int64_t>(cdiv(n, kDupTile), kDupBlocks * (int64_t)dev_sms), kThreads, 0, s>>>(
             n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
-            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, err);
+            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, gu);
     else
         k_dup_rect<<<(int)std::min<int64_t>(cdiv(n, kRectTile), 6 * (int64_t)dev_sms), kThreads, 0, s>>>(
             n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
-            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, err);
+            hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, gu);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: duplicate");
     if ((e = record_kernel_event(GS_KERNEL_DUPLICATE, true, s)) != cudaSuccess)
@@ -1608,7 +1630,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     // synchronising mode: the instance and pair counts, before any further work
     uint32_t I_grid = 0;  // pairs the later kernels are sized for
     if (!graph) {
-        uint64_t counts[2] = {0, 0};  // instances, supertile pairs (adjacent in the header)
+        uint64_t counts[3] = {0, 0, 0};  // instances, supertile pairs, give-up flag (adjacent in the header)
         if ((e = cudaMemcpyAsync(counts, total, sizeof(counts), cudaMemcpyDeviceToHost, s)) != cudaSuccess)
             return cuda_status(e, "gs_bin_sort: read count");
         if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return cuda_status(e, "gs_bin_sort: synchronize");
@@ -1618,7 +1640,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
                       (long long)capacity);
             return GS_ERR_CAPACITY;
         }
-        if (counts[0] == 0) return GS_OK;  // k_keys cleared the ranges
+        if (counts[0] == 0 || counts[2] != 0) return GS_OK;  // k_keys cleared the ranges
         I_grid = (uint32_t)counts[1];
         if ((e = cudaMemsetAsync(status, 0, 8 * 256 * (size_t)radix_tiles_max(I_grid), s)) != cudaSuccess)
             return cuda_status(e, "gs_bin_sort: clear pair-sort status");
@@ -1644,7 +1666,7 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
     pair_masks<<<(int)std::min<int64_t>(pair_grid, cdiv(I_grid, (int64_t)kPairBatch * (kThreads / 32))), kThreads, 0,
                  s>>>(
         sv2, mean2d, radius, ck[which], cv[which], I_grid, ctotal, (uint32_t)n, pack, masks, tile_ranges, st_count,
-        st_beg, st_end);
+        st_beg, st_end, gave_up);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: tile counts");
     k_tile_scan<<<1, kScanThreads, 0, s>>>(sv2, ntiles, tile_ranges, (uint64_t)capacity, fine_total,
