@@ -353,10 +353,9 @@ def blend_roofline(kind, variant, t_ms, evals, issued, pixels, peaks):
     if tc and tf and flops_pair > 0:
         tpeak = tf * 1e12 * (2.0 if variant == "fp8_split" else 1.0)
         terms["tensor"] = {"per_s": tpeak / flops_pair,
-                           "note": f"{flops_pair:.1f} MMA FLOPs per evaluated pair at {tpeak / 1e12:.0f} TFLOP/s "
-                                   f"(measured bf16{' x 2, e4m3 nominal ratio' if variant == 'fp8_split' else ''})",
-                           "achieved_tflops": round(flops_pair * achieved / 1e12, 2),
-                           "frac": round(flops_pair * achieved / tpeak, 4)}
+                           "note": f"at most {flops_pair:.1f} MMA FLOPs per evaluated pair (list entries that reach no "
+                                   f"pixel of the tile are counted, not contracted) at {tpeak / 1e12:.0f} TFLOP/s "
+                                   f"(measured bf16{' x 2, e4m3 nominal ratio' if variant == 'fp8_split' else ''})"}
     bound = min(terms, key=lambda k: terms[k]["per_s"])
     for v in terms.values():
         v["per_s"] = round(v["per_s"] / 1e9, 1)  # G evals/s
@@ -562,7 +561,7 @@ def run_ours(args):
     assert gs.gs_sync_status() == gs.GS_OK
     eager_ms = statistics.mean(e[0].elapsed_time(e[4]) for e in e_ev)
 
-    # ---- issued pairs: the chunks the tensor-core forward evaluates before a tile's exit
+    # ---- issued pairs: the list entries the tensor-core forward goes through before a tile's exit
     issued_fwd = evals_fwd
     if args.variant != "fp32":
         cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
@@ -713,9 +712,10 @@ def run_ours(args):
         **({"workload_1280x720": sweep_c1} if sweep_c1 else {}),
         "forward_pairs": {"evaluated_per_frame": evals_fwd, "issued_per_frame": issued_fwd,
                           "backward_issued_per_frame": issued_bwd,
-                          "note": "evaluated = sum of n_contrib (the metric's pairs); issued = 256 x the splats of "
-                                  "every chunk the forward evaluates before a tile's exit, entries that reach no "
-                                  "pixel of the tile left out; backward: an upper bound that counts them"},
+                          "note": "evaluated = sum of n_contrib (the metric's pairs); issued = 256 x the list "
+                                  "entries up to the end of every chunk the forward evaluates before a tile's exit; "
+                                  "backward: 256 x those up to the tile's largest n_contrib, in chunks; both count "
+                                  "entries that reach no pixel of the tile, which are not contracted"},
         **({"projection_backward": pb_line} if pb_line else {}),
         **({"small_scene_fused": small_line} if small_line else {}),
         **({"batched_views": batched_line} if batched_line else {}),

@@ -120,11 +120,12 @@ typedef struct gs_blend_opts {
                                    entry per tile of the call; an entry >= the tile count is clamped
                                    (a wrong image, never an access outside the tile ranges) */
     uint64_t* issued_pairs;     /* NULL, or a DEVICE counter the tensor-core forward adds its issued
-                                   Gaussian-pixel pairs to: 256 x the list entries it takes before a
-                                   tile's exit (every pixel stopped), whether or not a pixel still
-                                   needs them, and whether or not an entry reaches the tile; the
-                                   evaluated pairs of Eq. 1 are the sum of n_contrib.  The caller
-                                   zeroes it */
+                                   Gaussian-pixel pairs to: 256 x the list entries up to the end of
+                                   every chunk it evaluates before a tile's exit (every pixel
+                                   stopped), whether or not a pixel still needs them; entries that
+                                   reach no pixel of the tile are counted where they stand, though
+                                   they are left out of the chunks.  The evaluated pairs of Eq. 1
+                                   are the sum of n_contrib.  The caller zeroes it */
     const float* splat_records; /* NULL, or a DEVICE table from gs_pack_splats over the call's items
                                    (the same mean2d, conic, opacity, rgb), 16-byte aligned: the
                                    tensor-core kernels then stage each chunk's splat records into

@@ -531,13 +531,14 @@ struct StageHdr {
     int n;
     int slot;  // queue position of the tile (gs_tile_power output row)
     float xc, yc;  // the upper half's reference pixel
-    int pad;
+    int upto;      // list entries up to the chunk's end; 0: up to its last splat
 };
-
 
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
-template <int V, int CH, int SS, bool DUMP>
+// COUNT: adds to *a.issued (a kernel of its own: counting in the row builder cost the
+// calls that do not ask for it 1 to 2%)
+template <int V, int CH, int SS, bool DUMP, bool COUNT>
 __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
     using TR = Traits<V>;
     using LY = Layout<SS, CH, V>;
@@ -988,11 +989,14 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             // chunk, so that its pixels are written
             if (fill > 0 || sent == 0) {
                 if (!open && !acquire()) break;
-                publish(StageHdr{tile, seq, sent, fill, q, xc, yc, 0});
+                publish(StageHdr{tile, seq, sent, fill, q, xc, yc, len});
+            } else if constexpr (COUNT) {
+                // issued pairs: the entries after the last chunk, none of them kept (the
+                // row builder counts the others)
+                const int upto = (int)sRaw[(k - 1) % kRawSlots * (kRawFields * CH) + 9 * CH + CH - 1];
+                if (gi == ng && lane == 0 && sDoneRing[seq % kDoneRing] < kEpiWarps)
+                    atomicAdd(a.issued, 256ull * (unsigned long long)(len - upto));
             }
-            // issued pairs: 256 for every list entry taken, kept or not
-            if (!DUMP && a.issued != nullptr && lane == 0 && gi > 0)
-                atomicAdd(a.issued, 256ull * (unsigned long long)min(len, gi * kGroup));
         }
         // copies still in flight land before the block leaves
         for (int r = 0; r < kRecSlots; ++r)
@@ -1005,6 +1009,9 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
         const float bx0 = origin ? -15.0f : -7.5f, bx1 = origin ? 0.0f : 7.5f;
         const float by0 = origin ? -7.0f : -3.5f, by1 = origin ? 0.0f : 3.5f;
         int k = 0;
+        // issued pairs: every list entry up to the end of each chunk that is evaluated
+        [[maybe_unused]] uint32_t issued = 0;
+        [[maybe_unused]] int upto = 0;
         for (int kr = 0;; ++kr) {
             const int s = k % SS, rs = kr % kRawSlots;
             if (!mbar_wait_bounded(bar_rfull(rs), (uint32_t)(kr / kRawSlots) & 1u, tmo, sAbort) ||
@@ -1104,10 +1111,18 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                 }
             }
             __syncwarp();
+            if constexpr (COUNT)
+                if (hd.n >= 0) {  // (only this warp writes the stage)
+                    const int to = hd.upto > 0 || hd.n == 0 ? hd.upto : (int)sIdx[s * CH + hd.n - 1];
+                    issued += (uint32_t)(to - (hd.base > 0 ? upto : 0));
+                    upto = to;
+                }
             ++k;
             if (hd.n < 0) break;
         }
         if (lane == 0) {
+            if constexpr (COUNT)
+                if (issued > 0) atomicAdd(a.issued, 256ull * issued);
             // every MMA this thread issued has finished before TMEM is freed (a
             // fresh barrier: no phase of another stage can be mistaken for it)
             tc_commit(bar_drain);
@@ -1124,11 +1139,13 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
 
 // Persistent grid: as many CTAs as fit on the GPU at once, from the kernel's
 // registers, shared memory and threads and the SM's 512 TMEM columns.
-template <int V, int CH, int SS, bool DUMP>
+template <int V, int CH, int SS, bool DUMP, bool COUNT = false>
 cudaError_t launch_inst(const BlendArgs& a, int items, cudaStream_t s) {
+    if constexpr (!DUMP && !COUNT)
+        if (a.issued != nullptr) return launch_inst<V, CH, SS, DUMP, true>(a, items, s);
     using LY = Layout<SS, CH, V>;
     constexpr int bytes = LY::BYTES;
-    auto kern = k_blend_tc<V, CH, SS, DUMP>;
+    auto kern = k_blend_tc<V, CH, SS, DUMP, COUNT>;
     static std::mutex mu;
     static LaunchShape cache;
     LaunchShape sh;
