@@ -1,19 +1,28 @@
 // Preprocessing stage (Sec. 2.1 (a)): EWA projection of 3D Gaussians, one
 // thread per Gaussian.  FP32 throughout; the 2D covariance and its inverse are
 // recomputed in FP64 when the FP32 determinant is below 1e-6.
+#include <algorithm>
+
 #include "project.cuh"
 
 namespace gs {
 namespace {
 
-// Block b: view b % views, the (b / views)-th 128 Gaussians, so that the views
-// of the same Gaussians run together and their inputs come from HBM once (16
-// views of 1.5M: 1.24 GB -> 78 MB read); outputs of view v, Gaussian g at index
-// v * n + g.  Bound by the latency of a chain of loads (means, then shape, then
-// the coefficients of what is visible), so by resident warps: 64 registers and
-// small blocks.  3M Gaussians, degree 3, one view 146 -> 127 us (663 MB, 5.2
-// TB/s); 16 views of 1.5M, degree 0 565 -> 519 us.
+// Blocks run chunk by chunk of Gaussians (grid z), within a chunk view by view (y),
+// so that a chunk's inputs come from HBM once and its other views read them from
+// L2; outputs of view v, Gaussian g at index v * n + g.  How many blocks a chunk
+// has is a matter of what moves.  Degrees 0 and 1 write nearly as much as they
+// read, and every view's outputs are streams of their own: whole waves per view
+// (1024 blocks, 131072 Gaussians).  Degrees 2 and 3 are bound by the coefficients,
+// which 16 blocks keep closest.  Degree 0, 16 views of 300k / 1.5M: view by view
+// over all Gaussians 74 / 567 us, views innermost (chunks of one block) 107 / 514,
+// in chunks of 1024 74 / 340; degree 3, 16 views of 1.5M: 1124, 747, 787, in
+// chunks of 16 748 (5 views of 3M 710, 514, 524, 500).
+// Bound by the latency of a chain of loads (means, then shape, then the
+// coefficients of what is visible), so by resident warps: 64 registers and small
+// blocks.  3M Gaussians, degree 3, one view 146 -> 127 us (663 MB, 5.2 TB/s).
 constexpr int kProjThreads = 128;
+constexpr unsigned chunk_blocks(int sh_degree) { return sh_degree <= 1 ? 1024 : 16; }
 template <int SH_DEGREE, bool VEC16>
 __global__ void __launch_bounds__(kProjThreads, 8) k_project(int n, const float* __restrict__ means,
                                                  const float* __restrict__ scales, const float* __restrict__ quats,
@@ -22,9 +31,9 @@ __global__ void __launch_bounds__(kProjThreads, 8) k_project(int n, const float*
                                                  float2* __restrict__ mean2d_all, float* __restrict__ conic_all,
                                                  float* __restrict__ depth_all, int* __restrict__ radius_all,
                                                  float* __restrict__ rgb_all, uint32_t* __restrict__ touched_all) {
-    const int v = blockIdx.x % views.num_views, g = blockIdx.x / views.num_views * kProjThreads + threadIdx.x;
-    if (g >= n) return;
-    project_gaussian<SH_DEGREE, VEC16>(g, means, scales, quats, sh, views.cams[v], (size_t)v * n,
+    const unsigned g = (blockIdx.z * gridDim.x + blockIdx.x) * kProjThreads + threadIdx.x, v = blockIdx.y;
+    if (g >= (unsigned)n) return;
+    project_gaussian<SH_DEGREE, VEC16>((int)g, means, scales, quats, sh, views.cams[v], (size_t)v * n,
                                        mean2d_all, conic_all, depth_all, radius_all, rgb_all, touched_all);
 }
 
@@ -34,7 +43,11 @@ cudaError_t launch_project(int n, const float* means, const float* scales, const
                            int sh_degree, const CamViews& cams, float* mean2d, float* conic, float* depth,
                            int* radius, float* rgb, uint32_t* tiles_touched, cudaStream_t s) {
     const int block = kProjThreads;
-    const unsigned grid = (unsigned)((n + block - 1) / block) * (unsigned)cams.num_views;
+    const unsigned nblk = ((unsigned)n + block - 1) / block;
+    // (at most 65535 chunks; blocks split evenly, the last chunk may be a few short)
+    const unsigned chunk = std::max(chunk_blocks(sh_degree), (nblk + 65534) / 65535);
+    const unsigned chunks = (nblk + chunk - 1) / chunk;
+    const dim3 grid((nblk + chunks - 1) / chunks, cams.num_views, chunks);
     // 16-byte coefficient loads for degrees 1 and 3 (3K a multiple of 4) on an aligned array
     const bool vec = (reinterpret_cast<uintptr_t>(sh) & 15) == 0;
     switch (sh_degree) {
