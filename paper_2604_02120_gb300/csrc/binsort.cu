@@ -907,22 +907,27 @@ __global__ void __launch_bounds__(kThreads, kDupBlocks)
 }
 
 // The same for full rectangles.  An item's supertiles are then a rectangle too,
-// so nothing is evaluated per row: persistent blocks take tiles of kRectTile
-// depth-ordered items from the ticket (four consecutive items per thread),
+// so nothing is evaluated per row: persistent blocks take tiles of 256 ITEMS
+// depth-ordered items from the ticket (ITEMS consecutive ones per thread),
 // scan their supertile counts, publish the sum, look back, and write the
 // tile's pairs with consecutive threads on consecutive pairs; a thread finds
 // its pair's item by a search over the items' first pairs and the supertile,
 // key and 16-bit tile mask from the rectangle.  The digit histograms stay in
 // shared memory over all tiles of a block.  It waits for its barriers and the
-// chain ticket, items, gather, look-back per tile (51% of the issue slots at 6
+// chain ticket, items, gather, look-back per tile (48% of the issue slots at 6
 // blocks per SM; 4 and 8 blocks, a look-back window of 128 tiles and fetching
 // the next tile's items ahead were all slower).  Against the per-row kernel
 // above, which full rectangles used to go through: 16 views of 1.5M splats 2.85
 // -> 0.87 ms; 1920 x 1080, 1M 128 -> 34 us; 1280 x 720, 200k 43 -> 18 us.
 // Counts beyond 32 bits: the starts saturate (no pair past the
 // capacity, below 2^32, is written).
-constexpr int kRectItems = 4;
-constexpr int kRectTile = kThreads * kRectItems;
+// Items per thread: four (half the look-back; 1M small splats, the whole sort 194 us,
+// with one 216) where that leaves tiles for most SMs, one up to 2^16 items, where
+// large rectangles would otherwise be the work of a few blocks: 2000 splats of
+// 20000 tiles each 2.79 -> 0.83 ms, 20k of 2500 each 0.54 -> 0.27; small splats
+// take the same time either way (100k: 89 and 91 us).
+inline int rect_items(int64_t n) { return n <= 1 << 16 ? 1 : 4; }
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uint32_t* __restrict__ perm,
                                                           const __grid_constant__ SortViews sv,
                                                           const float2* __restrict__ mean2d,
@@ -934,15 +939,16 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
                                                           unsigned long long* __restrict__ radix_status,
                                                           uint32_t coarse_tile, uint32_t* __restrict__ st_zero,
                                                           int st_n, GiveUp gu) {
+    constexpr int TILE = kThreads * ITEMS;
     __shared__ uint64_t s_warp[kThreads / 32 + 1];
     __shared__ uint64_t s_prefix;
     __shared__ unsigned long long s_fine;
     __shared__ uint32_t s_tile;
     __shared__ uint32_t s_h[4 * 256];
-    __shared__ uint32_t s_start[kRectTile];  // each item's first pair within the tile
-    __shared__ uint2 s_rect[kRectTile];      // x0 | x1 << 16, y0 | y1 << 16 in tiles
-    __shared__ uint32_t s_item[kRectTile];
-    __shared__ uint8_t s_view[kRectTile];
+    __shared__ uint32_t s_start[TILE];  // each item's first pair within the tile
+    __shared__ uint2 s_rect[TILE];      // x0 | x1 << 16, y0 | y1 << 16 in tiles
+    __shared__ uint32_t s_item[TILE];
+    __shared__ uint8_t s_view[TILE];
     if (st_zero != nullptr)  // the supertile counters of k_pair_masks
         for (int i = blockIdx.x * kThreads + threadIdx.x; i < st_n; i += gridDim.x * kThreads) st_zero[i] = 0;
     for (int i = threadIdx.x; i < passes * 256; i += kThreads) s_h[i] = 0;
@@ -952,40 +958,39 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
         if (threadIdx.x == 0) s_tile = atomicAdd(&tickets[kMaxPasses], 1u);
         __syncthreads();  // (also: the last tile's pairs have left shared memory)
         const uint32_t tile = s_tile;
-        const int64_t base = (int64_t)tile * kRectTile;
+        const int64_t base = (int64_t)tile * TILE;
         if (base >= n_items) break;
-        uint32_t item[kRectItems];
-        float2 m[kRectItems];
-        int r[kRectItems];
-        const int64_t k0 = base + (int64_t)threadIdx.x * kRectItems;
-        if (k0 + kRectItems <= n_items) {
+        uint32_t item[ITEMS];
+        float2 m[ITEMS];
+        int r[ITEMS];
+        const int64_t k0 = base + (int64_t)threadIdx.x * ITEMS;
+        if (ITEMS == 4 && k0 + ITEMS <= n_items) {
             const uint4 q = *reinterpret_cast<const uint4*>(perm + k0);  // k0 is a multiple of 4, perm 256-byte aligned
-            item[0] = q.x;
-            item[1] = q.y;
-            item[2] = q.z;
-            item[3] = q.w;
+            const uint32_t qi[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int i = 0; i < ITEMS; ++i) item[i] = qi[i];
         } else {
 #pragma unroll
-            for (int i = 0; i < kRectItems; ++i) item[i] = k0 + i < n_items ? perm[k0 + i] : 0xffffffffu;
+            for (int i = 0; i < ITEMS; ++i) item[i] = k0 + i < n_items ? perm[k0 + i] : 0xffffffffu;
         }
 #pragma unroll
-        for (int i = 0; i < kRectItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const bool ok = item[i] < (uint32_t)n_items;  // always, unless a look-back gave up (timeout bit set)
             r[i] = ok ? radius[item[i]] : 0;
             m[i] = ok ? mean2d[item[i]] : make_float2(0.f, 0.f);
         }
-        uint32_t c[kRectItems];
+        uint32_t c[ITEMS];
         uint64_t sum = 0;
         unsigned long long fine = 0;
 #pragma unroll
-        for (int i = 0; i < kRectItems; ++i) {
+        for (int i = 0; i < ITEMS; ++i) {
             const int v = item[i] < (uint32_t)n_items ? (int)(item[i] / (uint32_t)sv.n_per_view) : 0;
             int x0, x1, y0, y1;
             c[i] = 0;
             if (tile_rect(m[i].x, m[i].y, r[i], sv.views[v].W, sv.views[v].H, x0, x1, y0, y1)) {
                 c[i] = (uint32_t)(x1 / kSuper - x0 / kSuper + 1) * (uint32_t)(y1 / kSuper - y0 / kSuper + 1);
                 fine += (unsigned long long)(x1 - x0 + 1) * (unsigned long long)(y1 - y0 + 1);
-                const int at = threadIdx.x * kRectItems + i;
+                const int at = threadIdx.x * ITEMS + i;
                 s_rect[at] = make_uint2((uint32_t)x0 | ((uint32_t)x1 << 16), (uint32_t)y0 | ((uint32_t)y1 << 16));
                 s_item[at] = item[i];
                 s_view[at] = (uint8_t)v;
@@ -999,8 +1004,8 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
         uint64_t at = block_excl_scan<uint64_t, kThreads>(sum, tile_sum, s_warp);
         if (threadIdx.x == 0) st_status(status + tile, tile == 0 ? 2u : 1u, tile_sum);
 #pragma unroll
-        for (int i = 0; i < kRectItems; ++i) {
-            s_start[threadIdx.x * kRectItems + i] = (uint32_t)min(at, (uint64_t)0xffffffffu);
+        for (int i = 0; i < ITEMS; ++i) {
+            s_start[threadIdx.x * ITEMS + i] = (uint32_t)min(at, (uint64_t)0xffffffffu);
             at += c[i];
         }
         if (warp == 0) {
@@ -1011,7 +1016,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
             }
             if (lane == 0) {
                 s_prefix = prefix;
-                if (base + kRectTile >= n_items) *total = prefix + tile_sum;  // the last tile: the total
+                if (base + TILE >= n_items) *total = prefix + tile_sum;  // the last tile: the total
             }
         }
         __syncthreads();
@@ -1027,7 +1032,7 @@ __global__ void __launch_bounds__(kThreads, 6) k_dup_rect(int n_items, const uin
             // the last item whose first pair is at or before p
             int i = 0;
 #pragma unroll
-            for (int d = kRectTile / 2; d > 0; d >>= 1)
+            for (int d = TILE / 2; d > 0; d >>= 1)
                 if (s_start[i + d] <= p) i += d;
             const uint2 q = s_rect[i];
             const int v = s_view[i];
@@ -1618,10 +1623,12 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
         k_dup_coarse<<<(int)std::min<int64_t>(cdiv(n, kDupTile), kDupBlocks * (int64_t)dev_sms), kThreads, 0, s>>>(
             n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
             hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, gu);
-    else
-        k_dup_rect<<<(int)std::min<int64_t>(cdiv(n, kRectTile), 6 * (int64_t)dev_sms), kThreads, 0, s>>>(
+    else {
+        auto dup_rect = rect_items(n) == 1 ? k_dup_rect<1> : k_dup_rect<4>;
+        dup_rect<<<(int)std::min<int64_t>(cdiv(n, kThreads * rect_items(n)), 6 * (int64_t)dev_sms), kThreads, 0, s>>>(
             n, perm, sv2, mean2d, radius, (uint64_t)capacity, st_passes, pack, tickets, dup_status, ck[0], cv[0],
             hist + 256 * 4, ctotal, fine_total, status, coarse_tile, st_count, nst, gu);
+    }
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: duplicate");
     if ((e = record_kernel_event(GS_KERNEL_DUPLICATE, true, s)) != cudaSuccess)
