@@ -37,6 +37,7 @@
 //   memset, keys, 4 depth passes, coarse duplicate, ceil(bits / 8) supertile
 //   passes, tile counts, tile scan, fine write.
 #include <algorithm>
+#include <type_traits>
 
 #include "internal.h"
 #include "tight.cuh"
@@ -1264,10 +1265,14 @@ __global__ void __launch_bounds__(kThreads) k_pair_masks(const __grid_constant__
 // all pairs of a round: 1280 x 720, 200k, full rectangles with keys 114 -> 44
 // us; 1920 x 1080, 1M 252 -> 93; opacity-aware lists at 3840 x 2160, 139M
 // instances, no keys 225 -> 206 (2.7 TB/s of ids); 16 views 563 -> 524 us.
-constexpr int kFineThreads = 512;
-constexpr int kFineWarps = kFineThreads / 32;
-template <bool KEYS>
-__global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ SortViews sv,
+// With more supertiles than items (no counts or ends then) most blocks find a pair or
+// none, so a block is half as large: 20k items on 20000 x 20000 pixels 1.70 -> 1.38 ms
+// for the whole sort (four warps 1.23), but 15k items on one supertile of 8000 x 8000
+// 276 -> 298 us (four warps 348).
+constexpr int kFineWarps = 16;
+constexpr int kFineSparseWarps = 8;
+template <bool KEYS, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) k_fine(const __grid_constant__ SortViews sv,
                                                        const float* __restrict__ depth,
                                                        const uint32_t* __restrict__ ckey,
                                                        const uint32_t* __restrict__ cval, uint32_t n_host,
@@ -1279,11 +1284,13 @@ __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ S
                                                        const uint32_t* __restrict__ st_beg,
                                                        const uint32_t* __restrict__ st_end, uint32_t n_items,
                                                        uint32_t* __restrict__ ids_out, uint64_t* __restrict__ keys_out) {
+    constexpr int THREADS = 32 * WARPS;
     __shared__ uint32_t s_rng[2];
     __shared__ uint32_t s_beg[16], s_len[16];
     // instances per round (double-buffered), tile and warp, one byte each (<= 32)
-    __shared__ uint4 s_cnt[2][16];
-    static_assert(kFineWarps == 16, "16 warps' bytes make the 16 bytes of a tile");
+    static_assert(WARPS == 8 || WARPS == 16, "the warps' bytes make two words of a tile or four");
+    using Counts = std::conditional_t<WARPS == 16, uint4, uint2>;
+    __shared__ Counts s_cnt[2][16];
     const int s = st_order != nullptr ? (int)st_order[blockIdx.x] : (int)blockIdx.x;  // largest first
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned lt = (1u << lane) - 1u;
@@ -1330,10 +1337,10 @@ __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ S
         fetch(e);
     };
     fetch(cs + threadIdx.x);
-    advance(cs + kFineThreads + threadIdx.x);
-    for (uint32_t r0 = cs, round = 0; r0 < ce; r0 += kFineThreads, round ^= 1u) {
+    advance(cs + THREADS + threadIdx.x);
+    for (uint32_t r0 = cs, round = 0; r0 < ce; r0 += THREADS, round ^= 1u) {
         const uint32_t m = mk, id = it, dep = dp;
-        advance(r0 + 2 * kFineThreads + threadIdx.x);
+        advance(r0 + 2 * THREADS + threadIdx.x);
         // lane t: the warp's instances of tile t in this round, from four lane reductions of
         // the masks' bits spread to bytes
         uint32_t cnt = 0;
@@ -1345,16 +1352,23 @@ __global__ void __launch_bounds__(kFineThreads) k_fine(const __grid_constant__ S
         }
         if (lane < 16) reinterpret_cast<uint8_t*>(&s_cnt[round][lane])[warp] = (uint8_t)cnt;
         __syncthreads();  // (a warp two rounds ahead has passed the next barrier: two tables suffice)
-        const uint4 c4 = s_cnt[round][tl];
         // where the warp's instances of tile t start: after those of the lower warps
         const uint32_t lo = 0xFFFFFFFFu >> (31 - 8 * (warp & 3)) >> 1;  // the bytes of the lower warps in this warp's word
-        const int wq = warp >> 2;
         uint32_t off = run;
-        off = __dp4a(wq > 0 ? c4.x : c4.x & lo, 0x01010101u, off);
-        off = __dp4a(wq > 1 ? c4.y : wq == 1 ? c4.y & lo : 0u, 0x01010101u, off);
-        off = __dp4a(wq > 2 ? c4.z : wq == 2 ? c4.z & lo : 0u, 0x01010101u, off);
-        off = __dp4a(wq == 3 ? c4.w & lo : 0u, 0x01010101u, off);
-        run = __dp4a(c4.x, 0x01010101u, __dp4a(c4.y, 0x01010101u, __dp4a(c4.z, 0x01010101u, __dp4a(c4.w, 0x01010101u, run))));
+        if constexpr (WARPS == 16) {
+            const uint4 c4 = s_cnt[round][tl];
+            const int wq = warp >> 2;
+            off = __dp4a(wq > 0 ? c4.x : c4.x & lo, 0x01010101u, off);
+            off = __dp4a(wq > 1 ? c4.y : wq == 1 ? c4.y & lo : 0u, 0x01010101u, off);
+            off = __dp4a(wq > 2 ? c4.z : wq == 2 ? c4.z & lo : 0u, 0x01010101u, off);
+            off = __dp4a(wq == 3 ? c4.w & lo : 0u, 0x01010101u, off);
+            run = __dp4a(c4.x, 0x01010101u, __dp4a(c4.y, 0x01010101u, __dp4a(c4.z, 0x01010101u, __dp4a(c4.w, 0x01010101u, run))));
+        } else {
+            const uint2 c2 = s_cnt[round][tl];
+            off = __dp4a(warp < 4 ? c2.x & lo : c2.x, 0x01010101u, off);
+            off = __dp4a(warp < 4 ? 0u : c2.y & lo, 0x01010101u, off);
+            run = __dp4a(c2.x, 0x01010101u, __dp4a(c2.y, 0x01010101u, run));
+        }
         // whole unless the lists are cut off at the capacity
         const bool whole = __all_sync(0xffffffffu, off + cnt <= len);
         const uint32_t place = beg + off;
@@ -1680,8 +1694,10 @@ gs_status bin_sort_run(const SortViews& sv, const float* mean2d_f, const int* ra
                                            graph ? n_instances_dev : nullptr, st_count, st_order, err);
     count_launches();
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_status(e, "gs_bin_sort: tile ranges");
-    auto fine = keys_sorted != nullptr ? k_fine<true> : k_fine<false>;
-    fine<<<nst, kFineThreads, 0, s>>>(sv2, depth, ck[which], cv[which], I_grid, ctotal, pack ? 0xFFFFu : 0xFFFFFFFFu,
+    const bool sparse = st_count == nullptr;
+    auto fine = keys_sorted != nullptr ? (sparse ? k_fine<true, kFineSparseWarps> : k_fine<true, kFineWarps>)
+                                       : (sparse ? k_fine<false, kFineSparseWarps> : k_fine<false, kFineWarps>);
+    fine<<<nst, 32 * (sparse ? kFineSparseWarps : kFineWarps), 0, s>>>(sv2, depth, ck[which], cv[which], I_grid, ctotal, pack ? 0xFFFFu : 0xFFFFFFFFu,
                                       masks, tile_ranges, st_order, st_count, st_beg, st_end, (uint32_t)n, ids_sorted,
                                       keys_sorted);
     count_launches();
