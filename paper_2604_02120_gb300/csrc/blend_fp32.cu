@@ -11,8 +11,8 @@
 // list order and with their list positions: the same decisions and the same
 // values as the walk over all.  Forward and backward against the walk over all:
 // full rectangles, 641 x 479, 50k splats 105 -> 60 us and 217 -> 152 us; 1920 x
-// 1080, 1M clustered 995 -> 410 us and 2209 -> 1256 us; opacity-aware lists there
-// 379 -> 321 us and 1228 -> 1101 us; 1280 x 720, 200k 99 -> 86 us and 281 -> 262 us.
+// 1080, 1M clustered 1072 -> 445 us and 2315 -> 1321 us; opacity-aware lists there
+// 418 -> 350 us and 1304 -> 1166 us; 1280 x 720, 200k 110 -> 93 us and 305 -> 281 us.
 #include "blend_tc.cuh"
 #include "internal.h"
 
@@ -27,7 +27,7 @@ constexpr float kTMin = 1e-4f;
 struct SplatSm {
     float4 geo;  // mx, my, A, B
     float4 oc;   // C, o, r, g
-    float2 bl;   // b, log2 o
+    float b;
 };
 
 // alpha of a splat at a pixel; `e` receives exp(min(power, 0)) and `pw` power.
@@ -47,7 +47,7 @@ __device__ __forceinline__ void load_splat(const BlendArgs& a, uint32_t g, uint3
     const float2 m = a.mean2d[g];
     s.geo = make_float4(m.x, m.y, a.conic[3 * g], a.conic[3 * g + 1]);
     s.oc = make_float4(a.conic[3 * g + 2], a.opac[g - opac_off], a.rgb[3 * g], a.rgb[3 * g + 1]);
-    s.bl = make_float2(a.rgb[3 * g + 2], __log2f(s.oc.y));
+    s.b = a.rgb[3 * g + 2];
 }
 
 // Whether the splat may reach alpha >= 1/255 at a pixel of the warp's 8 x 4
@@ -63,8 +63,12 @@ __device__ __forceinline__ bool warp_reaches(const float4& geo, const float4& oc
 // A batch whose first 32 splats include four in five that the warp needs is walked
 // whole, by the plain loop: it costs less per splat than one over set bits, and
 // what the tests would spare there does not pay for them.  Opacity-aware lists of
-// large splats (3840 x 2160, 3M, heavy tails), forward / backward: without any
-// test 636 / 2266 us, with this rule 660 / 2317, with every group tested 793 / 2482.
+// large splats (3840 x 2160, 3M, heavy tails: 95% needed, a warp walks 54), forward /
+// backward: without any test 636 / 2263 us, with this rule 627 / 2315, with every
+// group tested 793 / 2482.  (The forward holds nothing of the test's over the walk
+// and takes two splats per turn; with both staged and held it took 662.  What the
+// backward loses is the second loop's place in the code: a kernel of the plain loop
+// alone takes 2245, tests by a cheaper bound or one loop for both were slower.)
 __device__ __forceinline__ bool dense_group(unsigned hits, int n) { return 5 * __popc(hits) >= 4 * n; }
 
 // Geometry of the block's tile (blockIdx.x is a global tile id).
@@ -96,13 +100,12 @@ __device__ __forceinline__ TileGeo tile_geo(const BlendArgs& a, int tile) {
 __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant__ BlendArgs a) {
     __shared__ float4 s_geo[kBatch];
     __shared__ float4 s_oc[kBatch];
-    __shared__ float2 s_bl[kBatch];
+    __shared__ float s_b[kBatch];
     const int tile = tile_at(a, blockIdx.x * a.shard_count + a.shard_index);
     const TileGeo tg = tile_geo(a, tile);
     const int px = tg.px, py = tg.py;
     const bool inside = px < tg.W && py < tg.H;
     const float xp = px + 0.5f, yp = py + 0.5f;
-    const int lane = threadIdx.x & 31;
     const uint32_t start = a.ranges[2 * tile], end = a.ranges[2 * tile + 1];
     const int len = end > start ? (int)(end - start) : 0;
 
@@ -117,7 +120,7 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
             load_splat(a, a.ids[start + i], tg.opac_off, s);
             s_geo[threadIdx.x] = s.geo;
             s_oc[threadIdx.x] = s.oc;
-            s_bl[threadIdx.x] = s.bl;
+            s_b[threadIdx.x] = s.b;
         }
         __syncthreads();
         const int nb = min(kBatch, len - base);
@@ -134,33 +137,20 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
             const float w = alpha * T;
             cr = __fmaf_rn(oc.z, w, cr);
             cg = __fmaf_rn(oc.w, w, cg);
-            cb = __fmaf_rn(s_bl[j].x, w, cb);
+            cb = __fmaf_rn(s_b[j], w, cb);
             T = tT;
             last = base + j + 1;
         };
+        // (the warp's corner and log2 o are worked out here, not held over the walk)
         auto test = [&](int c) {
-            const int t = c + lane;
-            return __ballot_sync(0xffffffffu, t < nb && warp_reaches(s_geo[t], s_oc[t], s_bl[t].y, tg.bx, tg.by));
+            const int lane = threadIdx.x & 31, t = c + lane;
+            return __ballot_sync(0xffffffffu, t < nb && warp_reaches(s_geo[t], s_oc[t], __log2f(s_oc[t].y),
+                                                                     xp - (float)(lane & 7), yp - (float)(lane >> 3)));
         };
         unsigned hits = test(0);
         if (dense_group(hits, min(32, nb))) {
-            for (int j = 0; !done && j < nb; ++j) {
-                const float4 geo = s_geo[j], oc = s_oc[j];
-                float e, pw, dx, dy;
-                const float alpha = splat_alpha(geo, oc, xp, yp, e, pw, dx, dy);
-                if (alpha < kAlphaMin) continue;
-                const float tT = T * (1.0f - alpha);
-                if (tT < kTMin) {
-                    done = true;
-                    break;
-                }
-                const float w = alpha * T;
-                cr = __fmaf_rn(oc.z, w, cr);
-                cg = __fmaf_rn(oc.w, w, cg);
-                cb = __fmaf_rn(s_bl[j].x, w, cb);
-                T = tT;
-                last = base + j + 1;
-            }
+#pragma unroll 2
+            for (int j = 0; !done && j < nb; ++j) step(j);
         } else {
             for (int c = 0;;) {
                 for (; hits; hits &= hits - 1) step(c + __ffs(hits) - 1);
@@ -268,7 +258,7 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_bwd(const __grid_constant
             load_splat(a, g, tg.opac_off, s);
             s_geo[threadIdx.x] = s.geo;
             s_oc[threadIdx.x] = s.oc;
-            s_bl[threadIdx.x] = s.bl;
+            s_bl[threadIdx.x] = make_float2(s.b, __log2f(s.oc.y));
             s_id[threadIdx.x] = g;
         }
         __syncthreads();
