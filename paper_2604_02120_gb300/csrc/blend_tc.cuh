@@ -21,7 +21,7 @@
 //    entries, copies the splats a group ahead by cp.async (or by TMA gathers
 //    of packed records), drops the entries whose alpha stays below 1/255 on
 //    the whole tile (splat_reaches) and packs the others, with their list
-//    positions, into chunks of CH raw splats, two slots ahead.
+//    positions, into chunks of CH raw splats, raw_slots ahead.
 //  - The builder turns a raw chunk into a stage of the shared-memory ring
 //    (SS stages: header, v_g rows, per-splat colour and position), issues its
 //    MMA into one of 2 TMEM stages and drops the chunks of a tile whose pixels
@@ -157,7 +157,15 @@ __device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t adesc, uint64_t
         tc_mma_f16(d_tmem, adesc, bdesc, idesc, accumulate);
 }
 
-constexpr int kRawSlots = 2;   // chunks of raw splats between the scanner and the row builders
+// Chunks of raw splats between the scanner and the row builder.  Two keep the
+// epilogue fed where most entries are dropped (one: 1920 x 1080, full lists 343 ->
+// 356 us).  The CUDA-core variant's epilogue takes longer per splat, and what the
+// scanner takes past a tile's end costs it more: one there (3840 x 2160, 3M,
+// opacity-aware lists 611 -> 597 us, full lists the same).
+template <int V>
+constexpr int raw_slots() {
+    return Traits<V>::CC ? 1 : 2;
+}
 constexpr int kRawFields = 10;  // mean x, y, conic A, B, C, log2 opacity, r, g, b, list position + 1
 constexpr int kGroup = 32;      // list entries the scanner tests at a time
 constexpr int kGeoFields = 9;   // mean (2), conic (3), opacity, colour (3)
@@ -166,6 +174,7 @@ constexpr int kRecSlots = 4;    // TMA slots of a group's records
 
 template <int SS, int CH, int V>
 struct Layout {
+    static constexpr int RAW = raw_slots<V>();
     static constexpr int A_BYTES = 128 * Traits<V>::ROW_BYTES;
     static constexpr int B_BYTES = 2 * CH * Traits<V>::ROW_BYTES;
     static constexpr int OFF_B = A_BYTES;
@@ -174,15 +183,15 @@ struct Layout {
     static constexpr int OFF_SCL = OFF_IDX + SS * CH * 4;    // FP8: row scales (float2 per splat)
     static constexpr int OFF_RAW = OFF_SCL + (Traits<V>::FP8 ? SS * CH * 8 : 0);
     static constexpr int OFF_RECT =
-        (OFF_RAW + kRawSlots * kRawFields * CH * 4 + 255) / 256 * 256;  // TMA record slots (256-aligned)
+        (OFF_RAW + RAW * kRawFields * CH * 4 + 255) / 256 * 256;  // TMA record slots (256-aligned)
     static constexpr int OFF_GEO = OFF_RECT;  // the same memory: a launch uses one or the other
     static_assert(kGeoSlots * kGeoFields * 4 <= kRecSlots * kRecBytes, "splat slots");
     static constexpr int OFF_BAR = OFF_RECT + kRecSlots * kGroup * kRecBytes;
     // full[SS], empty[SS], tfull, tempty, drain, raw full, raw empty, record slots
-    static constexpr int NBAR = 2 * SS + 2 * kTStages + 1 + 2 * kRawSlots + kRecSlots;
+    static constexpr int NBAR = 2 * SS + 2 * kTStages + 1 + 2 * RAW + kRecSlots;
     static constexpr int OFF_HDR = OFF_BAR + NBAR * 8;
     static constexpr int OFF_RAWHDR = OFF_HDR + SS * 32;
-    static constexpr int OFF_MISC = OFF_RAWHDR + kRawSlots * 32;
+    static constexpr int OFF_MISC = OFF_RAWHDR + RAW * 32;
     static constexpr int BYTES = OFF_MISC + 16 + 4 * kDoneRing;
     static constexpr uint32_t TCOLS_RAW = 2u * kTStages * CH;
     static constexpr uint32_t TCOLS = TCOLS_RAW <= 32 ? 32 : TCOLS_RAW <= 64 ? 64 : TCOLS_RAW <= 128 ? 128
@@ -542,9 +551,11 @@ template <int V, int CH, int SS, bool DUMP, bool COUNT>
 __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
     using TR = Traits<V>;
     using LY = Layout<SS, CH, V>;
-    constexpr int SBO = TR::SBO;
+    constexpr int SBO = TR::SBO, RAW = LY::RAW;
     constexpr uint32_t IDESC = idesc_f16(TR::FMT, 128, 2 * CH);
-    constexpr int EC = 4;  // accumulator columns an epilogue thread holds at a time
+    // columns an epilogue thread takes at a time (CC: of shared memory, more loads in
+    // flight; 3840 x 2160, 3M 621 -> 611 us, 1920 x 1080 465 -> 452)
+    constexpr int EC = TR::CC ? 8 : 4;
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sA = smem;
     uint8_t* sB = smem + LY::OFF_B;
@@ -564,8 +575,8 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
     auto bar_tempty = [&](int t) { return smem_u32(bars + 2 * SS + kTStages + t); };
     const uint32_t bar_drain = smem_u32(bars + 2 * SS + 2 * kTStages);
     auto bar_rfull = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + r); };
-    auto bar_rempty = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + kRawSlots + r); };
-    auto bar_rec = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + 2 * kRawSlots + r); };
+    auto bar_rempty = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + RAW + r); };
+    auto bar_rec = [&](int r) { return smem_u32(bars + 2 * SS + 2 * kTStages + 1 + 2 * RAW + r); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int n_items = a.total_tiles;  // gs_tile_power: the number of listed tiles
@@ -581,7 +592,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             mbar_init(bar_tempty(t), kEpiWarps);
         }
         mbar_init(bar_drain, 1);
-        for (int r = 0; r < kRawSlots; ++r) {
+        for (int r = 0; r < RAW; ++r) {
             mbar_init(bar_rfull(r), 1);
             mbar_init(bar_rempty(r), 1);
         }
@@ -695,7 +706,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                         p = __ffma2_rn(make_float2(a1.x, a2.z), make_float2(mp[4], mp[4]), p);
                         return __fadd2_rn(make_float2(a1.y, a2.w), p);
                     };
-                    if constexpr (!TR::CC) {
+                    if constexpr (EC == 4 && !TR::CC) {
                         tmem_ld_32x32b_x4(tb + (uint32_t)c0, vu);
                         tmem_ld_32x32b_x4(tb + (uint32_t)(CH + c0), vl);
                         tmem_ld_wait();
@@ -722,8 +733,10 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                             }
                         }
                     } else {
-                        const float4 ix4 = *reinterpret_cast<const float4*>(idx1 + c0);
-                        const float ix[EC] = {ix4.x, ix4.y, ix4.z, ix4.w};
+                        float ix[EC];
+#pragma unroll
+                        for (int q = 0; q < EC; q += 4)
+                            *reinterpret_cast<float4*>(ix + q) = *reinterpret_cast<const float4*>(idx1 + c0 + q);
 #pragma unroll
                         for (int c = 0; c < EC; ++c) {
                             float2 pw;
@@ -862,7 +875,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
         int k = 0;
         bool open = false, quit = false;
         auto acquire = [&]() -> bool {
-            if (!mbar_wait_bounded(bar_rempty(k % kRawSlots), ((uint32_t)(k / kRawSlots) & 1u) ^ 1u, tmo, sAbort)) {
+            if (!mbar_wait_bounded(bar_rempty(k % RAW), ((uint32_t)(k / RAW) & 1u) ^ 1u, tmo, sAbort)) {
                 *sAbort = 1;
                 atomicOr(a.err, kErrTimeout);
                 return false;
@@ -871,9 +884,9 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             return !*sAbort;
         };
         auto publish = [&](const StageHdr& h) {
-            if (lane == 0) sRawHdr[k % kRawSlots] = h;
+            if (lane == 0) sRawHdr[k % RAW] = h;
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar_rfull(k % kRawSlots));
+            if (lane == 0) mbar_arrive(bar_rfull(k % RAW));
             ++k;
             open = false;
         };
@@ -961,7 +974,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
                             break;
                         }
                         if (pos >= 0 && pos < CH) {
-                            float* w = sRaw + (k % kRawSlots) * (kRawFields * CH) + pos;
+                            float* w = sRaw + (k % RAW) * (kRawFields * CH) + pos;
                             w[0] = m.x;
                             w[CH] = m.y;
                             w[2 * CH] = A;
@@ -993,7 +1006,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
             } else if constexpr (COUNT) {
                 // issued pairs: the entries after the last chunk, none of them kept (the
                 // row builder counts the others)
-                const int upto = (int)sRaw[(k - 1) % kRawSlots * (kRawFields * CH) + 9 * CH + CH - 1];
+                const int upto = (int)sRaw[(k - 1) % RAW * (kRawFields * CH) + 9 * CH + CH - 1];
                 if (gi == ng && lane == 0 && sDoneRing[seq % kDoneRing] < kEpiWarps)
                     atomicAdd(a.issued, 256ull * (unsigned long long)(len - upto));
             }
@@ -1013,8 +1026,8 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
         [[maybe_unused]] uint32_t issued = 0;
         [[maybe_unused]] int upto = 0;
         for (int kr = 0;; ++kr) {
-            const int s = k % SS, rs = kr % kRawSlots;
-            if (!mbar_wait_bounded(bar_rfull(rs), (uint32_t)(kr / kRawSlots) & 1u, tmo, sAbort) ||
+            const int s = k % SS, rs = kr % RAW;
+            if (!mbar_wait_bounded(bar_rfull(rs), (uint32_t)(kr / RAW) & 1u, tmo, sAbort) ||
                 !mbar_wait_bounded(bar_empty(s), ((uint32_t)(k / SS) & 1u) ^ 1u, tmo, sAbort)) {
                 *sAbort = 1;
                 atomicOr(a.err, kErrTimeout);
