@@ -229,13 +229,19 @@ __device__ __forceinline__ float box_max_quadratic(float A, float B, float C, fl
     return best;
 }
 
-// Relative error, per unit of the magnitude sum of Eq. 3's terms, that the
-// variant's exponent may have against the quadratic (an upper bound with room:
-// the split operands err by 2^-21 of that sum at most, one fp16 or bf16 term by
-// 2^-11 or 2^-8 of each coefficient, the e4m3 terms by 2^-10 of the largest).
+// Relative error, per unit of the magnitude sum S of Eq. 3's terms, that the
+// variant's exponent may have against the quadratic, with room.  The products of
+// Eq. 6 add up to log2(e) S in magnitude at most, so one fp16 or bf16 term (2^-11
+// or 2^-8 of each coefficient; log2 o's own share is inside box_reaches' margin)
+// errs by 0.00071 S or 0.0057 S, the split operands by 2^-21 S.  The five e4m3 terms
+// err by 2^-20 of a coefficient or 2^-21 of the largest, the monomials add up to 402
+// at most: 0.0003 S.  Twice these bounds for one term kept so many dead entries that
+// the bf16 backward of 500k splats on 64 x 64 pixels was slower than without
+// culling: 1768 -> 1869 us, with these 1789; 1920 x 1080, 1M, full lists, bf16
+// forward 389 -> 363 us, backward 727 -> 676.
 template <int V>
 constexpr float reach_rel() {
-    return V == GS_BLEND_TC_FP16 ? 1.0f / 512 : V == GS_BLEND_TC_BF16 ? 1.0f / 64
+    return V == GS_BLEND_TC_FP16 ? 1.0f / 1024 : V == GS_BLEND_TC_BF16 ? 1.0f / 128
            : V == GS_BLEND_TC_FP8_SPLIT ? 1.0f / 256 : 1.0f / 131072;
 }
 
@@ -262,13 +268,14 @@ __device__ __forceinline__ bool box_reaches(float A, float B, float C, float l2o
 // 1/255 at every pixel of the tile; such a splat changes no pixel (the skip
 // rule of Alg. 1) and its MMA columns and compositing can be left out.  The
 // margin (0.3 in base-2 units) is more than coeff_row's own test of far splats
-// allows; S is taken at offsets enlarged by 24 px (which covers either
-// reference pixel).  (xh, yh): splat centre minus the upper half's reference;
-// bx0..by1: the offsets of that half's pixels from it.
+// allows; S is taken at offsets enlarged by 16 px (a pixel is at most 15 from the
+// upper half's reference in either direction, counted over the lower half's).
+// (xh, yh): splat centre minus the upper half's reference; bx0..by1: the offsets of
+// that half's pixels from it.
 template <int V>
 __device__ __forceinline__ bool splat_reaches(float A, float B, float C, float l2o, float xh, float yh, float bx0,
                                               float bx1, float by0, float by1) {
-    const float ax = fabsf(xh) + 24.f, ay = fabsf(yh) + 24.f;
+    const float ax = fabsf(xh) + 16.f, ay = fabsf(yh) + 16.f;
     const float S = fmaf(0.5f * fabsf(A) * ax, ax, fmaf(fabsf(B) * ax, ay, 0.5f * fabsf(C) * ay * ay));
     return box_reaches(A, B, C, l2o, xh + bx0, xh + bx1, yh + by0 - 8.0f, yh + by1, S, reach_rel<V>());
 }
