@@ -630,15 +630,15 @@ gs_status gs_blend_autotune_backward(int32_t n_views, const int32_t* widths, con
         set_error("gs_blend_autotune_backward: needs a TC variant and reps >= 1");
         return GS_ERR_INVALID_ARG;
     }
-    static const int kStages[] = {2, 3, 4, 6};
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     gs_status st = cuda_status(cudaEventCreate(&e0), "gs_blend_autotune_backward: event");
     if (st == GS_OK) st = cuda_status(cudaEventCreate(&e1), "gs_blend_autotune_backward: event");
     float best = 1e30f;
-    int best_i = -1;
-    for (int i = 0; st == GS_OK && i < 3; ++i) {
+    int best_stages = 0;
+    for (const int stages : kBwdStagesBuilt) {
+        if (st != GS_OK) break;
         gs_blend_opts o = *opts;
-        o.bwd_stages = kStages[i];
+        o.bwd_stages = stages;
         auto run = [&]() {
             return gs_blend_backward_views(n_views, widths, heights, n_per_view, tile_ranges, ids_sorted, mean2d,
                                            conic, opacity, rgb, &o, T_final, n_contrib, dL_dimage, dmean2d, dconic,
@@ -656,13 +656,13 @@ gs_status gs_blend_autotune_backward(int32_t n_views, const int32_t* widths, con
         ms /= (float)reps;
         if (ms < best) {
             best = ms;
-            best_i = i;
+            best_stages = stages;
         }
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
     if (st != GS_OK) return st;
-    opts->bwd_stages = kStages[best_i];
+    opts->bwd_stages = best_stages;
     if (best_ms) *best_ms = best;
     return gs_sync_status(stream);
 }

@@ -20,7 +20,9 @@ cudaError_t launch_blend_tc_bwd(const BlendArgs& a0, const GradArgs& g, int vari
 }
 
 bool tc_bwd_stages_supported(int stages) {
-    return stages == 0 || stages == 2 || stages == 3 || stages == 4 || stages == 6;
+    for (const int built : kBwdStagesBuilt)
+        if (stages == built) return true;
+    return stages == 0;
 }
 
 }  // namespace gs

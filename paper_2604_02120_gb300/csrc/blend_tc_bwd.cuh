@@ -66,13 +66,9 @@ namespace gs {
 namespace tc {
 
 constexpr int kBwdChunk = 16;
-// Built depths of the ring of chunk splats; 4 is the deepest that keeps 3 blocks per
-// SM for the bf16 and FP8 rows (76.6 KB each).
-constexpr int kBwdStagesBuilt[4] = {2, 3, 4, 6};
-template <int V>
-constexpr int bwd_default_stages() {
-    return 4;
-}
+// Default depth of the ring of chunk splats: the deepest that keeps 3 blocks per SM
+// for the bf16 and FP8 rows (76.6 KB each).
+constexpr int kBwdStages = 4;
 constexpr float kTScale = 4096.0f;  // 2^12
 
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -776,14 +772,14 @@ cudaError_t launch_bwd_inst(const BlendArgs& a, const GradArgs& g, cudaStream_t 
     return cudaGetLastError();
 }
 
-// stages 0: the variant's default; otherwise one of kBwdStagesBuilt
-template <int V>
+// stages 0: the default; otherwise one of kBwdStagesBuilt
+template <int V, int I = 0>
 cudaError_t launch_bwd_stages(const BlendArgs& a, const GradArgs& g, int stages, cudaStream_t s) {
-    if (stages == 0) stages = bwd_default_stages<V>();
-    if (stages == 2) return launch_bwd_inst<V, 2>(a, g, s);
-    if (stages == 3) return launch_bwd_inst<V, 3>(a, g, s);
-    if (stages == 4) return launch_bwd_inst<V, 4>(a, g, s);
-    if (stages == 6) return launch_bwd_inst<V, 6>(a, g, s);
+    if constexpr (I < (int)(sizeof(kBwdStagesBuilt) / sizeof(int))) {
+        if ((stages == 0 ? kBwdStages : stages) == kBwdStagesBuilt[I])
+            return launch_bwd_inst<V, kBwdStagesBuilt[I]>(a, g, s);
+        return launch_bwd_stages<V, I + 1>(a, g, stages, s);
+    }
     return cudaErrorInvalidValue;
 }
 

@@ -197,6 +197,7 @@ bool tc_config_supported(int variant, int chunk, int stages);
 // Gradient of the tensor-core blend of `variant` (exponents recomputed with the
 // forward pass's tensor-core arithmetic).
 cudaError_t launch_blend_tc_bwd(const BlendArgs& a, const GradArgs& g, int variant, int stages, cudaStream_t s);
+constexpr int kBwdStagesBuilt[] = {2, 3, 4, 6};  // depths of the backward's ring of splat chunks
 bool tc_bwd_stages_supported(int stages);
 // A zeroed tile-queue counter for one persistent launch on stream s.
 unsigned* tile_queue_slot(cudaStream_t s, cudaError_t* err);
