@@ -128,11 +128,11 @@ typedef struct gs_blend_opts {
                                    are the sum of n_contrib.  The caller zeroes it */
     const float* splat_records; /* NULL, or a DEVICE table from gs_pack_splats over the call's items
                                    (the same mean2d, conic, opacity, rgb), 16-byte aligned: the
-                                   tensor-core kernels then stage each chunk's splat records into
-                                   shared memory with TMA gather copies (cp.async.bulk.tensor
-                                   tile::gather4) issued chunks ahead, instead of loading the splat
+                                   tensor-core forward then stages its splats in shared memory by TMA
+                                   gather copies of the records (cp.async.bulk.tensor tile::gather4),
+                                   a group of 32 entries ahead, instead of copying from the splat
                                    arrays thread by thread.  Same results bit for bit; ignored by the
-                                   FP32 variant */
+                                   FP32 variant and by the backward */
     int64_t splat_record_count; /* rows of splat_records (n_items of gs_pack_splats), 1 .. 2^31 - 1;
                                    a row beyond it reads as zeros, never outside the table */
 } gs_blend_opts;

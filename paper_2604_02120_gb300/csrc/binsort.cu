@@ -46,11 +46,6 @@ namespace gs {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr uint32_t kSmallPass = 1u << 20;
-// Items per thread of a radix pass: tiles of 1024 up to 2^18 items, so that a
-// small pass reaches all SMs; of 2048 up to 9 x 2^17, one wave of 4 blocks per
-// SM (a pass of 1M: 13.5 us, in tiles of 1024 17.4); of 4096 beyond, which
-// halves the look-back.
 constexpr int kDupTile = kThreads;          // items per tile of the opacity-aware duplication
 constexpr int kMaxPasses = 8;               // 4 depth passes + up to 4 tile-id passes
 #ifndef GS_LOOKBACK_LIMIT_NS
@@ -70,10 +65,17 @@ struct GiveUp {
 
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
+// Items per thread of a radix pass: tiles of 1024 up to 2^18 items, so that a
+// small pass reaches all SMs; of 2048 up to 9 x 2^17 items, 576 tiles, the most that
+// 4 blocks on each of 152 SMs take in one wave (a pass of 1M: 13.5 us, in tiles of
+// 1024 17.4); of 4096 beyond, which halves the look-back.  (A literal: the workspace
+// size is asked for without a device.)
 inline int pass_items(uint64_t n) { return n <= 1u << 18 ? 4 : n <= 9u << 17 ? 8 : 16; }
-// An upper bound of the radix tiles of a pass over at most m items.
+// An upper bound of the radix tiles of a pass over at most m items; it grows with m
+// (a pass of fewer items can have more tiles than one just past a step of
+// pass_items: the first 2^20 items are counted in the smallest tiles).
 inline int64_t radix_tiles_max(int64_t m) {
-    return std::max(cdiv(std::min<int64_t>(m, kSmallPass), kThreads * 4), cdiv(m, kThreads * pass_items(m)));
+    return std::max(cdiv(std::min<int64_t>(m, 1 << 20), kThreads * 4), cdiv(m, kThreads * pass_items(m)));
 }
 
 // ---------------------------------------------------------- block helpers --
@@ -1114,7 +1116,7 @@ __device__ __forceinline__ uint32_t supertile_mask(const SortViews& sv, const fl
 // bits with four lane reductions (bit j of every mask spread to its own byte)
 // into lane j's count, adding it to ranges with one atomic per tile when the
 // supertile changes.  32 pairs of several supertiles: one atomic per group
-// of equal supertiles and tile.  With st_count (zeroed by k_dup_coarse), each
+// of equal supertiles and tile.  With st_count (zeroed by the duplication), each
 // supertile's total is added there as well, and the ends of its pairs go to
 // st_beg / st_end (supertiles without pairs are left alone).  Segments are 128 to 512 pairs
 // (the least that gives every warp at most one), loaded 128 pairs at a time
@@ -1400,7 +1402,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_fine(const __grid_constant__ Sor
 // (st_order, total_st entries), so that the fine writes start the longest
 // supertiles first (the order within a bucket is arbitrary; the output does
 // not depend on it).  Graph mode: the instance count (fine_total, from
-// k_dup_coarse) to *count_out, and the capacity bit when it exceeds the
+// the duplication) to *count_out, and the capacity bit when it exceeds the
 // capacity.
 constexpr int kScanThreads = 1024;
 constexpr int kStBuckets = 33;  // 0: empty, b: counts in [2^(b-1), 2^b)

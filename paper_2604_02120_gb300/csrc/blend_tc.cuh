@@ -66,8 +66,7 @@ namespace gs {
 namespace tc {
 
 constexpr int kEpiWarps = 4;
-constexpr int kThreads = 192;     // 4 epilogue warps, scanner, row builder
-constexpr int kFwdThreads = 192;  // forward: epilogue warps, scanner, row builder
+constexpr int kThreads = 192;  // 4 epilogue warps, scanner, row builder
 constexpr int kTStages = 2;
 constexpr int kDoneRing = 16;  // tiles in flight between scanner and epilogue < kDoneRing
 constexpr float kAlphaMin = 1.0f / 255.0f;
@@ -555,7 +554,7 @@ __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y
 // COUNT: adds to *a.issued (a kernel of its own: counting in the row builder cost the
 // calls that do not ask for it 1 to 2%)
 template <int V, int CH, int SS, bool DUMP, bool COUNT>
-__global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
+__global__ void __launch_bounds__(kThreads, 4) k_blend_tc(const __grid_constant__ BlendArgs a) {
     using TR = Traits<V>;
     using LY = Layout<SS, CH, V>;
     constexpr int SBO = TR::SBO, RAW = LY::RAW;
@@ -608,7 +607,7 @@ __global__ void __launch_bounds__(kFwdThreads, 4) k_blend_tc(const __grid_consta
         mbar_fence_init();
     }
     // pixel matrix M_p of a 16 x 8 half-tile (A operand)
-    for (int row = threadIdx.x; row < 128; row += kFwdThreads) {
+    for (int row = threadIdx.x; row < 128; row += kThreads) {
         const float xb = (origin ? 0.f : 7.5f) - (float)lane_col(row);
         const float yb = (origin ? 0.f : 3.5f) - (float)lane_row(row);
         store_mp_row<V>(sA, row, xb, yb);
@@ -1181,9 +1180,9 @@ cudaError_t launch_inst(const BlendArgs& a, int items, cudaStream_t s) {
         if ((e = cudaFuncGetAttributes(&fa, kern)) != cudaSuccess) return e;
         // registers are granted per warp in units of 256
         const int regs_warp = ((fa.numRegs * 32 + 255) / 256) * 256;
-        const int by_regs = 65536 / (regs_warp * (kFwdThreads / 32));
+        const int by_regs = 65536 / (regs_warp * (kThreads / 32));
         const int by_smem = smem_sm / (bytes + (int)fa.sharedSizeBytes + 1024);
-        const int by_threads = 2048 / kFwdThreads;
+        const int by_threads = 2048 / kThreads;
         const int by_tmem = (int)(512 / LY::TCOLS);
         r.per_sm = by_regs;
         if (by_smem < r.per_sm) r.per_sm = by_smem;
@@ -1194,7 +1193,7 @@ cudaError_t launch_inst(const BlendArgs& a, int items, cudaStream_t s) {
     });
     if (es != cudaSuccess) return es;
     const int grid = items < sh.per_sm * sh.sms ? (items > 0 ? items : 1) : sh.per_sm * sh.sms;
-    kern<<<grid, kFwdThreads, bytes, s>>>(a);
+    kern<<<grid, kThreads, bytes, s>>>(a);
     count_launches();
     return cudaGetLastError();
 }

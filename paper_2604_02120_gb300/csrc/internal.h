@@ -77,8 +77,8 @@ struct BlendArgs {
     float* dump;
     // Packed splat records (kRecFloats floats per item, gs_pack_splats) and
     // the TMA descriptor of that table (2D: kRecFloats x items, box 16 x 1):
-    // when use_rec is set the tensor-core kernels stage each chunk's records
-    // into shared memory with tile::gather4 copies instead of loading the
+    // when use_rec is set the tensor-core forward stages its groups' records in
+    // shared memory with tile::gather4 copies instead of copying from the
     // splat arrays thread by thread.
     int use_rec;
     alignas(64) CUtensorMap rec_map;

@@ -47,12 +47,6 @@ __device__ __forceinline__ ViewIn load_view(size_t item, const int* radius_all, 
     return in;
 }
 
-// 4 bytes from global to shared memory without a register in between.
-__device__ __forceinline__ void copy_word_async(float* dst, const float* src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
-                 : "memory");
-}
-
 // Floats per Gaussian row of the shared coefficient arrays (odd).
 template <int SH_DEGREE>
 __host__ __device__ constexpr int sh_row() { return (3 * (SH_DEGREE + 1) * (SH_DEGREE + 1)) | 1; }
@@ -86,7 +80,7 @@ __global__ void __launch_bounds__(kProjBwdThreads, ONE ? 5 : 4) k_project_bwd(in
 #pragma unroll 12
     for (int j = 0; j < KC; ++j) {
         const int i = threadIdx.x + j * kProjBwdThreads, r = i / KC, q = i - r * KC;
-        if (i < nb * KC) copy_word_async(s_cf + r * ROW + q, src + i);
+        if (i < nb * KC) cp_async4(s_cf + r * ROW + q, src + i);
     }
     if constexpr (!ONE)
         for (int i = threadIdx.x; i < kProjBwdThreads * ROW; i += kProjBwdThreads) s_dcf[i] = 0.f;
