@@ -13,16 +13,19 @@ namespace {
 // L2; outputs of view v, Gaussian g at index v * n + g.  How many blocks a chunk
 // has is a matter of what moves.  Degrees 0 and 1 write nearly as much as they
 // read, and every view's outputs are streams of their own: whole waves per view
-// (1024 blocks, 131072 Gaussians).  Degrees 2 and 3 are bound by the coefficients,
-// which 16 blocks keep closest.  Degree 0, 16 views of 300k / 1.5M: view by view
-// over all Gaussians 74 / 567 us, views innermost (chunks of one block) 107 / 514,
-// in chunks of 1024 74 / 340; degree 3, 16 views of 1.5M: 1124, 747, 787, in
-// chunks of 16 748 (5 views of 3M 710, 514, 524, 500).
+// (1024 blocks, 131072 Gaussians).  Degree 3 is bound by the coefficients, which 16
+// blocks keep closest; degree 2 lies between (16 views of 200k 98 us in chunks of 16,
+// 94 in chunks of 1024; two views of 3M 204 and 209).  Degree 0, 16 views of 300k /
+// 1.5M: view by view over all Gaussians 74 / 567 us, views innermost (chunks of one
+// block) 107 / 514, in chunks of 1024 74 / 340; degree 3, 16 views of 1.5M: 1124, 747,
+// 787, in chunks of 16 748 (5 views of 3M 710, 514, 524, 500).
 // Bound by the latency of a chain of loads (means, then shape, then the
 // coefficients of what is visible), so by resident warps: 64 registers and small
 // blocks.  3M Gaussians, degree 3, one view 146 -> 127 us (663 MB, 5.2 TB/s).
 constexpr int kProjThreads = 128;
-constexpr unsigned chunk_blocks(int sh_degree) { return sh_degree <= 1 ? 1024 : 16; }
+constexpr unsigned chunk_blocks(int sh_degree, int views) {
+    return sh_degree <= 1 || (sh_degree == 2 && views > 2) ? 1024 : 16;
+}
 template <int SH_DEGREE, bool VEC16>
 __global__ void __launch_bounds__(kProjThreads, 8) k_project(int n, const float* __restrict__ means,
                                                  const float* __restrict__ scales, const float* __restrict__ quats,
@@ -45,7 +48,7 @@ cudaError_t launch_project(int n, const float* means, const float* scales, const
     const int block = kProjThreads;
     const unsigned nblk = ((unsigned)n + block - 1) / block;
     // (at most 65535 chunks; blocks split evenly, the last chunk may be a few short)
-    const unsigned chunk = std::max(chunk_blocks(sh_degree), (nblk + 65534) / 65535);
+    const unsigned chunk = std::max(chunk_blocks(sh_degree, cams.num_views), (nblk + 65534) / 65535);
     const unsigned chunks = (nblk + chunk - 1) / chunk;
     const dim3 grid((nblk + chunks - 1) / chunks, cams.num_views, chunks);
     // 16-byte coefficient loads for degrees 1 and 3 (3K a multiple of 4) on an aligned array
