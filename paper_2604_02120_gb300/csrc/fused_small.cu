@@ -176,9 +176,15 @@ __global__ void __launch_bounds__(fused_threads(BLEND)) k_project_bin_small(cons
 
     // 3. every splat appends its index to the tiles it covers (the other
     // blocks' outputs are read through L2: this SM's L1 may hold lines from
-    // before the barrier).  Up to half as many splats as threads: eight lanes share a
-    // splat's rows, as a chain of atomics per thread is what this step waits for.
-    const int share = n <= (int)(gridDim.x * kFusedThreads / 2) ? 8 : 1;
+    // before the barrier).  A chain of atomics per thread is what this step waits for, so
+    // lanes share a splat's rows: with the blend eight of them up to half as many splats
+    // as threads, else one; without it, in more and smaller blocks, up to eight, as many
+    // as leave a thread two splats (60k at 400 x 300 with eight lanes 60.2 us, two 57.9;
+    // 30k at 640 x 480 with one 45.6, four 43.9).
+    const int threads = (int)(gridDim.x * kFusedThreads);
+    int share = BLEND && n > threads / 2 ? 1 : 8;
+    if constexpr (!BLEND)
+        while (share > 1 && (long long)n * share > 2ll * threads) share >>= 1;
     for (long long q = blockIdx.x * kFusedThreads + threadIdx.x; ok && q < (long long)n * share;
          q += gridDim.x * kFusedThreads) {
         const int g = (int)(q / share), sub = (int)(q % share);
