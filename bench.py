@@ -633,7 +633,7 @@ def run_ours(args):
                     "frac": round(ach / hbm, 4) if hbm else None, "traffic": None, "launch_ms": round(dup_ms, 5),
                     "algorithmic_bytes": dup_bytes, "pairs": n_pairs,
                     "peak_source": "MEASURED_PEAKS.json hbm_gbs (copy, burst) of measured",
-                    "note": "bound by instruction issue and latency, not by HBM (ncu: issue 55% busy, 4 blocks "
+                    "note": "bound by instruction issue and latency, not by HBM (ncu: issue 61% busy, 4 blocks "
                             "per SM); algorithmic bytes: 32 per Gaussian read, 8 per supertile pair written"}
     else:
         r = rf if dom == "blend_forward" else rb

@@ -654,7 +654,7 @@ __device__ __forceinline__ Runs4 unpack_runs(uint4 v) {
 // of the pair sort's tiles that start within its pairs (below `limit`), and
 // the blocks together zero st_zero[0, st_n).
 //
-// Bound by issue slots (55%) and by waits of every kind in a tile's chain of
+// Bound by issue slots (61%) and by waits of every kind in a tile's chain of
 // about 34000 cycles: 20% the gathers of the items, 20% evaluating, 17% making
 // pairs, 17% the look-back.  Nothing may wait between a tile's ticket and its
 // sum: drawing the next ticket before the look-back's end (to load its items

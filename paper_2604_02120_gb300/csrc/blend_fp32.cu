@@ -65,10 +65,12 @@ __device__ __forceinline__ bool warp_reaches(const float4& geo, const float4& oc
 // what the tests would spare there does not pay for them.  Opacity-aware lists of
 // large splats (3840 x 2160, 3M, heavy tails: 95% needed, a warp walks 54), forward /
 // backward: without any test 636 / 2263 us, with this rule 627 / 2315, with every
-// group tested 793 / 2482.  (The forward holds nothing of the test's over the walk
-// and takes two splats per turn; with both staged and held it took 662.  What the
-// backward loses is the second loop's place in the code: a kernel of the plain loop
-// alone takes 2245, tests by a cheaper bound or one loop for both were slower.)
+// group tested 793 / 2482.  The forward holds nothing of the test's over the walk and
+// takes two splats per turn; with both staged and held it took 662.  Where walks are
+// shorter still (24 splats a pixel, L2 flushed) the one test of a batch shows: 344 /
+// 1271 us without, 361 / 1285 with.  A cheaper test before it (the middle of the
+// warp's pixels, or of the tile's by one warp), one loop for both walks and other
+// unrolling were all slower.
 __device__ __forceinline__ bool dense_group(unsigned hits, int n) { return 5 * __popc(hits) >= 4 * n; }
 
 // Geometry of the block's tile (blockIdx.x is a global tile id).

@@ -33,7 +33,7 @@
 // Why the lists are culled here: with full 3-sigma rectangles 50 to 72% of a
 // tile's entries reach none of its pixels, and an entry dropped costs the
 // scanner about 2 instructions per epilogue warp, one kept 29 (the kernel runs
-// at 60 to 67% of the issue slots).  1920 x 1080, 1M clustered splats, full
+// at 62 to 71% of the issue slots).  1920 x 1080, 1M clustered splats, full
 // rectangles: 0.828 -> 0.339 ms; 1280 x 720, 200k: 0.119 -> 0.079 ms; 256 x 256,
 // 10k: 0.036 -> 0.028 ms; opacity-aware lists, where every entry is kept:
 // 0.286 -> 0.273 ms (1920 x 1080), 0.482 -> 0.470 ms (3840 x 2160, 3M).

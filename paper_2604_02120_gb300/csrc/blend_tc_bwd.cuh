@@ -48,7 +48,7 @@
 // out in 9 atomics per splat and tile (15 with one set per half).
 // All waits are bounded by opts.timeout_ns as in the forward kernel.
 //
-// What bounds it: issue slots (58 to 61% of them, about 70 instructions per
+// What bounds it: issue slots (56 to 62% of them, about 70 instructions per
 // splat and warp) and the instruction cache: with all 16 splats of a chunk
 // unrolled and the finishing step written out twice, a third of the stalls at
 // 3840 x 2160 were warps without an instruction.  So the splats go through a
