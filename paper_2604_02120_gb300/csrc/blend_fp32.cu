@@ -24,6 +24,12 @@ constexpr float kAlphaMin = 1.0f / 255.0f;
 constexpr float kAlphaMax = 0.99f;
 constexpr float kTMin = 1e-4f;
 
+// The forward's first batch: many tiles stop within it, and what was staged past the
+// stop was gathered for nothing (3840 x 2160, 3M, opacity-aware: lists of 3500, a warp
+// walks 54; batches of 256 throughout 627 us, 128 first 598; 24 splats a pixel, L2
+// flushed, 361 and 326; 96 first is 1% better there; deep walks lose up to 1%).
+constexpr int kFirst = 128;
+
 struct SplatSm {
     float4 geo;  // mx, my, A, B
     float4 oc;   // C, o, r, g
@@ -63,7 +69,7 @@ __device__ __forceinline__ bool warp_reaches(const float4& geo, const float4& oc
 // A batch whose first 32 splats include four in five that the warp needs is walked
 // whole, by the plain loop: it costs less per splat than one over set bits, and
 // what the tests would spare there does not pay for them.  Opacity-aware lists of
-// large splats (3840 x 2160, 3M, heavy tails: 95% needed, a warp walks 54), forward /
+// large splats (3840 x 2160, 3M, heavy tails: 95% needed), batches of 256, forward /
 // backward: without any test 636 / 2263 us, with this rule 627 / 2315, with every
 // group tested 793 / 2482.  The forward holds nothing of the test's over the walk and
 // takes two splats per turn; with both staged and held it took 662.  Where walks are
@@ -114,10 +120,10 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
     float T = 1.0f, cr = 0.f, cg = 0.f, cb = 0.f;
     int last = 0;
     bool done = !inside;
-    for (int base = 0; base < len; base += kBatch) {
+    for (int base = 0; base < len; base += base ? kBatch : kFirst) {
         if (__syncthreads_count(done) == kBatch) break;
         const int i = base + threadIdx.x;
-        if (i < len) {
+        if (i < len && (base || threadIdx.x < kFirst)) {
             SplatSm s;
             load_splat(a, a.ids[start + i], tg.opac_off, s);
             s_geo[threadIdx.x] = s.geo;
@@ -125,7 +131,7 @@ __global__ void __launch_bounds__(kBatch) k_blend_fp32_fwd(const __grid_constant
             s_b[threadIdx.x] = s.b;
         }
         __syncthreads();
-        const int nb = min(kBatch, len - base);
+        const int nb = min(base ? kBatch : kFirst, len - base);
         auto step = [&](int j) {
             const float4 geo = s_geo[j], oc = s_oc[j];
             float e, pw, dx, dy;

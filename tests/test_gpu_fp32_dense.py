@@ -1,6 +1,6 @@
 """The FP32 blends walk a batch whole where nearly all of its first splats reach a
 warp's pixels: lists of wide splats, at lengths around the pairs, groups of 32 and
-batches of 256 of that walk, alone and followed by a batch out of reach; against a
+batches (128, then 256) of that walk, alone and followed by a batch out of reach; against a
 64-bit walk, with pixels that stop inside a batch."""
 import numpy as np
 import pytest
@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("opacity", [0.006, 0.4])  # every pixel runs to the end; pixels stop after about 18
 @pytest.mark.parametrize("tail", [0, 300])
-@pytest.mark.parametrize("n", [1, 2, 31, 33, 255, 256, 257, 600])
+@pytest.mark.parametrize("n", [1, 2, 31, 33, 127, 128, 129, 255, 257, 383, 384, 385, 600, 641])
 def test_dense_batches(n, tail, opacity):
     cam = scenes.look_at_camera((0, 0, -3), (0, 0, 0), 53, 37)
     rng = np.random.default_rng(n)
