@@ -10,9 +10,9 @@
 // instruction per pair) and only the splats that can contribute are walked, in
 // list order and with their list positions: the same decisions and the same
 // values as the walk over all.  Forward and backward against the walk over all:
-// full rectangles, 641 x 479, 50k splats 105 -> 60 us and 217 -> 152 us; 1920 x
-// 1080, 1M clustered 1072 -> 445 us and 2315 -> 1321 us; opacity-aware lists there
-// 418 -> 350 us and 1304 -> 1166 us; 1280 x 720, 200k 110 -> 93 us and 305 -> 281 us.
+// full rectangles, 641 x 479, 50k splats 112 -> 63 us and 233 -> 164 us; 1920 x
+// 1080, 1M clustered 1072 -> 446 us and 2315 -> 1321 us; opacity-aware lists there
+// 418 -> 355 us and 1304 -> 1166 us; 1280 x 720, 200k 110 -> 94 us and 305 -> 281 us.
 #include "blend_tc.cuh"
 #include "internal.h"
 
