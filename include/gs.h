@@ -306,6 +306,8 @@ gs_status gs_bin_sort(int32_t n, const float* mean2d, const int32_t* radius, con
  *    `capacity`; the instance count is written to *n_instances_dev; if it
  *    exceeds capacity the lists are truncated and gs_sync_status() later
  *    returns GS_ERR_CAPACITY.
+ * A device-side wait that gives up (GS_ERR_TIMEOUT from gs_sync_status) leaves
+ * every list of the call empty.
  * Opacity-aware lists (the tighter tile intersection; not in the paper): with
  * conic (the items' conics, 3 floats each, as gs_project writes them) and
  * power_min (one float per Gaussian, from gs_alpha_power_min) a splat keeps a
